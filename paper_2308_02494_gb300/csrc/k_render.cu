@@ -1,84 +1,23 @@
 // Headless neural volume renderer (Sec. 6) over a domain decomposition (Sec. 5.3).
 //
-// Per batch of rays: (1) every (ray, sample) computes its position, its brick
-// through the spatial hash and its brick-local coordinate, and takes a rank in
-// its brick's bucket; (2) bucket offsets; (3) samples are scattered into brick
-// order; (4) the fused forward query runs over the buckets (device-side offsets);
-// (5) each ray gathers its values back in sample order and composites front to
-// back.  Sampling and opacity: midpoints t_j = t0 + (j + 1/2) dt of the ray's
+// Per batch of rays, BF16: the forward query forms its samples itself, bundle by bundle
+// (render.h), and leaves their values in slot order.  Float32: (1) every (ray, sample)
+// computes its position, its brick through the spatial hash and its brick-local
+// coordinate, and takes a rank in its brick's bucket; (2) bucket offsets; (3) samples are
+// scattered into brick order; (4) the fused forward query runs over the buckets
+// (device-side offsets).  Then each ray reads its values in sample order and is
+// composited front to back.  Sampling and opacity: midpoints t_j = t0 + (j + 1/2) dt of the ray's
 // segment inside [-1,1]^3, alpha = 1 - exp(-a dt / (2/512)), the 256-entry RGBA
 // transfer function read with linear interpolation.
+#include <algorithm>
+#include <climits>
+
 #include "common.cuh"
 #include "kernels.h"
 #include "render.h"
 
 namespace srn {
 namespace {
-
-struct Ray {
-  float ox, oy, oz, dx, dy, dz, t0, dt;
-  bool hit;
-};
-
-__device__ __forceinline__ Ray make_ray(const RenderParams& rp, int pix) {
-  const int px = pix % rp.width, py = pix / rp.width;
-  const float aspect = (float)rp.width / (float)rp.height;
-  const float nx = (2.f * ((float)px + 0.5f) / (float)rp.width - 1.f) * rp.cam.scale * aspect;
-  const float ny = (1.f - 2.f * ((float)py + 0.5f) / (float)rp.height) * rp.cam.scale;
-  Ray r;
-  const float* e = rp.cam.eye;
-  const float* f = rp.cam.forward;
-  const float* ri = rp.cam.right;
-  const float* u = rp.cam.up;
-  if (rp.cam.ortho) {
-    r.ox = e[0] + nx * ri[0] + ny * u[0];
-    r.oy = e[1] + nx * ri[1] + ny * u[1];
-    r.oz = e[2] + nx * ri[2] + ny * u[2];
-    r.dx = f[0]; r.dy = f[1]; r.dz = f[2];
-  } else {
-    r.ox = e[0]; r.oy = e[1]; r.oz = e[2];
-    float dx = f[0] + nx * ri[0] + ny * u[0];
-    float dy = f[1] + nx * ri[1] + ny * u[1];
-    float dz = f[2] + nx * ri[2] + ny * u[2];
-    const float inv = rsqrtf(dx * dx + dy * dy + dz * dz);
-    r.dx = dx * inv; r.dy = dy * inv; r.dz = dz * inv;
-  }
-  // slab test against [-1, 1]^3
-  float tmin = -INFINITY, tmax = INFINITY;
-  const float o[3] = {r.ox, r.oy, r.oz}, d[3] = {r.dx, r.dy, r.dz};
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const float inv = 1.f / d[a];
-    const float ta = (-1.f - o[a]) * inv, tb = (1.f - o[a]) * inv;
-    tmin = fmaxf(tmin, fminf(ta, tb));
-    tmax = fminf(tmax, fmaxf(ta, tb));
-  }
-  tmin = fmaxf(tmin, 0.f);
-  r.hit = tmax > tmin;
-  r.t0 = tmin;
-  r.dt = r.hit ? (tmax - tmin) / (float)rp.samples : 0.f;
-  return r;
-}
-
-// Pixels of level l of the image hierarchy: its grid (a 2^l, b 2^l), ceil(W / 2^l) by
-// ceil(H / 2^l).  Together, the levels coarser than l hold exactly level l+1's grid.
-__device__ __forceinline__ int level_cols(const RenderParams& rp, int l) { return (rp.width + (1 << l) - 1) >> l; }
-__device__ __forceinline__ int level_pixels(const RenderParams& rp, int l) {
-  return level_cols(rp, l) * ((rp.height + (1 << l) - 1) >> l);
-}
-
-// Flat pixel of the k-th pixel of the render order.  Progressive order (Sec. 6): the
-// coarsest level's pixel (0, 0), then each finer level l's pixels not on level l+1's
-// grid, row by row: an even row b of the level has its odd columns, an odd row all.
-__device__ __forceinline__ int pixel_of(const RenderParams& rp, int k) {
-  if (!rp.order || k == 0) return k;
-  int l = rp.levels - 1;
-  while (level_pixels(rp, l) <= k) --l;   // level_pixels(0) = W H > k
-  const int q = k - level_pixels(rp, l + 1);
-  const int wa = level_cols(rp, l), half = wa >> 1, pair = q / (half + wa), r = q - pair * (half + wa);
-  const int a = r < half ? 2 * r + 1 : r - half, b = r < half ? 2 * pair : 2 * pair + 1;
-  return (b << l) * rp.width + (a << l);
-}
 
 // Position of pixel (x, y) in the progressive order (the inverse of pixel_of).
 __device__ __forceinline__ int order_of(const RenderParams& rp, int x, int y) {
@@ -96,39 +35,18 @@ __global__ void __launch_bounds__(256) k_render_gen(RenderParams rp, int pix0, i
                                                     uint32_t* __restrict__ cnt) {
   __shared__ uint32_t s_cnt[SRN_MAX_BRICKS], s_base[SRN_MAX_BRICKS];
   const int nb = rp.grid[0] * rp.grid[1] * rp.grid[2];
-  const int64_t total = render_slots(rp.rg, rp.jb, rp.samples, npix);
-  const int nsb = (rp.samples + rp.jb - 1) / rp.jb;
+  const int total = (int)render_slots(rp, npix);
   const int lane = threadIdx.x & 31;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < total; base += (int64_t)gridDim.x * blockDim.x) {
     for (int k = threadIdx.x; k < nb; k += blockDim.x) s_cnt[k] = 0;
     __syncthreads();
     const int64_t idx = base + threadIdx.x;
     uint32_t b = 0xffffffffu;
-    // the slot's ray and sample (the inverse of render_slot)
-    const int js = (int)(idx % rp.jb);
-    const int64_t q1 = idx / rp.jb;
-    const int rl = (int)(q1 % rp.rg);
-    const int64_t q2 = q1 / rp.rg;
-    const int ray = (int)(q2 / nsb) * rp.rg + rl, j = (int)(q2 % nsb) * rp.jb + js;
-    if (idx < total && ray < npix && j < rp.samples) {
-      const Ray r = make_ray(rp, pixel_of(rp, pix0 + ray));
-      if (r.hit) {
-        const float t = r.t0 + ((float)j + 0.5f) * r.dt;
-        const float p[3] = {r.ox + t * r.dx, r.oy + t * r.dy, r.oz + t * r.dz};
-        int cell[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {   // Sec. 5.3 hash, clamped to the brick grid
-          const int n = rp.grid[a];
-          cell[a] = min(max((int)floorf((float)n * (p[a] + 1.f) * 0.5f), 0), n - 1);
-        }
-        b = (uint32_t)(cell[0] + rp.grid[0] * (cell[1] + rp.grid[1] * cell[2]));
-        const float half = 0.5f * (float)(rp.vox - 1);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {   // global -> brick-local [-1, 1]
-          const float sc = (p[a] + 1.f) * half;
-          const float lo = (float)rp.lo[b][a], hi = (float)rp.hi[b][a];
-          loc[3 * idx + a] = (sc - lo) / (hi - lo) * 2.f - 1.f;
-        }
+    if (idx < total) {
+      const RaySlot rs = ray_slot(rp, (int)idx);
+      if (rs.ray < npix && rs.j < rp.samples) {
+        const Ray r = make_ray(rp, pixel_of(rp, pix0 + rs.ray));
+        if (r.hit) b = (uint32_t)ray_sample(rp, r, rs.j, loc[3 * idx], loc[3 * idx + 1], loc[3 * idx + 2]);
       }
     }
     const unsigned grp = __match_any_sync(0xffffffffu, b);
@@ -196,34 +114,56 @@ __global__ void k_decode_store(DecodeChunk c, const float* __restrict__ val, flo
   }
 }
 
-// One thread per ray: gather the ray's values in sample order and composite.
-__global__ void k_render_composite(RenderParams rp, int pix0, int npix, const uint32_t* __restrict__ pos,
-                                   const float* __restrict__ val, const float* __restrict__ lut,
-                                   float* __restrict__ rgba) {
-  const int ray = blockIdx.x * blockDim.x + threadIdx.x;
-  if (ray >= npix) return;
-  const int pix = pixel_of(rp, pix0 + ray);
-  const Ray r = make_ray(rp, pix);
+// Front-to-back compositing of 32 rays per block of 256 threads: thread (ray, segment)
+// composites one eighth of the ray's samples, then the segments are joined in order (the
+// compositing operator is associative).  One thread per ray left a batch of 8192 rays
+// with 54 threads per SM, each a chain of 512 dependent reads.
+constexpr int kSegs = 8;
+template <bool POS>
+__global__ void __launch_bounds__(32 * kSegs)
+k_render_composite(RenderParams rp, int pix0, int npix, const uint32_t* __restrict__ pos,
+                   const float* __restrict__ val, const float* __restrict__ lut, float* __restrict__ rgba) {
+  __shared__ float4 part[kSegs][32];
+  const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
+  const int ray = blockIdx.x * 32 + lane;
+  const int pix = ray < npix ? pixel_of(rp, pix0 + ray) : 0;
   float cr = 0.f, cg = 0.f, cb = 0.f, T = 1.f;
-  if (r.hit) {
-    const float k = r.dt / (2.f / 512.f);
-    const float inv_span = 1.f / (rp.vmax - rp.vmin);
-    for (int j = 0; j < rp.samples; ++j) {
-      const float f = val[pos[render_slot(rp.rg, rp.jb, rp.samples, ray, j)]];
-      const float s = fminf(fmaxf((f - rp.vmin) * inv_span, 0.f), 1.f) * 255.f;
-      const int i0 = min((int)s, 254);
-      const float fr = s - (float)i0;
-      const float4 a = reinterpret_cast<const float4*>(lut)[i0];
-      const float4 c = reinterpret_cast<const float4*>(lut)[i0 + 1];
-      const float red = a.x + (c.x - a.x) * fr, grn = a.y + (c.y - a.y) * fr, blu = a.z + (c.z - a.z) * fr;
-      const float op = a.w + (c.w - a.w) * fr;
-      const float alpha = 1.f - expf(-op * k);
-      const float w = T * alpha;
-      cr = fmaf(w, red, cr); cg = fmaf(w, grn, cg); cb = fmaf(w, blu, cb);
-      T *= 1.f - alpha;
+  if (ray < npix) {
+    const Ray r = make_ray(rp, pix);
+    if (r.hit) {
+      const float k = r.dt / (2.f / 512.f);
+      const float inv_span = 1.f / (rp.vmax - rp.vmin);
+      const int j0 = (int)((int64_t)rp.samples * seg / kSegs), j1 = (int)((int64_t)rp.samples * (seg + 1) / kSegs);
+      const int s0 = render_slot(rp, ray, 0);
+#pragma unroll 8
+      for (int j = j0; j < j1; ++j) {
+        const int slot = s0 + j * rp.rg;
+        const float f = val[POS ? pos[slot] : (uint32_t)slot];
+        const float s = fminf(fmaxf((f - rp.vmin) * inv_span, 0.f), 1.f) * 255.f;
+        const int i0 = min((int)s, 254);
+        const float fr = s - (float)i0;
+        const float4 a = reinterpret_cast<const float4*>(lut)[i0];
+        const float4 c = reinterpret_cast<const float4*>(lut)[i0 + 1];
+        const float red = a.x + (c.x - a.x) * fr, grn = a.y + (c.y - a.y) * fr, blu = a.z + (c.z - a.z) * fr;
+        const float op = a.w + (c.w - a.w) * fr;
+        const float alpha = 1.f - expf(-op * k);
+        const float w = T * alpha;
+        cr = fmaf(w, red, cr); cg = fmaf(w, grn, cg); cb = fmaf(w, blu, cb);
+        T *= 1.f - alpha;
+      }
     }
   }
-  reinterpret_cast<float4*>(rgba)[pix] = make_float4(cr, cg, cb, 1.f - T);
+  part[seg][lane] = make_float4(cr, cg, cb, T);
+  __syncthreads();
+  if (seg == 0 && ray < npix) {
+#pragma unroll
+    for (int q = 1; q < kSegs; ++q) {
+      const float4 p = part[q][lane];
+      cr = fmaf(T, p.x, cr); cg = fmaf(T, p.y, cg); cb = fmaf(T, p.z, cb);
+      T *= p.w;
+    }
+    reinterpret_cast<float4*>(rgba)[pix] = make_float4(cr, cg, cb, 1.f - T);
+  }
 }
 
 // In-progress image of progressive rendering: evaluated pixels as they are, the others
@@ -267,25 +207,35 @@ int blocks_for(int64_t n, int threads, int num_sms) {
 
 cudaError_t launch_render_batch(const Launch& L, const RenderParams& rp, const RenderWs& w, int pix0,
                                 int npix, const Model& md, const float* lut, float* rgba) {
-  const int64_t total = render_slots(rp.rg, rp.jb, rp.samples, npix);
+  const int64_t total = render_slots(rp, npix);
   const int nb = rp.grid[0] * rp.grid[1] * rp.grid[2];
-  cudaError_t e = cudaMemsetAsync(w.cnt, 0, sizeof(uint32_t) * nb, L.stream);
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
+  Bricks br{};
+  br.n = nb;
+  if (md.F16) {
+    FwdSource src{};
+    src.kind = kFwdRender;
+    src.group = kFwdGroup;
+    src.groups = (int)((total + kFwdGroup - 1) / kFwdGroup);
+    src.pix0 = pix0;
+    src.npix = npix;
+    src.rp = rp;
+    if ((e = launch_forward_bf16(L, md, br, src, w.val)) != cudaSuccess) return e;
+    k_render_composite<false><<<(npix + 31) / 32, 32 * kSegs, 0, L.stream>>>(rp, pix0, npix, nullptr, w.val, lut, rgba);
+    return cudaGetLastError();
+  }
+  if ((e = cudaMemsetAsync(w.cnt, 0, sizeof(uint32_t) * nb, L.stream)) != cudaSuccess) return e;
   k_render_gen<<<blocks_for(total, 256, L.num_sms), 256, 0, L.stream>>>(rp, pix0, npix, w.loc, w.rank, w.bid, w.cnt);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_render_offsets<<<1, 32, 0, L.stream>>>(nb, w.cnt, w.off);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_render_scatter<<<blocks_for(total, 256, L.num_sms), 256, 0, L.stream>>>(total, w.loc, w.rank, w.bid, w.off, w.xyz, w.pos);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  Bricks br{};
-  br.n = nb;
   br.dev = w.off;
   Grads gr{};
   TrainWs tw{};
-  e = md.F16 ? launch_forward_bf16(L, md, br, w.xyz, w.val)
-             : launch_query_fp32(L, kForward, md, gr, br, tw, w.xyz, nullptr, w.val);
-  if (e != cudaSuccess) return e;
-  k_render_composite<<<(npix + 127) / 128, 128, 0, L.stream>>>(rp, pix0, npix, w.pos, w.val, lut, rgba);
+  if ((e = launch_query_fp32(L, kForward, md, gr, br, tw, w.xyz, nullptr, w.val)) != cudaSuccess) return e;
+  k_render_composite<true><<<(npix + 31) / 32, 32 * kSegs, 0, L.stream>>>(rp, pix0, npix, w.pos, w.val, lut, rgba);
   return cudaGetLastError();
 }
 
@@ -295,6 +245,50 @@ cudaError_t launch_render_preview(const Launch& L, const RenderParams& rp, int d
   k_render_preview<<<(n + 255) / 256, 256, 0, L.stream>>>(rp, done, level, reinterpret_cast<const float4*>(rgba),
                                                          reinterpret_cast<float4*>(preview));
   return cudaGetLastError();
+}
+
+cudaError_t launch_decode_bf16(const Launch& L, const RenderParams& rp, const Model& md, float* out) {
+  FwdSource src{};
+  src.kind = kFwdDecode;
+  src.rp = rp;
+  src.dec.vox = rp.vox;
+  int n[3], nb = 1;
+  int64_t voxels = 1;
+  for (int a = 0; a < 3; ++a) {
+    src.dec.grid[a] = rp.grid[a];
+    nb *= rp.grid[a];
+    voxels *= rp.vox;
+    n[a] = 0;   // the longest brick along the axis
+    for (int c = 0; c < rp.grid[a]; ++c)
+      n[a] = std::max(n[a], (int)(decode_first(rp.vox, c + 1, rp.grid[a]) - decode_first(rp.vox, c, rp.grid[a])));
+    if (n[a] == 0) return cudaSuccess;
+  }
+  // Blocks of at most `cap` voxels: as large as they go while there are a few for every CTA,
+  // and of the shape with the fewest 128-sample tiles over the bricks, compact ones first.
+  int cap = kFwdGroup;
+  while (cap > 128 && voxels / cap < 8 * (int64_t)L.num_sms) cap /= 2;
+  double best = 0.0;
+  for (int x = 1; x <= std::min(16, n[0]); ++x)
+    for (int y = 1; y <= std::min(16, n[1]); ++y)
+      for (int z = 1; z <= std::min(16, n[2]) && x * y * z <= cap; ++z) {
+        const int64_t blocks = (int64_t)((n[0] + x - 1) / x) * ((n[1] + y - 1) / y) * ((n[2] + z - 1) / z);
+        const double cost = (double)blocks * ((x * y * z + 127) / 128 + 0.25) * (1.0 + 0.01 * (x + y + z));
+        if (best == 0.0 || cost < best) {
+          best = cost;
+          src.dec.blk[0] = x; src.dec.blk[1] = y; src.dec.blk[2] = z;
+        }
+      }
+  int64_t groups = nb;
+  for (int a = 0; a < 3; ++a) {
+    src.dec.nblk[a] = (n[a] + src.dec.blk[a] - 1) / src.dec.blk[a];
+    groups *= src.dec.nblk[a];
+  }
+  if (groups > INT32_MAX) return cudaErrorInvalidValue;
+  src.group = (src.dec.blk[0] * src.dec.blk[1] * src.dec.blk[2] + 127) / 128 * 128;
+  src.groups = (int)groups;
+  Bricks br{};
+  br.n = nb;
+  return launch_forward_bf16(L, md, br, src, out);
 }
 
 cudaError_t launch_decode_chunk(const Launch& L, const DecodeChunk& c, const RenderWs& w, const Model& md,
@@ -310,9 +304,7 @@ cudaError_t launch_decode_chunk(const Launch& L, const DecodeChunk& c, const Ren
   for (int b = 0; b <= c.n_bricks; ++b) br.off[b] = b <= c.brick ? 0 : n;
   Grads gr{};
   TrainWs tw{};
-  e = md.F16 ? launch_forward_bf16(L, md, br, w.xyz, w.val)
-             : launch_query_fp32(L, kForward, md, gr, br, tw, w.xyz, nullptr, w.val);
-  if (e != cudaSuccess) return e;
+  if ((e = launch_query_fp32(L, kForward, md, gr, br, tw, w.xyz, nullptr, w.val)) != cudaSuccess) return e;
   k_decode_store<<<blocks_for(n, 256, L.num_sms), 256, 0, L.stream>>>(c, w.val, out);
   return cudaGetLastError();
 }

@@ -303,7 +303,7 @@ srn_status run_query(srn_handle* h, void* stream, srn::QueryMode mode, const srn
   if (h->cfg.precision != SRN_BF16)
     e = srn::launch_query_fp32(L, mode, md, gr, br, ws, xyz, target, out);
   else if (mode == srn::kForward)
-    e = srn::launch_forward_bf16(L, md, br, xyz, out);
+    e = srn::launch_forward_bf16(L, md, br, srn::point_source(L, br, xyz), out);
   else
     e = srn::launch_train_bf16(L, mode == srn::kTrainDensity, md, gr, br, ws, xyz, target, h->tune,
                                timed && time_kernel ? &mark : nullptr, h->side.stream ? &h->side : nullptr);
@@ -918,12 +918,24 @@ srn_status srn_decode(srn_handle* h, void* stream, const int32_t grid[3], const 
     }
   // voxel i of an axis with I bricks belongs to brick min(floor(I i / (vox - 1)), I - 1):
   // brick k holds [ceil(k (vox - 1) / I), ceil((k + 1)(vox - 1) / I) - 1] (the last one up to vox - 1)
-  auto first = [&](int k, int I) { return (int64_t)((k * (vox - 1) + I - 1) / I); };
+  auto first = [&](int k, int I) { return srn::decode_first(vox, k, I); };
   unsigned char* ws = h->ws;
   srn::RenderWs w{};
   w.xyz = reinterpret_cast<float*>(ws + h->wl.r_xyz);
   w.val = reinterpret_cast<float*>(ws + h->wl.r_val);
   const srn::Model md = h->model();
+  if (h->cfg.precision == SRN_BF16) {
+    srn::RenderParams rp{};
+    rp.vox = vox;
+    for (int a = 0; a < 3; ++a) rp.grid[a] = grid[a];
+    for (int b = 0; b < h->cfg.n_bricks; ++b)
+      for (int a = 0; a < 3; ++a) {
+        rp.lo[b][a] = (int32_t)boxes[6 * b + a];
+        rp.hi[b][a] = (int32_t)boxes[6 * b + 3 + a];
+      }
+    const cudaError_t e = srn::launch_decode_bf16(h->launch(stream), rp, md, out);
+    return e == cudaSuccess ? SRN_OK : cuda_fail(e, "decode");
+  }
   const int64_t cap = h->max_points;
   for (int bz = 0; bz < grid[2]; ++bz)
     for (int by = 0; by < grid[1]; ++by)
@@ -987,10 +999,6 @@ srn_status render_params(srn_handle* h, const srn_camera* cam, const float* lut,
   rp.width = width; rp.height = height; rp.samples = samples;
   rp.order = 0;
   rp.levels = 0;
-  // bundles of 8 rays x 16 samples when a batch holds at least one bundle of whole rays
-  const bool bundle = 8 * (((int64_t)samples + 15) / 16 * 16) <= h->max_points;
-  rp.rg = bundle ? 8 : 1;
-  rp.jb = bundle ? 16 : 1;
   while ((1 << rp.levels) < std::max(width, height)) ++rp.levels;
   for (int a = 0; a < 3; ++a) rp.grid[a] = grid[a];
   rp.vox = vox; rp.vmin = vmin; rp.vmax = vmax;
@@ -1005,7 +1013,7 @@ srn_status render_params(srn_handle* h, const srn_camera* cam, const float* lut,
 
 // Renders the pixels first .. first + count - 1 of rp's order in batches of at most
 // max_points samples.
-srn_status render_pixels(srn_handle* h, void* stream, const srn::RenderParams& rp, const float* lut,
+srn_status render_pixels(srn_handle* h, void* stream, const srn::RenderParams& rpi, const float* lut,
                          int64_t first, int64_t count, float* rgba) {
   unsigned char* ws = h->ws;
   srn::RenderWs w;
@@ -1017,9 +1025,18 @@ srn_status render_pixels(srn_handle* h, void* stream, const srn::RenderParams& r
   w.val = reinterpret_cast<float*>(ws + h->wl.r_val);
   w.cnt = reinterpret_cast<uint32_t*>(ws + h->wl.r_cnt);
   w.off = reinterpret_cast<int64_t*>(ws + h->wl.r_off);
-  // whole ray groups whose slots fit the workspace's max_points samples
-  const int64_t spr = ((int64_t)rp.samples + rp.jb - 1) / rp.jb * rp.jb;
-  const int64_t batch = h->max_points / spr / rp.rg * rp.rg;
+  // Ray groups of 64 neighbouring pixels (8 x 8 of the raster order), 16 of the progressive
+  // order's rows, fewer for a smaller image or workspace; a ray's samples are padded to
+  // whole query groups where that adds at most an eighth.
+  srn::RenderParams rp = rpi;
+  rp.rg = rp.order ? 16 : 64;
+  while (rp.rg > 1 && (rp.rg > count || (int64_t)rp.rg * rp.samples > h->max_points)) rp.rg /= 2;
+  const int per = srn::kFwdGroup / rp.rg;
+  const int64_t pad = ((int64_t)rp.samples + per - 1) / per * per;
+  rp.spr = pad * 8 <= (int64_t)rp.samples * 9 && pad * rp.rg <= h->max_points ? (int)pad : rp.samples;
+  // whole ray groups whose slots fit the workspace's max_points samples (and 31 bits)
+  const int64_t cap = std::min<int64_t>(h->max_points, (int64_t)1 << 30);
+  const int64_t batch = std::max<int64_t>(1, cap / rp.spr / rp.rg) * rp.rg;
   const srn::Model md = h->model();
   for (int64_t p0 = first; p0 < first + count; p0 += batch) {
     const int n = (int)std::min<int64_t>(batch, first + count - p0);
