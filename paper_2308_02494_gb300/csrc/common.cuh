@@ -55,6 +55,21 @@ struct Grads {
   int64_t sF, sW1, sW2, sw3;
 };
 
+// A batch of the caller's points and its Morton-sorted copy (launch_sort), which stands in
+// for it when more than `limit` of its points come before their predecessor: *moved is
+// counted on the device, so the choice needs no host round trip.  moved == NULL: no copy.
+struct SortedBatch {
+  float* xyz;          // [N][3] in bin order within each brick
+  float* target;       // [N] the targets in that order (training), or NULL
+  uint32_t* index;     // [N] the points' places in the caller's batch (queries), or NULL
+  uint32_t* rank;      // [N] scratch: rank inside the bin
+  uint32_t* hist;      // [B][kSortBins] bin starts within the brick (written with the copy)
+  uint32_t* moved;
+  uint32_t limit;
+  int32_t* ustart;     // training: [B][kUnits + 1] first point of each Morton unit, else NULL
+  __device__ __forceinline__ bool use() const { return moved && *moved > limit; }
+};
+
 // Workspace pieces the training kernels write.
 struct TrainWs {
   float* rho;       // [N] feature density of each point (Eq. 7)
@@ -73,8 +88,11 @@ struct TrainWs {
   uint16_t* gmax_blk;
   int32_t* ustart;    // [B][kUnits + 1] first point of each Morton unit (BF16 scatter tiles)
   const uint32_t* bin_start;   // [B][kSortBins] the sampler's bin starts of this batch, or NULL
+  SortedBatch sorted;          // its sorted copy, if one was made
   struct ScatTile* tiles;  // scatter tiles (BF16 training pass)
-  int32_t* tile_ctr;  // [0] tiles written, [1] next tile to take
+  // [0] tiles written; next tile to take of [1] the scatter, [2] the encoder, [3] the density
+  // gradient, [4] rho; cleared with the accumulators
+  int32_t* tile_ctr;
   const struct BrickSched* sched;   // per-brick training routine, or NULL (caller's flags)
   float eps;          // the density loss's epsilon (Eq. 8-9)
 };

@@ -60,6 +60,14 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
   return r;
 }
 
+// (1 - w) a + w b, rounded as trilinear_bf16's expression is (one product, one FMA):
+// packed over two channels, v = 1 - w, and for one.
+__device__ __forceinline__ unsigned long long blend2(unsigned long long a, unsigned long long b,
+                                                     unsigned long long w, unsigned long long v) {
+  return fma2(v, a, mul2(w, b));
+}
+__device__ __forceinline__ float blend1(float a, float b, float w, float v) { return fmaf(v, a, __fmul_rn(w, b)); }
+
 // axis_cell for two axes at once, u = (ua, ub) as a packed pair, hs2 = (hs, hs),
 // ct2 = (ct, ct), m2 = (kMagic, kMagic): the same roundings as two axis_cell calls.
 __device__ __forceinline__ void axis_cell2(unsigned long long u, unsigned long long hs2, unsigned long long ct2,
@@ -150,7 +158,8 @@ __device__ __forceinline__ void enc_stage(const EncBox& e, const EncNode<C>* __r
 // C bf16 (0 outside the grid: Eq. 2's inclusive mask), from the staged box when the
 // point's cell lies in it, else from global memory.  gi is the grid's transform, hs =
 // (R-1)/2, ct = hs - 1/2 + kMagic (used when R is even), Fi the grid's BF16 nodes.
-template <int C, bool EVEN_R>
+// PROD: the blend as trilinear_bf16's products ((1 - w) a + w b), else a + w (b - a).
+template <int C, bool EVEN_R, bool PROD>
 __device__ __forceinline__ uint32_t encode_point(const float (&gi)[12], float x, float y, float z, const EncBox& e,
                                                  float hs, float ct, int R, const __nv_bfloat16* Fi) {
   constexpr uint32_t kRow = 32 * sizeof(EncSNode<C>);
@@ -185,21 +194,24 @@ __device__ __forceinline__ uint32_t encode_point(const float (&gi)[12], float x,
       const uint32_t a1 = a0 + e.oy, a2 = a0 + e.oz, a3 = a2 + e.oy;
       if constexpr (C == 2) {
         const unsigned long long px = f2_bits(wx, wx), py = f2_bits(wy, wy), pz = f2_bits(wz, wz);
-        const unsigned long long e0 = lerp2(enc_node<C, 0>(a0), enc_node<C, kRow>(a0), px);
-        const unsigned long long e1 = lerp2(enc_node<C, 0>(a1), enc_node<C, kRow>(a1), px);
-        const unsigned long long e2 = lerp2(enc_node<C, 0>(a2), enc_node<C, kRow>(a2), px);
-        const unsigned long long e3 = lerp2(enc_node<C, 0>(a3), enc_node<C, kRow>(a3), px);
-        const unsigned long long f = lerp2(lerp2(e0, e1, py), lerp2(e2, e3, py), pz);
+        auto mix = [](unsigned long long a, unsigned long long b, float w, unsigned long long w2) {
+          if constexpr (PROD) return blend2(a, b, w2, f2_bits(1.f - w, 1.f - w));
+          else return lerp2(a, b, w2);
+        };
+        const unsigned long long e0 = mix(enc_node<C, 0>(a0), enc_node<C, kRow>(a0), wx, px);
+        const unsigned long long e1 = mix(enc_node<C, 0>(a1), enc_node<C, kRow>(a1), wx, px);
+        const unsigned long long e2 = mix(enc_node<C, 0>(a2), enc_node<C, kRow>(a2), wx, px);
+        const unsigned long long e3 = mix(enc_node<C, 0>(a3), enc_node<C, kRow>(a3), wx, px);
+        const unsigned long long f = mix(mix(e0, e1, wy, py), mix(e2, e3, wy, py), wz, pz);
         yv = pack_bf16(__uint_as_float((uint32_t)f), __uint_as_float((uint32_t)(f >> 32)));
       } else {
         const float v0 = enc_node<C, 0>(a0), v1 = enc_node<C, kRow>(a0);
         const float v2 = enc_node<C, 0>(a1), v3 = enc_node<C, kRow>(a1);
         const float v4 = enc_node<C, 0>(a2), v5 = enc_node<C, kRow>(a2);
         const float v6 = enc_node<C, 0>(a3), v7 = enc_node<C, kRow>(a3);
-        const float e0 = fmaf(wx, v1 - v0, v0), e1 = fmaf(wx, v3 - v2, v2);
-        const float e2 = fmaf(wx, v5 - v4, v4), e3 = fmaf(wx, v7 - v6, v6);
-        const float f01 = fmaf(wy, e1 - e0, e0), f23 = fmaf(wy, e3 - e2, e2);
-        yv = __bfloat16_as_ushort(__float2bfloat16_rn(fmaf(wz, f23 - f01, f01)));
+        auto mix = [](float a, float b, float w) { return PROD ? blend1(a, b, w, 1.f - w) : fmaf(w, b - a, a); };
+        const float e0 = mix(v0, v1, wx), e1 = mix(v2, v3, wx), e2 = mix(v4, v5, wx), e3 = mix(v6, v7, wx);
+        yv = __bfloat16_as_ushort(__float2bfloat16_rn(mix(mix(e0, e1, wy), mix(e2, e3, wy), wz)));
       }
     } else if (!EVEN_R || ((fabsf(ux) <= 1.f) & (fabsf(uy) <= 1.f) & (fabsf(uz) <= 1.f))) {
       yv = enc_global<C>(Fi, make_cell(ux, uy, uz, R), R);   // outside the box: corners from global memory

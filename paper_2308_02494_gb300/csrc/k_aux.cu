@@ -6,6 +6,7 @@
 //   * the batch sampler (Philox4x32-10, then a counting sort by 32^3 Morton bin);
 //   * the ground-truth lookup v(x) of Sec. 4.3.1 (trilinear in a float32 volume).
 #include <algorithm>
+#include <cooperative_groups.h>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -63,6 +64,7 @@ k_density_rho(Model md, Bricks brp, TrainWs ws, const float* __restrict__ xyz) {
   __shared__ double red[RHT / 32];
   __shared__ int s_tile;
   load_bricks(brp, br);
+  if (ws.sorted.use()) xyz = ws.sorted.xyz;
   const int tid = threadIdx.x, lane = tid & 31, M = md.M;
   if (tid == 0) build_tile_map(br, RHP, tm);
   __syncthreads();
@@ -232,6 +234,7 @@ k_density_grad(Model md, Bricks br, TrainWs ws, const float* __restrict__ xyz, f
   __shared__ float sg[kMaxGrids * 12];
   __shared__ double red[DNT];
   __shared__ int s_tile;
+  if (ws.sorted.use()) xyz = ws.sorted.xyz;
   const int tid = threadIdx.x, M = md.M;
   const int npg = DNT / M;             // point groups (M divides 256)
   const int gi = tid % M, pg = tid / M;
@@ -581,16 +584,15 @@ __global__ void k_sample_gen(Bricks br, unsigned long long seed, unsigned long l
   }
 }
 
-// Exclusive scan of one brick's kSortBins counters (one block of 1024 threads per brick):
-// each warp scans 1024 consecutive counters, 128 at a time (a lane reads four, so every
+// Exclusive scan of one brick's kSortBins counters by a block of 1024 threads: each warp scans 1024 consecutive counters, 128 at a time (a lane reads four, so every
 // load of a warp is one line), with shuffles, and one warp scans the 32 warp totals.
 // (With 32 consecutive counters per thread every load touched 32 lines: 11 us.)
-__global__ void __launch_bounds__(1024) k_sample_scan(uint32_t* hist) {
+__device__ __forceinline__ void scan_bins(uint32_t* hist) {
   constexpr int rounds = kSortBins / 32 / 128;
   static_assert(rounds * 32 * 128 == kSortBins, "a warp's counters are whole rounds of 128");
   __shared__ uint32_t wsum[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint4* h = reinterpret_cast<uint4*>(hist + (int64_t)blockIdx.x * kSortBins) + warp * (rounds * 32) + lane;
+  uint4* h = reinterpret_cast<uint4*>(hist) + warp * (rounds * 32) + lane;
   uint4 v[rounds];
   uint32_t incl[rounds];
 #pragma unroll
@@ -632,6 +634,9 @@ __global__ void __launch_bounds__(1024) k_sample_scan(uint32_t* hist) {
     h[32 * k] = make_uint4(s, s + v[k].x, s + v[k].x + v[k].y, s + v[k].x + v[k].y + v[k].z);
   }
 }
+__global__ void __launch_bounds__(1024) k_sample_scan(uint32_t* hist) {
+  scan_bins(hist + (int64_t)blockIdx.x * kSortBins);
+}
 
 // Pass 2 (after the scan): the point drawn again (cheaper than storing and re-reading
 // it) and written at its bin's start plus its rank.
@@ -646,6 +651,86 @@ __global__ void k_sample_scatter(Bricks br, unsigned long long seed, unsigned lo
     const float3 p = draw_point((uint32_t)(gi - br.off[b]), b, s, key);
     const int64_t dst = br.off[b] + hist[(int64_t)b * kSortBins + morton_bin(p.x, p.y, p.z)] + rank[gi];
     xyz[3 * dst] = p.x; xyz[3 * dst + 1] = p.y; xyz[3 * dst + 2] = p.z;
+  }
+}
+
+// ------------------------------------------------------------ sorted copy of a batch
+// Neighbouring points of a batch in no order share nothing: each corner read of a warp
+// touches 32 lines, a tile's node boxes cover the grid, and the scatter takes one global
+// atomic per corner.  The counting sort of the sampler on points in memory costs 24 bytes
+// per point and two atomics' latencies (about 0.05 ns per point) and makes such a batch
+// what the sampler's is.
+// One cooperative launch (as launches of their own the phases cost 17 us of a 32768-point
+// query): clear the counters; for a training batch the unit starts and how many units come
+// before their predecessor; ranks, bin counts and, for a query, how many points come before
+// their predecessor; then, if the batch needs the copy, scan and write it.
+constexpr int kSortNT = 1024;
+
+__global__ void __launch_bounds__(kSortNT) k_sort(Bricks br, const float* __restrict__ xyz,
+                                                  const float* __restrict__ target, SortedBatch s) {
+  cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+  const bool units = s.ustart != nullptr;
+  const int64_t total = br.off[br.n], first = (int64_t)blockIdx.x * kSortNT + threadIdx.x;
+  const int64_t step = (int64_t)gridDim.x * kSortNT;
+  const int lane = threadIdx.x & 31;
+  uint4* h4 = reinterpret_cast<uint4*>(s.hist);
+  for (int64_t q = first; q < (int64_t)br.n * kSortBins / 4; q += step) h4[q] = make_uint4(0u, 0u, 0u, 0u);
+  if (units)
+    for (int64_t q = first; q < (int64_t)br.n * (kUnits + 1); q += step) s.ustart[q] = -1;
+  if (first == 0) *s.moved = 0u;
+  grid.sync();
+  if (units) {   // first point of every unit that starts a run of that unit in its brick
+    uint32_t back = 0;
+    for (int64_t gi = first; gi < total; gi += step) {
+      const int b = brick_of_point(br, gi);
+      const int64_t p = gi - br.off[b];
+      const float* q = xyz + 3 * gi;
+      const uint32_t u = morton_bin(q[0], q[1], q[2]) >> 3;
+      const uint32_t before = p == 0 ? u : morton_bin(q[-3], q[-2], q[-1]) >> 3;
+      if (p == 0 || before != u) s.ustart[(int64_t)b * (kUnits + 1) + u] = (int32_t)p;
+      back += before > u;
+    }
+    back = __reduce_add_sync(0xffffffffu, back);
+    if (lane == 0 && back) atomicAdd(s.moved, back);
+    grid.sync();
+    if (*(volatile uint32_t*)s.moved <= s.limit) return;
+  }
+  uint32_t moved = 0;
+  for (int64_t gi = first; gi - lane < total; gi += step) {
+    const bool in = gi < total;
+    uint32_t key = 0xffffffffu;
+    if (in) {
+      const int b = brick_of_point(br, gi);
+      const uint32_t c = morton_bin(xyz[3 * gi], xyz[3 * gi + 1], xyz[3 * gi + 2]);
+      key = (uint32_t)b * kSortBins + c;
+      if (!units && gi > br.off[b] && morton_bin(xyz[3 * gi - 3], xyz[3 * gi - 2], xyz[3 * gi - 1]) > c) ++moved;
+    }
+    // one atomic per distinct bin of the warp
+    const unsigned grp = __match_any_sync(0xffffffffu, key);
+    const int leader = __ffs(grp) - 1;
+    uint32_t r = 0;
+    if (in && lane == leader) r = atomicAdd(s.hist + key, (uint32_t)__popc(grp));
+    r = __shfl_sync(0xffffffffu, r, leader);
+    if (in) s.rank[gi] = r + __popc(grp & ((1u << lane) - 1u));
+  }
+  if (!units) {
+    moved = __reduce_add_sync(0xffffffffu, moved);
+    if (lane == 0 && moved) atomicAdd(s.moved, moved);
+  }
+  grid.sync();
+  if (*(volatile uint32_t*)s.moved <= s.limit) return;
+  for (int b = blockIdx.x; b < br.n; b += gridDim.x) {
+    scan_bins(s.hist + (int64_t)b * kSortBins);
+    __syncthreads();
+  }
+  grid.sync();
+  for (int64_t gi = first; gi < total; gi += step) {
+    const int b = brick_of_point(br, gi);
+    const float x = xyz[3 * gi], y = xyz[3 * gi + 1], z = xyz[3 * gi + 2];
+    const int64_t dst = br.off[b] + s.hist[(int64_t)b * kSortBins + morton_bin(x, y, z)] + s.rank[gi];
+    s.xyz[3 * dst] = x; s.xyz[3 * dst + 1] = y; s.xyz[3 * dst + 2] = z;
+    if (s.target) s.target[dst] = target[gi];
+    if (s.index) s.index[dst] = (uint32_t)gi;
   }
 }
 
@@ -720,8 +805,6 @@ int blocks_for(int64_t n, int threads, int num_sms, int per_sm) {
 cudaError_t launch_density_rho(const Launch& L, const Model& md, const Bricks& br, const TrainWs& ws,
                                const float* xyz) {
   if (br.off[br.n] == 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(ws.tile_ctr + 4, 0, sizeof(int32_t), L.stream);
-  if (e != cudaSuccess) return e;
   if (md.p == 10) k_density_rho<true><<<L.num_sms, RHT, 0, L.stream>>>(md, br, ws, xyz);
   else k_density_rho<false><<<L.num_sms, RHT, 0, L.stream>>>(md, br, ws, xyz);
   return cudaGetLastError();
@@ -740,7 +823,6 @@ cudaError_t launch_density(const Launch& L, const Model& md, const Bricks& br, c
   int tiles = 0;
   for (int b = 0; b < br.n; ++b) tiles += (int)((br.off[b + 1] - br.off[b] + DT - 1) / DT);
   const int grid = tiles < ctas_per_sm * L.num_sms ? tiles : ctas_per_sm * L.num_sms;   // 8 warps each
-  if ((e = cudaMemsetAsync(ws.tile_ctr + 3, 0, sizeof(int32_t), L.stream)) != cudaSuccess) return e;
   if (md.p == 10) k_density_grad<true><<<grid, DNT, 0, L.stream>>>(md, br, ws, xyz, eps);
   else k_density_grad<false><<<grid, DNT, 0, L.stream>>>(md, br, ws, xyz, eps);
   return cudaGetLastError();
@@ -795,6 +877,16 @@ cudaError_t launch_sample(const Launch& L, const Bricks& br, unsigned long long 
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_sample_scatter<<<blocks, 256, 0, L.stream>>>(br, seed, step, step_dev, rank, hist, xyz);
   return cudaGetLastError();
+}
+
+cudaError_t launch_sort(const Launch& L, const Bricks& br, const float* xyz, const float* target,
+                        const SortedBatch& s) {
+  const int64_t total = br.off[br.n];
+  if (total == 0) return cudaSuccess;
+  // (at most one CTA per SM: all of them are resident, as the grid's barriers need)
+  const int blocks = blocks_for(total, kSortNT, L.num_sms, 1);
+  void* args[] = {(void*)&br, (void*)&xyz, (void*)&target, (void*)&s};
+  return cudaLaunchCooperativeKernel((const void*)k_sort, dim3(blocks), dim3(kSortNT), args, 0, L.stream);
 }
 
 cudaError_t launch_target(const Launch& L, const Bricks& br, const float* vol, int64_t dx,

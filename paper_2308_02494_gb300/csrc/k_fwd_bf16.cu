@@ -64,14 +64,6 @@ struct FwdLay {
   static constexpr int POOL = (STG + M * 12 + 15) / 16 * 16;   // staged nodes, C float32 each
 };
 
-// (1 - w) a + w b, rounded as trilinear_bf16's expression is (one product, one FMA):
-// packed over two channels, v = 1 - w, and for one.
-__device__ __forceinline__ unsigned long long blend2(unsigned long long a, unsigned long long b,
-                                                     unsigned long long w, unsigned long long v) {
-  return fma2(v, a, mul2(w, b));
-}
-__device__ __forceinline__ float blend1(float a, float b, float w, float v) { return fmaf(v, a, __fmul_rn(w, b)); }
-
 // Node box of grid g over the block [lo, hi]: block_box with a margin that covers the
 // rounding of the per-sample map for any transform, so that every sample of the block
 // inside the grid has its cell in the box (no per-sample test is needed).
@@ -140,6 +132,8 @@ k_fwd_bf16(Model md, Bricks brp, FwdSource src, float* __restrict__ out, uint32_
     __syncthreads();
   }
   const int total = src.kind == kFwdPoints ? tm.first[br.n] : src.groups;
+  const bool copied = src.sorted.use();
+  const float* xyz = copied ? src.sorted.xyz : src.xyz;
   float4* xs = reinterpret_cast<float4*>(sm + L::X);
   float* w3s = reinterpret_cast<float*>(sm + L::W3);
   float* gs = reinterpret_cast<float*>(sm + L::G);
@@ -185,7 +179,7 @@ k_fwd_bf16(Model md, Bricks brp, FwdSource src, float* __restrict__ out, uint32_
         if (s < ns) {
           int b;
           if (src.kind == kFwdPoints) {
-            const float* q = src.xyz + 3 * (base + s);
+            const float* q = xyz + 3 * (base + s);
             v.x = q[0]; v.y = q[1]; v.z = q[2];
             b = hint;
           } else if (src.kind == kFwdRender) {
@@ -510,7 +504,7 @@ k_fwd_bf16(Model md, Bricks brp, FwdSource src, float* __restrict__ out, uint32_
             if (__float_as_int(xs[s].w) == b) {
               const float f = fmaf(t4 ? mhi : mlo, span, vmin);
               if (src.kind == kFwdDecode) out[decode_index(src, blk, s)] = f;
-              else out[base + s] = f;
+              else out[copied ? (int64_t)src.sorted.index[base + s] : base + s] = f;
             }
           }
         }

@@ -93,6 +93,7 @@ k_mlp_tc(Model md, Grads gr, Bricks brp, TrainWs ws, const float* __restrict__ t
   __shared__ uint32_t s_gmax[TK];   // largest |dL/dy| bits per grid of the tile being written
   __shared__ __align__(8) unsigned long long mbar_s, mbar_y_s;
   load_bricks(brp, br);
+  if (ws.sorted.use()) target = ws.sorted.target;
   const uint32_t base0 = su32(raw), base = (base0 + 1023u) & ~1023u;
   unsigned char* sm = raw + (base - base0);
   const uint32_t sY = base + TcLay::Y, sW1 = base + TcLay::W1, sW2 = base + TcLay::W2;

@@ -12,7 +12,7 @@
 //          K = 128 runs on tcgen05 instead (k_mlp_tc.cu).
 //  k_scat  adjoint of Eq. 2.  A tile is up to tile_points (<= 1024) points of one brick
 //          lying in one aligned Morton range of the sampler's bins (a small
-//          axis-aligned block of the brick), listed by k_unit_starts / k_tile_list.
+//          axis-aligned block of the brick), listed by k_tile_list.
 //          Two CTAs per SM take (tile, group of 32 grids) units.  Lane l of a warp
 //          takes grid l of the group: the block, mapped through the grid's Eq. 1,
 //          bounds a node box that the tile's level keeps within shared memory, and the
@@ -71,6 +71,7 @@ k_mlp(Model md, Grads gr, Bricks brp, TrainWs ws, const float* __restrict__ targ
   __shared__ TileMap tm;
   __shared__ Bricks br;
   load_bricks(brp, br);
+  if (ws.sorted.use()) target = ws.sorted.target;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g8 = lane >> 2, t4 = lane & 3;
   const int M = md.M, C = md.C;
@@ -478,22 +479,6 @@ __device__ __forceinline__ uint32_t dy_bits(const __nv_bfloat16* dY, int64_t p, 
   else return (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(dY) + p * M + g);
 }
 
-// First point of every Morton unit (2 x 2 x 2 bins) that starts a run of that unit in
-// each brick's batch; the other entries keep the -1 they were cleared to.
-__global__ void k_unit_starts(Bricks brp, const float* __restrict__ xyz, int32_t* __restrict__ ustart) {
-  __shared__ Bricks br;
-  load_bricks(brp, br);
-  __syncthreads();
-  const int b = blockIdx.y;
-  const int64_t o = br.off[b], n = br.off[b + 1] - o;
-  int32_t* us = ustart + (int64_t)b * (kUnits + 1);
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-    const float* q = xyz + 3 * (o + p);
-    const uint32_t u = morton_bin(q[0], q[1], q[2]) >> 3;
-    if (p == 0 || (morton_bin(q[-3], q[-2], q[-1]) >> 3) != u) us[u] = (int32_t)p;
-  }
-}
-
 // One CTA per brick.  The brick's largest tile level lmax is the largest L <= lcap whose
 // block, mapped through any of the brick's grids, has a node box of at most capn nodes:
 // per grid axis, the image's extent in cells plus the box margin, one partial cell at
@@ -535,14 +520,14 @@ __global__ void __launch_bounds__(1024) k_tile_list(Bricks brp, TrainWs ws, Mode
   const int64_t o = br.off[b];
   const int32_t n = (int32_t)(br.off[b + 1] - o);
   const int32_t* us = ws.ustart + (int64_t)b * (kUnits + 1);
+  const uint32_t* bins = ws.bin_start ? ws.bin_start : ws.sorted.use() ? ws.sorted.hist : nullptr;
   int32_t loc[UPT];
   {
     int32_t m = INT_MAX;
 #pragma unroll
     for (int k = UPT - 1; k >= 0; --k) {
-      // a batch from the sampler: unit u starts where its first bin starts
-      const int32_t v = ws.bin_start ? (int32_t)ws.bin_start[(int64_t)b * kSortBins + ((tid * UPT + k) << 3)]
-                                     : us[tid * UPT + k];
+      // a batch from the sampler or a sorted copy: unit u starts where its first bin starts
+      const int32_t v = bins ? (int32_t)bins[(int64_t)b * kSortBins + ((tid * UPT + k) << 3)] : us[tid * UPT + k];
       if (v >= 0) m = min(m, v);
       loc[k] = m;
     }
@@ -641,6 +626,7 @@ k_scat(Model md, Grads gr, Bricks brp, TrainWs ws, const float* __restrict__ xyz
   __shared__ Bricks br;
   __shared__ TileMap dtm;   // the decoder's 128-point tiles (ws.gmax_blk)
   load_bricks(brp, br);
+  if (ws.sorted.use()) xyz = ws.sorted.xyz;
   if (threadIdx.x == 0) build_tile_map(br, 128, dtm);
   const int tid = threadIdx.x, lane = tid & 31;
   const int M = md.M, R = md.R;
@@ -885,6 +871,10 @@ k_enc(Model md, Bricks brp, TrainWs ws, const float* __restrict__ xyz, int capn)
   SE* boxes = reinterpret_cast<SE*>(smraw + sizeof(EncHead));   // [capn][32 columns]
   __shared__ Bricks br;
   load_bricks(brp, br);
+  // a batch that was not sorted reads Eq. 2 in the form that its points used to take (all
+  // of them outside their tiles' boxes), so that the features keep their bits
+  const bool copied = ws.sorted.use();
+  if (copied) xyz = ws.sorted.xyz;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int M = md.M, R = md.R;
   const int ngrp = M >= 32 ? M >> 5 : 1;
@@ -932,10 +922,18 @@ k_enc(Model md, Bricks brp, TrainWs ws, const float* __restrict__ xyz, int capn)
     const float ct = hs - 0.5f + kMagic;   // an integer when R is even (axis_cell)
     E* Yt = reinterpret_cast<E*>(ws.Y) + p0 * M + mp.g;
     const __nv_bfloat16* Fi = md.F16 + (int64_t)b * md.sF + mp.g * gsz;
+    if (!copied) {
 #pragma unroll 2
-    for (int p = mp.pg; p < np; p += mp.npg) {
-      const float4 x = h.xs[p];
-      Yt[p * M] = (E)encode_point<C, EVEN_R>(gi, x.x, x.y, x.z, eb, hs, ct, R, Fi);
+      for (int p = mp.pg; p < np; p += mp.npg) {
+        const float4 x = h.xs[p];
+        Yt[p * M] = (E)encode_point<C, EVEN_R, false>(gi, x.x, x.y, x.z, eb, hs, ct, R, Fi);
+      }
+    } else {
+#pragma unroll 2
+      for (int p = mp.pg; p < np; p += mp.npg) {
+        const float4 x = h.xs[p];
+        Yt[p * M] = (E)encode_point<C, EVEN_R, true>(gi, x.x, x.y, x.z, eb, hs, ct, R, Fi);
+      }
     }
   }
 }
@@ -957,6 +955,7 @@ __global__ void __launch_bounds__(RNT) k_rec_dg(Model md, Bricks brp, TrainWs ws
   __shared__ float sg[kMaxGrids * 12];
   __shared__ double red[RNT];
   load_bricks(brp, br);
+  if (ws.sorted.use()) xyz = ws.sorted.xyz;
   const int tid = threadIdx.x, M = md.M, R = md.R;
   const int npg = RNT / M, gi = tid % M, pg = tid / M;   // M divides RNT (M = K / C, a power of two)
   if (tid == 0) build_tile_map(br, RT, tm);
@@ -1099,14 +1098,9 @@ cudaError_t launch_train_k(const Launch& L, bool dens, const Model& md, const Gr
     int64_t nmax = 0;
     for (int b = 0; b < br.n; ++b) nmax = std::max<int64_t>(nmax, br.off[b + 1] - br.off[b]);
     if (nmax > INT32_MAX) return cudaErrorInvalidValue;
-    if ((e = cudaMemsetAsync(ws.tile_ctr, 0, 3 * sizeof(int32_t), L.stream)) != cudaSuccess) return e;
-    if (!ws.bin_start) {   // else the sampler's histogram gives the unit starts
-      if ((e = cudaMemsetAsync(ws.ustart, 0xff, sizeof(int32_t) * (kUnits + 1) * br.n, L.stream)) != cudaSuccess)
-        return e;
-      const int bx = (int)std::min<int64_t>((nmax + 255) / 256, 4 * L.num_sms / std::max(1, br.n) + 1);
-      k_unit_starts<<<dim3(bx, br.n), 256, 0, L.stream>>>(br, xyz, ws.ustart);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
+    // unit starts (the sampler's histogram gives those of its batch), and a sorted copy if
+    // the batch is out of order
+    if (!ws.bin_start && (e = launch_sort(L, br, xyz, target, ws.sorted)) != cudaSuccess) return e;
     const int cap = std::min(scat_capn(md.M, md.C), enc_capn(md.M, md.C));   // both kernels' boxes fit
     if (cap < 8) return cudaErrorInvalidConfiguration;
     if (tn.tile_points < kMinTilePoints || tn.tile_points > ST || tn.tile_level < 0 || tn.tile_level > kMaxTileLevel)

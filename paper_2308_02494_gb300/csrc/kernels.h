@@ -120,6 +120,11 @@ cudaError_t launch_shadow(const Launch& L, const float* p, uint16_t* shadow, int
 cudaError_t launch_sample(const Launch& L, const Bricks& br, unsigned long long seed,
                           unsigned long long step, const unsigned long long* step_dev,
                           float* xyz, uint32_t* rank, uint32_t* hist);
+// The order of a batch in memory and, when more than s.limit of its points are out of it,
+// its Morton-sorted copy: the points with their targets and, first, the batch's unit starts
+// (training: s.target and s.ustart set) or with their places (queries: s.index set).
+cudaError_t launch_sort(const Launch& L, const Bricks& br, const float* xyz, const float* target,
+                        const SortedBatch& s);
 struct VolumeBoxes {
   int32_t lo[SRN_MAX_BRICKS][3];
   int32_t hi[SRN_MAX_BRICKS][3];

@@ -181,7 +181,8 @@ struct FwdSource {
   int32_t kind;
   int32_t group, groups;   // (kFwdPoints counts its groups per brick itself)
   int32_t run;             // consecutive groups of a CTA (set by the launch)
-  const float* xyz;        // kFwdPoints
+  const float* xyz;        // kFwdPoints, and their sorted copy, if one was made
+  SortedBatch sorted;
   int32_t pix0, npix;      // kFwdRender: rays pix0 .. pix0 + npix - 1 of rp's order
   DecodeParams dec;        // kFwdDecode; the bricks' boxes are rp.lo, rp.hi
   RenderParams rp;

@@ -4,6 +4,7 @@
 #include <cstdio>
 #include <cstring>
 #include <algorithm>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -84,12 +85,15 @@ struct WsLayout {
   size_t state, acc, gsum, rsum, rho, herr, sort_rank, sort_hist, feat, dfeat, gmax, ustart, tiles, tile_ctr;
   size_t sched, sring;
   size_t r_loc, r_rank, r_bid, r_pos, r_xyz, r_val, r_cnt, r_off, total;
+  size_t t_xyz, t_target, t_rank, t_hist, q_xyz, q_index, q_rank, q_hist;
 };
 
 WsLayout ws_layout(const srn_config* c, int64_t maxp) {
   WsLayout w{};
   size_t o = 0;
   w.state = o; o += align256(sizeof(srn::StepState) + 64);
+  // (from here to r_sum's end: cleared by every backward pass)
+  w.tile_ctr = o; o += align256(sizeof(int32_t) * 5);
   w.acc = o; o += align256(sizeof(double) * srn::kAccPerBrick * c->n_bricks);
   w.gsum = o; o += align256(sizeof(double) * 13 * c->n_grids * c->n_bricks);
   w.rsum = o; o += align256(sizeof(double) * 12 * c->n_grids * c->n_bricks);
@@ -110,7 +114,6 @@ WsLayout ws_layout(const srn_config* c, int64_t maxp) {
   const int64_t max_tiles = (int64_t)c->n_bricks * (srn::kUnits + 1) + maxp / srn::kMinTilePoints + 1;
   w.ustart = o; o += bf16 ? align256(sizeof(int32_t) * (srn::kUnits + 1) * c->n_bricks) : 0;
   w.tiles = o; o += bf16 ? align256(sizeof(srn::ScatTile) * max_tiles) : 0;
-  w.tile_ctr = o; o += align256(sizeof(int32_t) * 4);
   w.sched = o; o += align256(sizeof(srn::BrickSched) * c->n_bricks);
   w.sring = o; o += align256(sizeof(double) * 2 * srn::kMaxDensityWindow * c->n_bricks);
   w.r_loc = o; o += align256(sizeof(float) * 3 * maxp);
@@ -121,6 +124,16 @@ WsLayout ws_layout(const srn_config* c, int64_t maxp) {
   w.r_val = o; o += align256(sizeof(float) * maxp);
   w.r_cnt = o; o += align256(sizeof(uint32_t) * c->n_bricks);
   w.r_off = o; o += align256(sizeof(int64_t) * (c->n_bricks + 1));
+  // sorted copies of a batch in memory: one of the training pass, one of the queries
+  const size_t hist = align256(sizeof(uint32_t) * ((size_t)srn::kSortBins * c->n_bricks + 1));   // and `moved`
+  w.t_xyz = o; o += align256(sizeof(float) * 3 * maxp);
+  w.t_target = o; o += align256(sizeof(float) * maxp);
+  w.t_rank = o; o += align256(sizeof(uint32_t) * maxp);
+  w.t_hist = o; o += hist;
+  w.q_xyz = o; o += align256(sizeof(float) * 3 * maxp);
+  w.q_index = o; o += align256(sizeof(uint32_t) * maxp);
+  w.q_rank = o; o += align256(sizeof(uint32_t) * maxp);
+  w.q_hist = o; o += hist;
   w.total = o;
   return w;
 }
@@ -174,6 +187,10 @@ struct srn_handle {
   // set by the training step around its backward pass: the batch is the sampler's, whose
   // histogram holds the bin starts the BF16 tile list needs
   const uint32_t* batch_bins = nullptr;
+  // srn_forward calls may come from several threads and streams: those that sort take the
+  // handle's one sorted copy in turn (query_done: the last one has read it)
+  std::mutex query_mu;
+  cudaEvent_t query_done = nullptr;
   // launch shape of the BF16 training pass (srn_set_tuning / srn_autotune)
   srn::Tuning tune = srn::kDefaultTuning;
 
@@ -206,7 +223,20 @@ struct srn_handle {
     w.sched = nullptr;
     w.eps = cfg.density_eps;
     w.bin_start = batch_bins;
+    w.sorted = srn::SortedBatch{};
     return w;
+  }
+  // Scratch of a training batch's (query's) sorted copy.
+  srn::SortedBatch sort_scratch(bool query) const {
+    srn::SortedBatch s{};
+    s.xyz = reinterpret_cast<float*>(ws + (query ? wl.q_xyz : wl.t_xyz));
+    if (query) s.index = reinterpret_cast<uint32_t*>(ws + wl.q_index);
+    else s.target = reinterpret_cast<float*>(ws + wl.t_target);
+    s.rank = reinterpret_cast<uint32_t*>(ws + (query ? wl.q_rank : wl.t_rank));
+    s.hist = reinterpret_cast<uint32_t*>(ws + (query ? wl.q_hist : wl.t_hist));
+    s.moved = s.hist + (size_t)srn::kSortBins * cfg.n_bricks;
+    if (!query) s.ustart = reinterpret_cast<int32_t*>(ws + wl.ustart);
+    return s;
   }
   srn::Model model() const {
     srn::Model m{};
@@ -265,6 +295,35 @@ srn_status check_training_counts(const srn::Bricks& br) {
   return SRN_OK;
 }
 
+// BF16 query of points in memory, through a sorted copy where that pays.  While `stream` is
+// being captured the copy is left alone: a replay could then meet another call's.
+cudaError_t forward_bf16(srn_handle* h, const srn::Launch& L, const srn::Model& md, const srn::Bricks& br,
+                         const float* xyz, float* out) {
+  srn::FwdSource src = srn::point_source(L, br, xyz);
+  const int64_t n = br.off[br.n];
+  // A sorted copy costs about 12 us and 0.05 ns per point.  It pays where the brick's grids
+  // are well beyond L1 (random points, with it and without: 1 MB of features, 32768 points
+  // 36 and 41 us; 8.4 MB, 53 and 84; 524288 points 161 and 430, 298 and 983); at 256 KB
+  // from about 250 thousand points on (131072: 58 and 48; 524288: 114 and 149), below
+  // that not at all (128 KB, 524288 points: 94 and 85).
+  const int64_t bytes = (int64_t)md.M * md.R * md.R * md.R * md.C * 2;
+  const int64_t least = bytes >= (512 << 10) ? 24576 : bytes >= (192 << 10) ? 262144 : INT64_MAX;
+  if (n < least || n > UINT32_MAX) return srn::launch_forward_bf16(L, md, br, src, out);
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(L.stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return srn::launch_forward_bf16(L, md, br, src, out);
+  }
+  std::lock_guard<std::mutex> lock(h->query_mu);
+  cudaError_t e = cudaStreamWaitEvent(L.stream, h->query_done, 0);   // (no-op before the first record)
+  if (e != cudaSuccess) return e;
+  src.sorted = h->sort_scratch(true);
+  src.sorted.limit = (uint32_t)(n / 32);   // scan lines and other nearly sorted batches stay as they are
+  if ((e = srn::launch_sort(L, br, xyz, nullptr, src.sorted)) != cudaSuccess) return e;
+  if ((e = srn::launch_forward_bf16(L, md, br, src, out)) != cudaSuccess) return e;
+  return cudaEventRecord(h->query_done, L.stream);
+}
+
 srn_status run_query(srn_handle* h, void* stream, srn::QueryMode mode, const srn::Bricks& br,
                      const float* xyz, const float* target, float* out, int upstream = 0,
                      const srn::BrickSched* sched = nullptr, int rec_dg = 0) {
@@ -303,10 +362,19 @@ srn_status run_query(srn_handle* h, void* stream, srn::QueryMode mode, const srn
   if (h->cfg.precision != SRN_BF16)
     e = srn::launch_query_fp32(L, mode, md, gr, br, ws, xyz, target, out);
   else if (mode == srn::kForward)
-    e = srn::launch_forward_bf16(L, md, br, srn::point_source(L, br, xyz), out);
-  else
+    e = forward_bf16(h, L, md, br, xyz, out);
+  else {
+    // A caller's batch that is out of order runs through a sorted copy (random points, with
+    // it and without: 2000 points 84 and 88 us at M = 8, R = 16, 162 and 293 at M = 64,
+    // R = 32; 131072 points 138 and 222, 271 and 720)
+    const int64_t n = br.off[br.n];
+    if (!ws.bin_start) {
+      ws.sorted = h->sort_scratch(false);
+      ws.sorted.limit = n >= 1024 && n <= UINT32_MAX ? (uint32_t)(n / 1024) : UINT32_MAX;
+    }
     e = srn::launch_train_bf16(L, mode == srn::kTrainDensity, md, gr, br, ws, xyz, target, h->tune,
                                timed && time_kernel ? &mark : nullptr, h->side.stream ? &h->side : nullptr);
+  }
   if (e != cudaSuccess) return cuda_fail(e, "query kernel");
   if (timed) {
     if (time_pass) cudaEventRecord(h->ev_stop[slot], L.stream);
@@ -339,7 +407,8 @@ srn_status do_backward(srn_handle* h, void* stream, const float* xyz, const floa
   const bool dens = (flags & SRN_DENSITY) != 0 || sched;
   cudaError_t e = cudaMemsetAsync(h->t.grads_dev, 0, sizeof(float) * h->lay.n_params, s);
   if (e == cudaSuccess)
-    e = cudaMemsetAsync(h->ws + h->wl.acc, 0, h->wl.rsum - h->wl.acc + sizeof(double) * 12 * h->cfg.n_grids * h->cfg.n_bricks, s);
+    e = cudaMemsetAsync(h->ws + h->wl.tile_ctr, 0,
+                        h->wl.rsum - h->wl.tile_ctr + sizeof(double) * 12 * h->cfg.n_grids * h->cfg.n_bricks, s);
   if (e != cudaSuccess) return cuda_fail(e, "memset");
   const int rec_dg = (flags & SRN_REC_DG) ? 1 : 0;
   h->side.defer_join = split;
@@ -475,7 +544,7 @@ srn_status srn_create(const srn_config* cfg, const srn_tensors* t, void* workspa
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return cuda_fail(e, "device query");
-  e = cudaMemset(static_cast<unsigned char*>(workspace) + wl.state, 0, wl.acc - wl.state);
+  e = cudaMemset(static_cast<unsigned char*>(workspace) + wl.state, 0, wl.tile_ctr - wl.state);
   if (e != cudaSuccess) return cuda_fail(e, "workspace init");
   srn_handle* h = new srn_handle();
   h->cfg = *cfg;
@@ -491,6 +560,7 @@ srn_status srn_create(const srn_config* cfg, const srn_tensors* t, void* workspa
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->side.fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->side.join, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->side.enc_done, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->query_done, cudaEventDisableTiming);
     if (e != cudaSuccess) {
       srn_destroy(h);
       return cuda_fail(e, "side stream");
@@ -512,6 +582,7 @@ srn_status srn_destroy(srn_handle* h) {
   if (h->side.join) cudaEventDestroy(h->side.join);
   if (h->side.enc_done) cudaEventDestroy(h->side.enc_done);
   if (h->side.stream) cudaStreamDestroy(h->side.stream);
+  if (h->query_done) cudaEventDestroy(h->query_done);
   delete h;
   return SRN_OK;
 }
