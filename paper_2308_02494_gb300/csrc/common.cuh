@@ -66,7 +66,6 @@ struct SortedBatch {
   uint32_t* hist;      // [B][kSortBins] bin starts within the brick (written with the copy)
   uint32_t* moved;
   uint32_t limit;
-  int32_t* ustart;     // training: [B][kUnits + 1] first point of each Morton unit, else NULL
   __device__ __forceinline__ bool use() const { return moved && *moved > limit; }
 };
 
@@ -86,7 +85,7 @@ struct TrainWs {
   // 128-point decoder tile (tiles numbered as build_tile_map numbers them for 128), or
   // NULL when the decoder does not produce them (the scatter then finds its scales itself)
   uint16_t* gmax_blk;
-  int32_t* ustart;    // [B][kUnits + 1] first point of each Morton unit (BF16 scatter tiles)
+  int32_t* ustart;    // [B][kUnits + 1] one more than the first point of each Morton unit, 0: none
   const uint32_t* bin_start;   // [B][kSortBins] the sampler's bin starts of this batch, or NULL
   SortedBatch sorted;          // its sorted copy, if one was made
   struct ScatTile* tiles;  // scatter tiles (BF16 training pass)

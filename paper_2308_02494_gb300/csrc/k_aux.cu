@@ -6,22 +6,13 @@
 //   * the batch sampler (Philox4x32-10, then a counting sort by 32^3 Morton bin);
 //   * the ground-truth lookup v(x) of Sec. 4.3.1 (trilinear in a float32 volume).
 #include <algorithm>
-#include <cooperative_groups.h>
 
 #include "common.cuh"
 #include "kernels.h"
+#include "sort.cuh"
 
 namespace srn {
 namespace {
-
-__device__ __forceinline__ int brick_of_point(const Bricks& br, int64_t g) {
-  int lo = 0, hi = br.n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (br.off[mid] <= g) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
 
 template <typename Tv>
 __device__ __forceinline__ Tv warp_sum(Tv v) {
@@ -175,6 +166,7 @@ __global__ void __launch_bounds__(ST) k_density_scalar(Bricks br, TrainWs ws, fl
   const int per = (total + gridDim.x - 1) / gridDim.x;
   const int tb = blockIdx.x * per, te = min(total, tb + per);
   float c_acc = 0.f, l_acc = 0.f;   // this thread's few points in float32; float64 across
+  __shared__ float s_inv[2];
   int cur = -1;
   float invS = 0.f, hbar = 0.f, n = 1.f;
   auto flush = [&](int b) {
@@ -199,8 +191,14 @@ __global__ void __launch_bounds__(ST) k_density_scalar(Bricks br, TrainWs ws, fl
       cur = b;
       const double nb = (double)(br.off[b + 1] - br.off[b]);
       n = (float)nb;
-      invS = (float)(1.0 / ws.acc[b * kAccPerBrick + ACC_SUM_RHO]);
-      hbar = (float)(ws.acc[b * kAccPerBrick + ACC_SUM_R2] / nb);
+      if (tid == 0) {   // (float64 divisions run at a few per clock and SM: one thread does them)
+        s_inv[0] = (float)(1.0 / ws.acc[b * kAccPerBrick + ACC_SUM_RHO]);
+        s_inv[1] = (float)(ws.acc[b * kAccPerBrick + ACC_SUM_R2] / nb);
+      }
+      __syncthreads();
+      invS = s_inv[0];
+      hbar = s_inv[1];
+      __syncthreads();
     }
     const int64_t p = br.off[b] + (int64_t)(tile - tm.first[b]) * ST + tid;
     if (p < br.off[b + 1] && !(ws.sched && !ws.sched[b].den_on)) {
@@ -221,7 +219,7 @@ constexpr int DT = 128;   // points per tile
 constexpr int DNT = 256;  // threads
 
 static_assert(sizeof(TileMap) + DT * 2 * sizeof(float4) + kMaxGrids * 12 * sizeof(float) +
-                  DNT * sizeof(double) + 1024 <= kDensityCtaSmem,
+                  DNT * sizeof(double) + 16 + 1024 <= kDensityCtaSmem,
               "k_density_grad's shared memory must fit beside the scatter");
 // P10: the paper's p = 10 at compile time, with the x and y axes of the map, the flat
 // top and the sums carried as packed float pairs (the same arithmetic, fewer issued
@@ -234,6 +232,7 @@ k_density_grad(Model md, Bricks br, TrainWs ws, const float* __restrict__ xyz, f
   __shared__ float sg[kMaxGrids * 12];
   __shared__ double red[DNT];
   __shared__ int s_tile;
+  __shared__ float s_inv[3];
   if (ws.sorted.use()) xyz = ws.sorted.xyz;
   const int tid = threadIdx.x, M = md.M;
   const int npg = DNT / M;             // point groups (M divides 256)
@@ -281,10 +280,15 @@ k_density_grad(Model md, Bricks br, TrainWs ws, const float* __restrict__ xyz, f
       for (int k = tid; k < M * 12; k += DNT) sg[k] = md.G[(int64_t)b * md.sG + k];
       const double nb = (double)(br.off[b + 1] - br.off[b]);
       n = (float)nb;
-      invS = (float)(1.0 / ws.acc[b * kAccPerBrick + ACC_SUM_RHO]);
-      hbar = (float)(ws.acc[b * kAccPerBrick + ACC_SUM_R2] / nb);
-      c = (float)ws.acc[b * kAccPerBrick + ACC_C];
+      if (tid == 0) {
+        s_inv[0] = (float)(1.0 / ws.acc[b * kAccPerBrick + ACC_SUM_RHO]);
+        s_inv[1] = (float)(ws.acc[b * kAccPerBrick + ACC_SUM_R2] / nb);
+        s_inv[2] = (float)ws.acc[b * kAccPerBrick + ACC_C];
+      }
       __syncthreads();
+      invS = s_inv[0];
+      hbar = s_inv[1];
+      c = s_inv[2];
       const float* g = sg + 12 * gi;
       gax = f2_pack(g[0], g[4]); gay = f2_pack(g[1], g[5]); gaz = f2_pack(g[2], g[6]); gt = f2_pack(g[3], g[7]);
       g8 = g[8]; g9 = g[9]; g10 = g[10]; g11 = g[11];
@@ -365,38 +369,36 @@ k_density_grad(Model md, Bricks br, TrainWs ws, const float* __restrict__ xyz, f
 }
 
 // ------------------------------------------------------------ finalisation
-// One block per brick: losses and (with the density step) dG from the sums.
-__global__ void k_finalize(Bricks br, Model md, TrainWs ws, int density, float* dG, int64_t sdG,
-                           double* losses) {
-  const int b = blockIdx.x, i = threadIdx.x;
-  const double n = (double)(br.off[b + 1] - br.off[b]);
+// Losses and (with the density step) dG from the sums: a block per brick and 8 grids, a
+// thread per entry of the grids' 3 x 4 maps.  The float64 arithmetic runs at a few operations
+// per clock and SM, so it is spread over SMs: one block per brick took 6.5 us.
+constexpr int kFinGrids = 8;
+__global__ void __launch_bounds__(12 * kFinGrids) k_finalize(Bricks br, Model md, TrainWs ws, int density, float* dG,
+                                                             int64_t sdG, double* losses) {
+  const int b = blockIdx.x, i = blockIdx.y * kFinGrids + threadIdx.x / 12, j = threadIdx.x % 12;
   const double* acc = ws.acc + b * kAccPerBrick;
   if (ws.sched) density = density && ws.sched[b].den_on;
-  if (ws.rec_dg && !density && i < md.M) {   // G's gradient is the part through the features alone
-    const double* r = ws.rsum + ((int64_t)b * md.M + i) * 12;
-    float* d = dG + (int64_t)b * sdG + 12 * i;
-    for (int j = 0; j < 12; ++j) d[j] = (float)r[j];
-  }
-  if (density && i < md.M) {
-    const float* g = md.G + (int64_t)b * md.sG + 12 * i;
-    const double a00 = g[0], a01 = g[1], a02 = g[2], a10 = g[4], a11 = g[5], a12 = g[6];
-    const double a20 = g[8], a21 = g[9], a22 = g[10];
-    // cofactors: det * A^{-T} is the cofactor matrix
-    const double c00 = a11 * a22 - a12 * a21, c01 = a12 * a20 - a10 * a22, c02 = a10 * a21 - a11 * a20;
-    const double c10 = a02 * a21 - a01 * a22, c11 = a00 * a22 - a02 * a20, c12 = a01 * a20 - a00 * a21;
-    const double c20 = a01 * a12 - a02 * a11, c21 = a02 * a10 - a00 * a12, c22 = a00 * a11 - a01 * a10;
-    const double det = a00 * c00 + a01 * c01 + a02 * c02;
-    const double* s = ws.gsum + ((int64_t)b * md.M + i) * 13;
-    float* d = dG + (int64_t)b * sdG + 12 * i;
-    const double cof[3][3] = {{c00, c01, c02}, {c10, c11, c12}, {c20, c21, c22}};
-    const double* rs = ws.rsum + ((int64_t)b * md.M + i) * 12;
-    const double rw = ws.rec_dg ? 1.0 : 0.0;   // plus the part through the features (SRN_REC_DG)
-    for (int r = 0; r < 3; ++r) {
-      for (int e = 0; e < 3; ++e) d[4 * r + e] = (float)(cof[r][e] * s[0] - det * s[4 + 3 * r + e] + rw * rs[4 * r + e]);
-      d[4 * r + 3] = (float)(-det * s[1 + r] + rw * rs[4 * r + 3]);
+  if ((density || ws.rec_dg) && i < md.M) {
+    double v = 0.0;
+    if (density) {
+      const float* g = md.G + (int64_t)b * md.sG + 12 * i;
+      const double* s = ws.gsum + ((int64_t)b * md.M + i) * 13;
+      // row r of det * A^{-T} (the cofactors): the product of A's two other rows, cyclically
+      const int r = j / 4, e = j % 4, r1 = (r + 1) % 3, r2 = (r + 2) % 3;
+      auto cof = [&](int c) {
+        const int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
+        return (double)g[4 * r1 + c1] * (double)g[4 * r2 + c2] - (double)g[4 * r1 + c2] * (double)g[4 * r2 + c1];
+      };
+      const double c0 = cof(0), c1 = cof(1), c2 = cof(2);
+      const double det = (double)g[4 * r] * c0 + (double)g[4 * r + 1] * c1 + (double)g[4 * r + 2] * c2;
+      v = e < 3 ? (e == 0 ? c0 : e == 1 ? c1 : c2) * s[0] - det * s[4 + 3 * r + e] : -det * s[1 + r];
     }
+    // the part through the features (SRN_REC_DG)
+    if (ws.rec_dg) v += ws.rsum[((int64_t)b * md.M + i) * 12 + j];
+    dG[(int64_t)b * sdG + 12 * i + j] = (float)v;
   }
-  if (i == 0) {
+  if (blockIdx.y == 0 && threadIdx.x == 0) {
+    const double n = (double)(br.off[b + 1] - br.off[b]);
     const double lrec = acc[ACC_SUM_R2] / n;
     const double lden = density ? acc[ACC_LDEN] : 0.0;
     if (!isfinite(lrec) || !isfinite(lden)) atomicOr(ws.status, 1);
@@ -584,56 +586,6 @@ __global__ void k_sample_gen(Bricks br, unsigned long long seed, unsigned long l
   }
 }
 
-// Exclusive scan of one brick's kSortBins counters by a block of 1024 threads: each warp scans 1024 consecutive counters, 128 at a time (a lane reads four, so every
-// load of a warp is one line), with shuffles, and one warp scans the 32 warp totals.
-// (With 32 consecutive counters per thread every load touched 32 lines: 11 us.)
-__device__ __forceinline__ void scan_bins(uint32_t* hist) {
-  constexpr int rounds = kSortBins / 32 / 128;
-  static_assert(rounds * 32 * 128 == kSortBins, "a warp's counters are whole rounds of 128");
-  __shared__ uint32_t wsum[32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint4* h = reinterpret_cast<uint4*>(hist) + warp * (rounds * 32) + lane;
-  uint4 v[rounds];
-  uint32_t incl[rounds];
-#pragma unroll
-  for (int k = 0; k < rounds; ++k) v[k] = h[32 * k];
-#pragma unroll
-  for (int k = 0; k < rounds; ++k) incl[k] = v[k].x + v[k].y + v[k].z + v[k].w;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {   // inclusive scans of the rounds' lane totals, side by side
-#pragma unroll
-    for (int k = 0; k < rounds; ++k) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, incl[k], o);
-      if (lane >= o) incl[k] += y;
-    }
-  }
-  uint32_t total = 0;
-#pragma unroll
-  for (int k = 0; k < rounds; ++k) {
-    const uint32_t t = __shfl_sync(0xffffffffu, incl[k], 31);
-    incl[k] += total - (v[k].x + v[k].y + v[k].z + v[k].w);   // exclusive within the warp
-    total += t;
-  }
-  if (lane == 0) wsum[warp] = total;
-  __syncthreads();
-  if (warp == 0) {
-    const uint32_t w = wsum[lane];
-    uint32_t wi = w;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, wi, o);
-      if (lane >= o) wi += y;
-    }
-    wsum[lane] = wi - w;   // exclusive
-  }
-  __syncthreads();
-  const uint32_t base = wsum[warp];
-#pragma unroll
-  for (int k = 0; k < rounds; ++k) {
-    const uint32_t s = base + incl[k];
-    h[32 * k] = make_uint4(s, s + v[k].x, s + v[k].x + v[k].y, s + v[k].x + v[k].y + v[k].z);
-  }
-}
 __global__ void __launch_bounds__(1024) k_sample_scan(uint32_t* hist) {
   scan_bins(hist + (int64_t)blockIdx.x * kSortBins);
 }
@@ -651,86 +603,6 @@ __global__ void k_sample_scatter(Bricks br, unsigned long long seed, unsigned lo
     const float3 p = draw_point((uint32_t)(gi - br.off[b]), b, s, key);
     const int64_t dst = br.off[b] + hist[(int64_t)b * kSortBins + morton_bin(p.x, p.y, p.z)] + rank[gi];
     xyz[3 * dst] = p.x; xyz[3 * dst + 1] = p.y; xyz[3 * dst + 2] = p.z;
-  }
-}
-
-// ------------------------------------------------------------ sorted copy of a batch
-// Neighbouring points of a batch in no order share nothing: each corner read of a warp
-// touches 32 lines, a tile's node boxes cover the grid, and the scatter takes one global
-// atomic per corner.  The counting sort of the sampler on points in memory costs 24 bytes
-// per point and two atomics' latencies (about 0.05 ns per point) and makes such a batch
-// what the sampler's is.
-// One cooperative launch (as launches of their own the phases cost 17 us of a 32768-point
-// query): clear the counters; for a training batch the unit starts and how many units come
-// before their predecessor; ranks, bin counts and, for a query, how many points come before
-// their predecessor; then, if the batch needs the copy, scan and write it.
-constexpr int kSortNT = 1024;
-
-__global__ void __launch_bounds__(kSortNT) k_sort(Bricks br, const float* __restrict__ xyz,
-                                                  const float* __restrict__ target, SortedBatch s) {
-  cooperative_groups::grid_group grid = cooperative_groups::this_grid();
-  const bool units = s.ustart != nullptr;
-  const int64_t total = br.off[br.n], first = (int64_t)blockIdx.x * kSortNT + threadIdx.x;
-  const int64_t step = (int64_t)gridDim.x * kSortNT;
-  const int lane = threadIdx.x & 31;
-  uint4* h4 = reinterpret_cast<uint4*>(s.hist);
-  for (int64_t q = first; q < (int64_t)br.n * kSortBins / 4; q += step) h4[q] = make_uint4(0u, 0u, 0u, 0u);
-  if (units)
-    for (int64_t q = first; q < (int64_t)br.n * (kUnits + 1); q += step) s.ustart[q] = -1;
-  if (first == 0) *s.moved = 0u;
-  grid.sync();
-  if (units) {   // first point of every unit that starts a run of that unit in its brick
-    uint32_t back = 0;
-    for (int64_t gi = first; gi < total; gi += step) {
-      const int b = brick_of_point(br, gi);
-      const int64_t p = gi - br.off[b];
-      const float* q = xyz + 3 * gi;
-      const uint32_t u = morton_bin(q[0], q[1], q[2]) >> 3;
-      const uint32_t before = p == 0 ? u : morton_bin(q[-3], q[-2], q[-1]) >> 3;
-      if (p == 0 || before != u) s.ustart[(int64_t)b * (kUnits + 1) + u] = (int32_t)p;
-      back += before > u;
-    }
-    back = __reduce_add_sync(0xffffffffu, back);
-    if (lane == 0 && back) atomicAdd(s.moved, back);
-    grid.sync();
-    if (*(volatile uint32_t*)s.moved <= s.limit) return;
-  }
-  uint32_t moved = 0;
-  for (int64_t gi = first; gi - lane < total; gi += step) {
-    const bool in = gi < total;
-    uint32_t key = 0xffffffffu;
-    if (in) {
-      const int b = brick_of_point(br, gi);
-      const uint32_t c = morton_bin(xyz[3 * gi], xyz[3 * gi + 1], xyz[3 * gi + 2]);
-      key = (uint32_t)b * kSortBins + c;
-      if (!units && gi > br.off[b] && morton_bin(xyz[3 * gi - 3], xyz[3 * gi - 2], xyz[3 * gi - 1]) > c) ++moved;
-    }
-    // one atomic per distinct bin of the warp
-    const unsigned grp = __match_any_sync(0xffffffffu, key);
-    const int leader = __ffs(grp) - 1;
-    uint32_t r = 0;
-    if (in && lane == leader) r = atomicAdd(s.hist + key, (uint32_t)__popc(grp));
-    r = __shfl_sync(0xffffffffu, r, leader);
-    if (in) s.rank[gi] = r + __popc(grp & ((1u << lane) - 1u));
-  }
-  if (!units) {
-    moved = __reduce_add_sync(0xffffffffu, moved);
-    if (lane == 0 && moved) atomicAdd(s.moved, moved);
-  }
-  grid.sync();
-  if (*(volatile uint32_t*)s.moved <= s.limit) return;
-  for (int b = blockIdx.x; b < br.n; b += gridDim.x) {
-    scan_bins(s.hist + (int64_t)b * kSortBins);
-    __syncthreads();
-  }
-  grid.sync();
-  for (int64_t gi = first; gi < total; gi += step) {
-    const int b = brick_of_point(br, gi);
-    const float x = xyz[3 * gi], y = xyz[3 * gi + 1], z = xyz[3 * gi + 2];
-    const int64_t dst = br.off[b] + s.hist[(int64_t)b * kSortBins + morton_bin(x, y, z)] + s.rank[gi];
-    s.xyz[3 * dst] = x; s.xyz[3 * dst + 1] = y; s.xyz[3 * dst + 2] = z;
-    if (s.target) s.target[dst] = target[gi];
-    if (s.index) s.index[dst] = (uint32_t)gi;
   }
 }
 
@@ -830,7 +702,8 @@ cudaError_t launch_density(const Launch& L, const Model& md, const Bricks& br, c
 
 cudaError_t launch_finalize(const Launch& L, const Bricks& br, const Model& md, const TrainWs& ws,
                             bool density, float* dG, int64_t sdG, double* losses) {
-  k_finalize<<<br.n, kMaxGrids, 0, L.stream>>>(br, md, ws, density ? 1 : 0, dG, sdG, losses);
+  k_finalize<<<dim3(br.n, (md.M + kFinGrids - 1) / kFinGrids), 12 * kFinGrids, 0, L.stream>>>(
+      br, md, ws, density ? 1 : 0, dG, sdG, losses);
   return cudaGetLastError();
 }
 
@@ -877,16 +750,6 @@ cudaError_t launch_sample(const Launch& L, const Bricks& br, unsigned long long 
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_sample_scatter<<<blocks, 256, 0, L.stream>>>(br, seed, step, step_dev, rank, hist, xyz);
   return cudaGetLastError();
-}
-
-cudaError_t launch_sort(const Launch& L, const Bricks& br, const float* xyz, const float* target,
-                        const SortedBatch& s) {
-  const int64_t total = br.off[br.n];
-  if (total == 0) return cudaSuccess;
-  // (at most one CTA per SM: all of them are resident, as the grid's barriers need)
-  const int blocks = blocks_for(total, kSortNT, L.num_sms, 1);
-  void* args[] = {(void*)&br, (void*)&xyz, (void*)&target, (void*)&s};
-  return cudaLaunchCooperativeKernel((const void*)k_sort, dim3(blocks), dim3(kSortNT), args, 0, L.stream);
 }
 
 cudaError_t launch_target(const Launch& L, const Bricks& br, const float* vol, int64_t dx,

@@ -1,567 +1,4 @@
-// BF16 forward query f(x) = d(e(x)) (Eq. 1-3 and Sec. 4.1.2) for srn_forward, the
-// renderer and the full-volume decode.
-//
-// A CTA takes groups of up to 512 neighbouring samples: consecutive points of a brick, a
-// bundle of ray samples (8 x 8 pixels x 8 samples), or a block of voxels, whose
-// coordinates it forms itself, so the renderer and the decode keep no coordinates in
-// memory.  Per group and brick the samples' bounding box, mapped through each grid's
-// Eq. 1, bounds the nodes that the grid can read; boxes that are worth it and fit are
-// staged in shared memory as the float32 values of their nodes.  Then 128 samples at a
-// time: a thread evaluates Eq. 1-2 for one or four samples and four grids (C = 2) before
-// it stores one 16-byte chunk of features (BF16, swizzled) each, and warp w runs the two hidden
-// layers for rows 16w..16w+15 on the tensor cores (m16n8k16, FP32 accumulate) and the
-// 64 -> 1 output layer in FP32.
-//
-// What bounds it: instruction issue and the shared-memory pipe (55% and 65% busy in a
-// decode).  Reading the corners from global memory took 116 warp instructions per 32
-// (sample, grid) pairs (unpacking BF16 nodes, float-int conversions, clamps) with the L1
-// pipe at 55-59%; staged float32 nodes need no unpacking, one address for eight reads and
-// packed f32x2 blends: 88.  319^3 decode of the paper-scale model 11.67 -> 8.4 ms, frame
-// of 1024^2 x 512 samples 220 -> 153 ms, progressive pass 418 -> 300 us (with the
-// coordinates, the brick sort and the serial compositing taken out of memory).
-// The blend is rounded as the global read's was, so the features are the same bits.
-#include <algorithm>
-
-#include "enc_ops.cuh"
-#include "kernels.h"
-#include "render.h"
-
-namespace srn {
-namespace {
-
-constexpr int T = 128;     // samples per feature tile
-constexpr int NT = 256;
-// CTAs per SM and samples per thread.  A thread's samples share the reads of a grid's map and
-// box (a warp-uniform 16-byte read takes two passes of the shared-memory pipe, 65% busy at
-// two samples per thread), which for K >= 64 pays for 128 registers and the two CTAs that
-// the feature tile and the boxes leave room for (frame of the paper-scale model: 157 ms at
-// two samples, 153 at four); the small models take three CTAs of one sample per thread
-// instead (progressive pass at K = 32: 318 and 292 us).
-constexpr int fwd_ctas(int K) { return K >= 64 ? 2 : 3; }
-
-// One grid's staged box as the encoder sees it.  With t the cell's float bits of
-// axis_cell (cell + kMagicBits) per axis, the byte address of the cell's first corner is
-// at + tz oz + ty oy + tx (node bytes), all modulo 2^32.
-struct __align__(16) FwdBox {
-  uint32_t at, oy, oz, pad;
-};
-// What staging needs: lo | nodes per axis as in block_box, and the pool offset in nodes.
-struct FwdStage {
-  uint32_t lo, n, at;
-};
-
-template <int K, int C>
-struct FwdLay {
-  static constexpr int M = K / C;
-  static constexpr int W1 = 0;                       // [64][K] bf16 swizzled
-  static constexpr int W2 = W1 + 64 * K * 2;         // [64][64] bf16
-  static constexpr int Y = W2 + 64 * 64 * 2;         // [T][K] bf16
-  static constexpr int X = Y + T * K * 2;            // [kFwdGroup] float4: x, y, z, brick bits
-  static constexpr int W3 = X + kFwdGroup * 16;      // [64] f32
-  static constexpr int G = W3 + 64 * 4;              // [M][12] f32: column pairs of the x and y rows, then the z row
-  static constexpr int BOX = G + M * 48;             // [M] FwdBox
-  static constexpr int STG = BOX + M * 16;           // [M] FwdStage
-  static constexpr int POOL = (STG + M * 12 + 15) / 16 * 16;   // staged nodes, C float32 each
-};
-
-// Node box of grid g over the block [lo, hi]: block_box with a margin that covers the
-// rounding of the per-sample map for any transform, so that every sample of the block
-// inside the grid has its cell in the box (no per-sample test is needed).
-// gp: the grid's map as load order keeps it, the column pairs of its x and y rows, then
-// its z row.
-__device__ __forceinline__ bool sample_box(const float (&lo)[3], const float (&hi)[3], const float* gp, int R,
-                                           uint32_t& blo, uint32_t& bn) {
-  const float h = 0.5f * (float)(R - 1), top = (float)(R - 1);
-  blo = 0;
-  bn = 0;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    auto g = [&](int k) { return d < 2 ? gp[2 * k + d] : gp[8 + k]; };
-    float umin = g(3), umax = umin, mag = fabsf(umin);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const float a = g(k), p = a * lo[k], q = a * hi[k];
-      umin += fminf(p, q);
-      umax += fmaxf(p, q);
-      mag += fmaxf(fabsf(p), fabsf(q));
-    }
-    // per sample and here: at most 5 roundings of sums of at most mag, each 2^-24 of them
-    const float pu = mag * 1e-6f, ps = fmaf(h, pu, 1e-3f);
-    if (umax + pu < -1.f || umin - pu > 1.f) return false;
-    const float a = fmaf(umin, h, h) - ps, b = fmaf(umax, h, h) + ps;
-    const float s0 = a >= 0.f ? fminf(a, top) : 0.f;     // (a NaN bound takes the whole axis)
-    const float s1 = b <= top ? fmaxf(b, 0.f) : top;
-    const int c0 = min((int)s0, R - 2), c1 = min((int)s1, R - 2);
-    blo |= (uint32_t)c0 << (8 * d);
-    bn |= (uint32_t)(c1 - c0 + 2) << (8 * d);
-  }
-  return true;
-}
-
-// Float order as unsigned integer order (for min/max reductions).
-__device__ __forceinline__ uint32_t ord(float v) {
-  const uint32_t b = __float_as_uint(v);
-  return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
-}
-__device__ __forceinline__ float unord(uint32_t o) {
-  return __uint_as_float(o ^ ((o & 0x80000000u) ? 0x80000000u : 0xffffffffu));
-}
-
-template <int K, int C, bool EVEN>
-__global__ void __launch_bounds__(NT, fwd_ctas(K))
-k_fwd_bf16(Model md, Bricks brp, FwdSource src, float* __restrict__ out, uint32_t pool_nodes) {
-  using L = FwdLay<K, C>;
-  constexpr int M = K / C;
-  constexpr int GPC = 8 / C;                 // grids per 16-byte feature chunk
-  constexpr int NCH = K / 8;                 // chunks of a feature row
-  constexpr int PP = K >= 64 ? 4 : 1;        // samples per thread
-  constexpr int NQ = 8 / (T / (32 * PP));    // warps sharing the same samples, each its own chunks
-  constexpr uint32_t kNB = 4 * C;            // bytes of a staged node
-  extern __shared__ __align__(128) unsigned char sm[];
-  __shared__ TileMap tm;
-  __shared__ Bricks br;
-  __shared__ uint32_t s_lo[3], s_hi[3], s_mask[2], s_np;
-  __shared__ uint32_t s_slow[kMaxGrids / 32];   // bit i: grid i's corners come from global memory
-  load_bricks(brp, br);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int g8 = lane >> 2, t4 = lane & 3;
-  const int R = md.R;
-  const int GS = src.group;
-  if (src.kind == kFwdPoints) {
-    if (tid == 0) build_tile_map(br, GS, tm);
-    __syncthreads();
-  }
-  const int total = src.kind == kFwdPoints ? tm.first[br.n] : src.groups;
-  const bool copied = src.sorted.use();
-  const float* xyz = copied ? src.sorted.xyz : src.xyz;
-  float4* xs = reinterpret_cast<float4*>(sm + L::X);
-  float* w3s = reinterpret_cast<float*>(sm + L::W3);
-  float* gs = reinterpret_cast<float*>(sm + L::G);
-  FwdBox* boxes = reinterpret_cast<FwdBox*>(sm + L::BOX);
-  FwdStage* stg = reinterpret_cast<FwdStage*>(sm + L::STG);
-  const uint32_t sW1 = su32(sm + L::W1), sW2 = su32(sm + L::W2), sY = su32(sm + L::Y);
-  const uint32_t spool = su32(sm + L::POOL);
-  const int64_t gsz = (int64_t)R * R * R * C;
-  const float hs = 0.5f * (float)(R - 1);
-  const float ct = hs - 0.5f + kMagic;   // an integer when R is even (axis_cell)
-
-  int cur = -1, hint = -1;
-  float span = 0.f, vmin = 0.f;
-  // runs of src.run consecutive groups, dealt round robin to the CTAs: neighbouring groups
-  // share a brick (and its weights), and a frame's empty corners are spread over the CTAs
-  for (int r0 = blockIdx.x * src.run; r0 < total; r0 += gridDim.x * src.run) {
-  const int r1 = min(total, r0 + src.run);
-  for (int grp = r0; grp < r1; ++grp) {
-    // ---- the group's samples: coordinates and brick (-1: no sample)
-    if (tid < 2) s_mask[tid] = 0u;
-    __syncthreads();   // also: the previous group is done with xs, the boxes and Y
-    int64_t base;      // first point (kFwdPoints) or first slot
-    int ns;            // slots of the group that can hold samples
-    FwdBlock blk;
-    if (src.kind == kFwdPoints) {
-      hint = brick_of_tile(tm, br.n, grp, hint);
-      base = br.off[hint] + (int64_t)(grp - tm.first[hint]) * GS;
-      ns = (int)min((int64_t)GS, br.off[hint + 1] - base);
-    } else if (src.kind == kFwdRender) {
-      base = (int64_t)grp * GS;
-      ns = GS;
-    } else {
-      blk = decode_block(src.dec, grp);
-      base = 0;
-      ns = blk.n[0] * blk.n[1] * blk.n[2];
-    }
-    {
-      Ray ray;
-      int last = -1;
-      uint32_t m0 = 0u, m1 = 0u;
-      for (int s = tid; s < GS; s += NT) {
-        float4 v = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
-        if (s < ns) {
-          int b;
-          if (src.kind == kFwdPoints) {
-            const float* q = xyz + 3 * (base + s);
-            v.x = q[0]; v.y = q[1]; v.z = q[2];
-            b = hint;
-          } else if (src.kind == kFwdRender) {
-            const RaySlot rs = ray_slot(src.rp, (int)base + s);
-            if (rs.ray != last) {   // slots NT apart share the ray when rg divides NT
-              last = rs.ray;
-              ray.hit = false;
-              if (rs.ray < src.npix) ray = make_ray(src.rp, pixel_of(src.rp, src.pix0 + rs.ray));
-            }
-            b = ray.hit && rs.j < src.rp.samples ? ray_sample(src.rp, ray, rs.j, v.x, v.y, v.z) : -1;
-          } else {
-            b = blk.brick;
-            decode_point(src, blk, s, v.x, v.y, v.z);
-          }
-          v.w = __int_as_float(b);
-          if (b >= 0) {
-            if (b < 32) m0 |= 1u << b; else m1 |= 1u << (b - 32);
-          }
-        }
-        xs[s] = v;
-      }
-      m0 = __reduce_or_sync(0xffffffffu, m0);
-      m1 = __reduce_or_sync(0xffffffffu, m1);
-      if (lane == 0) {
-        if (m0) atomicOr(&s_mask[0], m0);
-        if (m1) atomicOr(&s_mask[1], m1);
-      }
-    }
-    __syncthreads();
-    unsigned long long mask = (unsigned long long)s_mask[0] | ((unsigned long long)s_mask[1] << 32);
-    while (mask) {   // the bricks of the group (more than one only where rays cross a brick face)
-      const int b = __ffsll((long long)mask) - 1;
-      mask &= mask - 1;
-      if (tid < 3) { s_lo[tid] = 0xffffffffu; s_hi[tid] = 0u; }
-      if (tid == 3) s_np = 0u;
-      if (b != cur) {
-        cur = b;
-        const uint4* w1 = reinterpret_cast<const uint4*>(md.W1h + (int64_t)b * md.sW1);
-        for (int c = tid; c < 64 * K / 8; c += NT)
-          *reinterpret_cast<uint4*>(sm + L::W1 + swz<K>(c / (K / 8), (c % (K / 8)) * 8)) = w1[c];
-        const uint4* w2 = reinterpret_cast<const uint4*>(md.W2h + (int64_t)b * md.sW2);
-        for (int c = tid; c < 64 * 8; c += NT)
-          *reinterpret_cast<uint4*>(sm + L::W2 + swz<64>(c / 8, (c % 8) * 8)) = w2[c];
-        if (tid < 64) w3s[tid] = md.w3[(int64_t)b * md.sw3 + tid];
-        // each grid's map as the column pairs of its x and y rows, then its z row
-        const float* G = md.G + (int64_t)b * md.sG;
-        for (int c = tid; c < M * 12; c += NT) {
-          const int i = c / 12, j = c - 12 * i;
-          gs[c] = G[12 * i + (j < 8 ? (j >> 1) + 4 * (j & 1) : j)];
-        }
-        vmin = md.range[2 * b];
-        span = md.range[2 * b + 1] - vmin;
-      }
-      __syncthreads();
-      {  // bounding box of the brick's samples (non-finite ones are inside no grid)
-        uint32_t lo[3] = {0xffffffffu, 0xffffffffu, 0xffffffffu}, hi[3] = {0u, 0u, 0u};
-        int n = 0;
-        for (int s = tid; s < ns; s += NT) {
-          const float4 v = xs[s];
-          if (__float_as_int(v.w) == b && v.x - v.x == 0.f && v.y - v.y == 0.f && v.z - v.z == 0.f) {
-            ++n;
-            lo[0] = min(lo[0], ord(v.x)); hi[0] = max(hi[0], ord(v.x));
-            lo[1] = min(lo[1], ord(v.y)); hi[1] = max(hi[1], ord(v.y));
-            lo[2] = min(lo[2], ord(v.z)); hi[2] = max(hi[2], ord(v.z));
-          }
-        }
-        n = __reduce_add_sync(0xffffffffu, n);
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          lo[d] = __reduce_min_sync(0xffffffffu, lo[d]);
-          hi[d] = __reduce_max_sync(0xffffffffu, hi[d]);
-        }
-        if (lane == 0 && n) {
-          atomicAdd(&s_np, (uint32_t)n);
-#pragma unroll
-          for (int d = 0; d < 3; ++d) { atomicMin(&s_lo[d], lo[d]); atomicMax(&s_hi[d], hi[d]); }
-        }
-      }
-      __syncthreads();
-      if (warp == 0) {   // the grids' boxes, packed into the pool in grid order
-        const uint32_t np = s_np;
-        const float lo[3] = {unord(s_lo[0]), unord(s_lo[1]), unord(s_lo[2])};
-        const float hi[3] = {unord(s_hi[0]), unord(s_hi[1]), unord(s_hi[2])};
-        uint32_t used = 0u;
-        for (int i0 = 0; i0 < M; i0 += 32) {
-          const int i = i0 + lane;
-          uint32_t blo = 0u, bn = 0u, nodes = 0u;
-          bool any = false;
-          if (i < M && np) any = sample_box(lo, hi, gs + 12 * i, R, blo, bn);
-          const uint32_t nx = bn & 0xffu, ny = (bn >> 8) & 0xffu, nz = (bn >> 16) & 0xffu;
-          // staging a node costs about half of what it saves on one sample
-          if (any && nx * ny * nz <= np) nodes = nx * ny * nz;
-          uint32_t incl = nodes;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-          }
-          const uint32_t at = used + incl - nodes;
-          const bool fits = nodes && at + nodes <= pool_nodes;
-          if (i < M) {
-            FwdBox q;
-            q.oy = nx * kNB;
-            q.oz = nx * ny * kNB;
-            q.at = spool + at * kNB - ((blo >> 16 & 0xffu) + (uint32_t)kMagicBits) * q.oz -
-                   ((blo >> 8 & 0xffu) + (uint32_t)kMagicBits) * q.oy - ((blo & 0xffu) + (uint32_t)kMagicBits) * kNB;
-            q.pad = 0u;
-            boxes[i] = q;
-            stg[i] = FwdStage{blo, fits ? bn : 0u, at};
-          }
-          const uint32_t slow = __ballot_sync(0xffffffffu, any && !fits);
-          if (lane == 0) s_slow[i0 / 32] = slow;
-          used += __shfl_sync(0xffffffffu, incl, 31);
-        }
-      }
-      __syncthreads();
-      // ---- staging: a warp per grid, a lane per node
-      const __nv_bfloat16* Fb = md.F16 + (int64_t)b * md.sF;
-      for (int i = warp; i < M; i += NT / 32) {
-        const FwdStage q = stg[i];
-        if (!q.n) continue;
-        const uint32_t nx = q.n & 0xffu, ny = (q.n >> 8) & 0xffu, nxy = nx * ny, n = nxy * (q.n >> 16 & 0xffu);
-        const float ixy = 1.f / (float)nxy, ix = 1.f / (float)nx;
-        const EncNode<C>* Fg = reinterpret_cast<const EncNode<C>*>(Fb + i * gsz) +
-                               (((q.lo >> 16 & 0xffu) * R + (q.lo >> 8 & 0xffu)) * R + (q.lo & 0xffu));
-        EncSNode<C>* dst = reinterpret_cast<EncSNode<C>*>(sm + L::POOL) + q.at;
-#pragma unroll 2
-        for (uint32_t k = lane; k < n; k += 32) {   // n <= 512: the float quotients are exact
-          const uint32_t z = (uint32_t)(((float)k + 0.5f) * ixy), r = k - z * nxy;
-          const uint32_t y = (uint32_t)(((float)r + 0.5f) * ix), x = r - y * nx;
-          const EncNode<C> v = __ldg(Fg + ((z * R + y) * R + x));
-          if constexpr (C == 2) dst[k] = bf2_bits(v);
-          else dst[k] = __uint_as_float((uint32_t)v << 16);
-        }
-      }
-      __syncthreads();
-      for (int t0 = 0; t0 < ns; t0 += T) {
-        {  // ---- encode
-          const int pr = (warp / NQ) * 32 * PP + lane;   // this thread's rows: pr, pr + 32, ...
-          f2_t xx[PP], yy[PP], zz[PP];
-          bool valid[PP];
-#pragma unroll
-          for (int p = 0; p < PP; ++p) {
-            const float4 v = xs[t0 + pr + 32 * p];
-            xx[p] = f2_pack(v.x, v.x); yy[p] = f2_pack(v.y, v.y); zz[p] = f2_pack(v.z, v.z);
-            valid[p] = __float_as_int(v.w) == b;
-          }
-          // Eq. 1 and the cell of Eq. 2 of sample p in grid i
-          struct Place {
-            uint32_t tx, ty, tz;
-            float wx, wy, wz;
-            bool in;
-          };
-          auto place = [&](int i, Place (&c)[PP]) {
-            const ulonglong2 ab = *reinterpret_cast<const ulonglong2*>(gs + 12 * i);
-            const ulonglong2 cd = *reinterpret_cast<const ulonglong2*>(gs + 12 * i + 4);
-            const float4 gz = *reinterpret_cast<const float4*>(gs + 12 * i + 8);
-#pragma unroll
-            for (int p = 0; p < PP; ++p) {
-              const f2_t uxy = f2_fma(ab.x, xx[p], f2_fma(ab.y, yy[p], f2_fma(cd.x, zz[p], cd.y)));
-              const float uz = fmaf(gz.x, f2_lo(xx[p]), fmaf(gz.y, f2_lo(yy[p]), fmaf(gz.z, f2_lo(zz[p]), gz.w)));
-              c[p].in = valid[p] & (fabsf(f2_lo(uxy)) <= 1.f) & (fabsf(f2_hi(uxy)) <= 1.f) & (fabsf(uz) <= 1.f);
-              if constexpr (EVEN) {
-                int32_t tx, ty;
-                axis_cell2(uxy, f2_pack(hs, hs), f2_pack(ct, ct), f2_pack(kMagic, kMagic), tx, ty, c[p].wx, c[p].wy);
-                c[p].tx = (uint32_t)tx;
-                c[p].ty = (uint32_t)ty;
-                c[p].tz = (uint32_t)axis_cell(uz, hs, ct, c[p].wz);
-              } else {   // (s - 1/2) + kMagic: the cell floor(s) or, on a node, an even neighbour; at most R - 2
-                const float top = kMagic + (float)(R - 2);
-                auto axis = [&](float u, uint32_t& t, float& w) {
-                  const float sv = fmaf(u, hs, hs), cv = fminf(__fadd_rn(sv - 0.5f, kMagic), top);
-                  w = sv - (cv - kMagic);
-                  t = __float_as_uint(cv);
-                };
-                axis(f2_lo(uxy), c[p].tx, c[p].wx);
-                axis(f2_hi(uxy), c[p].ty, c[p].wy);
-                axis(uz, c[p].tz, c[p].wz);
-              }
-            }
-          };
-          // Eq. 2's blend of the eight corners (x fastest), as C bf16 in the low bits
-          auto blend = [&](const EncSNode<C> (&v)[8], const Place& c) -> uint32_t {
-            const float vx = 1.f - c.wx, vy = 1.f - c.wy, vz = 1.f - c.wz;
-            if constexpr (C == 2) {
-              const f2_t px = f2_pack(c.wx, c.wx), qx = f2_pack(vx, vx), py = f2_pack(c.wy, c.wy), qy = f2_pack(vy, vy);
-              const f2_t e0 = blend2(v[0], v[1], px, qx), e1 = blend2(v[2], v[3], px, qx);
-              const f2_t e2 = blend2(v[4], v[5], px, qx), e3 = blend2(v[6], v[7], px, qx);
-              const f2_t f = blend2(blend2(e0, e1, py, qy), blend2(e2, e3, py, qy), f2_pack(c.wz, c.wz), f2_pack(vz, vz));
-              return pack_bf16(f2_lo(f), f2_hi(f));
-            } else {
-              const float e0 = blend1(v[0], v[1], c.wx, vx), e1 = blend1(v[2], v[3], c.wx, vx);
-              const float e2 = blend1(v[4], v[5], c.wx, vx), e3 = blend1(v[6], v[7], c.wx, vx);
-              const float f = blend1(blend1(e0, e1, c.wy, vy), blend1(e2, e3, c.wy, vy), c.wz, vz);
-              return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(f));
-            }
-          };
-          // from a staged box (a sample outside the grid reads, and drops, nodes at the pool's
-          // start: the offsets to a cell's last corner are less than the box's size)
-          auto from_box = [&](const FwdBox& q, const Place& c) -> uint32_t {
-            const uint32_t a = q.at + c.tz * q.oz + c.ty * q.oy + c.tx * kNB, a0 = c.in ? a : spool;
-            const uint32_t a1 = a0 + q.oy, a2 = a0 + q.oz, a3 = a2 + q.oy;
-            const EncSNode<C> v[8] = {enc_node<C, 0>(a0), enc_node<C, kNB>(a0), enc_node<C, 0>(a1), enc_node<C, kNB>(a1),
-                                      enc_node<C, 0>(a2), enc_node<C, kNB>(a2), enc_node<C, 0>(a3), enc_node<C, kNB>(a3)};
-            const uint32_t f = blend(v, c);
-            return c.in ? f : 0u;
-          };
-          auto from_grid = [&](int i, const Place& c) -> uint32_t {
-            if (!c.in) return 0u;
-            constexpr uint32_t mb = (uint32_t)kMagicBits;
-            const EncNode<C>* F0 = reinterpret_cast<const EncNode<C>*>(Fb + i * gsz) +
-                                   (((c.tz - mb) * R + (c.ty - mb)) * R + (c.tx - mb));
-            const EncNode<C>* F2 = F0 + (uint32_t)(R * R);
-            const EncNode<C> n[8] = {__ldg(F0), __ldg(F0 + 1), __ldg(F0 + R), __ldg(F0 + R + 1),
-                                     __ldg(F2), __ldg(F2 + 1), __ldg(F2 + R), __ldg(F2 + R + 1)};
-            EncSNode<C> v[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              if constexpr (C == 2) v[k] = bf2_bits(n[k]);
-              else v[k] = __uint_as_float((uint32_t)n[k] << 16);
-            }
-            return blend(v, c);
-          };
-#pragma unroll 1
-          for (int ch = warp % NQ; ch < NCH; ch += NQ) {
-            uint32_t o[PP][4];
-            const uint32_t unstaged = (s_slow[ch * GPC / 32] >> (ch * GPC % 32)) & ((1u << GPC) - 1u);
-            if (unstaged == 0u) {   // straight-line code over the chunk's grids
-#pragma unroll
-              for (int j = 0; j < GPC; ++j) {
-                Place c[PP];
-                place(ch * GPC + j, c);
-                const FwdBox q = boxes[ch * GPC + j];
-#pragma unroll
-                for (int p = 0; p < PP; ++p) {
-                  const uint32_t f = from_box(q, c[p]);
-                  if constexpr (C == 2) o[p][j] = f;
-                  else o[p][j / 2] = j % 2 ? o[p][j / 2] | f << 16 : f;
-                }
-              }
-            } else {
-#pragma unroll
-              for (int j = 0; j < GPC; ++j) {
-                Place c[PP];
-                place(ch * GPC + j, c);
-                uint32_t f[PP];
-                if (unstaged >> j & 1u) {
-#pragma unroll
-                  for (int p = 0; p < PP; ++p) f[p] = from_grid(ch * GPC + j, c[p]);
-                } else {
-                  const FwdBox q = boxes[ch * GPC + j];
-#pragma unroll
-                  for (int p = 0; p < PP; ++p) f[p] = from_box(q, c[p]);
-                }
-#pragma unroll
-                for (int p = 0; p < PP; ++p) {
-                  if constexpr (C == 2) o[p][j] = f[p];
-                  else o[p][j / 2] = j % 2 ? o[p][j / 2] | f[p] << 16 : f[p];
-                }
-              }
-            }
-#pragma unroll
-            for (int p = 0; p < PP; ++p)
-              *reinterpret_cast<uint4*>(sm + L::Y + swz<K>(pr + 32 * p, 8 * ch)) =
-                  make_uint4(o[p][0], o[p][1], o[p][2], o[p][3]);
-          }
-        }
-        __syncthreads();
-        {  // ---- decoder
-          const int r0w = warp * 16;
-          float acc[8][4];
-#pragma unroll
-          for (int j = 0; j < 8; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-#pragma unroll
-          for (int ks = 0; ks < K / 16; ++ks) {
-            uint32_t a[4];
-            ldsm4(a, sY + swz<K>(r0w + (lane & 15), ks * 16 + (lane >> 4) * 8));
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              uint32_t bb[4];
-              ldsm4(bb, sW1 + swz<K>(q * 16 + (lane & 7) + ((lane >> 4) << 3), ks * 16 + ((lane >> 3) & 1) * 8));
-              mma(acc[2 * q], a, bb[0], bb[1]);
-              mma(acc[2 * q + 1], a, bb[2], bb[3]);
-            }
-          }
-          uint32_t h1a[4][4];
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            h1a[kk][0] = pack_bf16(fmaxf(acc[2 * kk][0], 0.f), fmaxf(acc[2 * kk][1], 0.f));
-            h1a[kk][1] = pack_bf16(fmaxf(acc[2 * kk][2], 0.f), fmaxf(acc[2 * kk][3], 0.f));
-            h1a[kk][2] = pack_bf16(fmaxf(acc[2 * kk + 1][0], 0.f), fmaxf(acc[2 * kk + 1][1], 0.f));
-            h1a[kk][3] = pack_bf16(fmaxf(acc[2 * kk + 1][2], 0.f), fmaxf(acc[2 * kk + 1][3], 0.f));
-          }
-#pragma unroll
-          for (int j = 0; j < 8; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              uint32_t bb[4];
-              ldsm4(bb, sW2 + swz<64>(q * 16 + (lane & 7) + ((lane >> 4) << 3), kk * 16 + ((lane >> 3) & 1) * 8));
-              mma(acc[2 * q], h1a[kk], bb[0], bb[1]);
-              mma(acc[2 * q + 1], h1a[kk], bb[2], bb[3]);
-            }
-          }
-          float mlo = 0.f, mhi = 0.f;
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              const float w = w3s[j * 8 + 2 * t4 + e];
-              mlo = fmaf(fmaxf(acc[j][e], 0.f), w, mlo);
-              mhi = fmaf(fmaxf(acc[j][2 + e], 0.f), w, mhi);
-            }
-          }
-          mlo += __shfl_xor_sync(0xffffffffu, mlo, 1);
-          mlo += __shfl_xor_sync(0xffffffffu, mlo, 2);
-          mhi += __shfl_xor_sync(0xffffffffu, mhi, 1);
-          mhi += __shfl_xor_sync(0xffffffffu, mhi, 2);
-          if (t4 < 2) {   // lane t4 = 0 writes row g8, lane 1 row g8 + 8
-            const int s = t0 + r0w + g8 + 8 * t4;
-            if (__float_as_int(xs[s].w) == b) {
-              const float f = fmaf(t4 ? mhi : mlo, span, vmin);
-              if (src.kind == kFwdDecode) out[decode_index(src, blk, s)] = f;
-              else out[copied ? (int64_t)src.sorted.index[base + s] : base + s] = f;
-            }
-          }
-        }
-        __syncthreads();
-      }
-    }
-  }
-  }
-}
-
-template <int K, int C, bool EVEN>
-cudaError_t launch_k(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
-  using Lay = FwdLay<K, C>;
-  auto kern = k_fwd_bf16<K, C, EVEN>;
-  // all of an SM's shared memory, halved (1 KB of each half is reserved), less the static part
-  int dev = 0, per_sm = 0;
-  cudaFuncAttributes fa;
-  cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess) return e;
-  if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
-  const int smem = (per_sm / fwd_ctas(K) - 1024 - (int)fa.sharedSizeBytes) / 128 * 128;
-  const int pool = (smem - Lay::POOL) / (4 * C);
-  if (pool < 8) return cudaErrorInvalidConfiguration;
-  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
-  int total = src.groups;
-  if (src.kind == kFwdPoints) {
-    total = 0;
-    for (int b = 0; b < br.n; ++b) total += (int)((br.off[b + 1] - br.off[b] + src.group - 1) / src.group);
-  }
-  if (total == 0) return cudaSuccess;
-  FwdSource s = src;
-  const int ctas = fwd_ctas(K) * L.num_sms;
-  s.run = std::max(1, std::min(4, total / (8 * ctas)));
-  kern<<<std::min((total + s.run - 1) / s.run, ctas), NT, smem, L.stream>>>(md, br, s, out, (uint32_t)pool);
-  return cudaGetLastError();
-}
-
-template <int K, int C>
-cudaError_t launch_c(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
-  return md.R % 2 ? launch_k<K, C, false>(L, md, br, src, out) : launch_k<K, C, true>(L, md, br, src, out);
-}
-template <int K>
-cudaError_t launch_kc(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
-  return md.C == 2 ? launch_c<K, 2>(L, md, br, src, out) : launch_c<K, 1>(L, md, br, src, out);
-}
-
-}  // namespace
-
-cudaError_t launch_forward_bf16(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
-  switch (md.K) {
-    case 16: return launch_kc<16>(L, md, br, src, out);
-    case 32: return launch_kc<32>(L, md, br, src, out);
-    case 64: return launch_kc<64>(L, md, br, src, out);
-    case 128: return launch_kc<128>(L, md, br, src, out);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-}  // namespace srn
+// The forward query of BF16 models (k_fwd.cuh).
+#define SRN_FWD_LAUNCH launch_forward_bf16
+namespace srn { namespace { constexpr bool kF32 = false; } }
+#include "k_fwd.cuh"

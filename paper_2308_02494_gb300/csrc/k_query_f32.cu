@@ -1,4 +1,4 @@
-// FP32 fused point-query kernel: the same computation as the BF16 kernel (encoder
+// FP32 fused training kernel: the same computation as the BF16 kernels (encoder
 // Eq. 1-3, decoder Sec. 4.1.2, L_rec backward, Eq. 7 density) entirely in float32,
 // with the decoder on the SIMT pipes.  It is the full-precision reference path:
 // 64-point tiles, 256 threads, every matrix product a register-blocked loop over
@@ -72,12 +72,10 @@ struct Lay {
   static constexpr int FLOATS = RG + kMaxGrids * 12;
 };
 
-template <int K, int MODE>
+template <int K, bool DENS>
 __global__ void __launch_bounds__(NT, 1)
 k_query_f32(Model md, Grads gr, Bricks brp, TrainWs ws, const float* __restrict__ xyz,
-            const float* __restrict__ target, float* __restrict__ out) {
-  constexpr bool TRAIN = MODE >= kTrain;
-  constexpr bool DENS = MODE == kTrainDensity;
+            const float* __restrict__ target) {
   constexpr int NC1 = K / 16;  // feature columns per thread
   using L = Lay<K>;
   extern __shared__ __align__(128) float smf[];
@@ -100,7 +98,7 @@ k_query_f32(Model md, Grads gr, Bricks brp, TrainWs ws, const float* __restrict_
 
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
   const int M = md.M, C = md.C, R = md.R;
-  if (TRAIN && ws.rec_dg)
+  if (ws.rec_dg)
     for (int c = tid; c < M * 12; c += NT) rgs[c] = 0.f;
   if (tid == 0) build_tile_map(br, T, tm);
   __syncthreads();
@@ -154,7 +152,7 @@ k_query_f32(Model md, Grads gr, Bricks brp, TrainWs ws, const float* __restrict_
   for (int tile = tb; tile < te; ++tile) {
     const int b = brick_of_tile(tm, br.n, tile, cur);
     if (b != cur) {
-      if (TRAIN && cur >= 0) flush(cur);
+      if (cur >= 0) flush(cur);
       __syncthreads();
       cur = b;
       const float* W1 = md.W1f + (int64_t)b * md.sW1;
@@ -177,7 +175,7 @@ k_query_f32(Model md, Grads gr, Bricks brp, TrainWs ws, const float* __restrict_
       if (tid < np) {
         const float* q = xyz + 3 * (p0 + tid);
         v.x = q[0]; v.y = q[1]; v.z = q[2];
-        if (TRAIN) v.w = target[p0 + tid];
+        v.w = target[p0 + tid];
       }
       xs[tid] = v;
     }
@@ -260,15 +258,7 @@ k_query_f32(Model md, Grads gr, Bricks brp, TrainWs ws, const float* __restrict_
       s += __shfl_xor_sync(0xffffffffu, s, 8);
       m[r] = s;
     }
-    if constexpr (!TRAIN) {
-      if (tx == 0) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-          if (4 * ty + r < np) out[p0 + 4 * ty + r] = fmaf(m[r], span, vmin);
-      }
-      __syncthreads();
-      continue;
-    } else {
+    {
       float dm[4];
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
@@ -435,51 +425,40 @@ k_query_f32(Model md, Grads gr, Bricks brp, TrainWs ws, const float* __restrict_
       __syncthreads();
     }
   }
-  if constexpr (TRAIN) {
-    if (cur >= 0) flush(cur);
-  }
+  if (cur >= 0) flush(cur);
 }
 
-template <int K, int MODE>
-cudaError_t launch_k(const Launch& L, const Model& md, const Grads& gr, const Bricks& br,
-                     const TrainWs& ws, const float* xyz, const float* target, float* out) {
+template <int K, bool DENS>
+cudaError_t launch_k(const Launch& L, const Model& md, const Grads& gr, const Bricks& br, const TrainWs& ws,
+                     const float* xyz, const float* target) {
   const int smem = Lay<K>::FLOATS * 4;
-  auto kern = k_query_f32<K, MODE>;
+  auto kern = k_query_f32<K, DENS>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  int grid = L.num_sms;
-  if (!br.dev) {
-    int total = 0;
-    for (int b = 0; b < br.n; ++b) total += (int)((br.off[b + 1] - br.off[b] + T - 1) / T);
-    if (total == 0) return cudaSuccess;
-    grid = total < L.num_sms ? total : L.num_sms;
-  }
-  kern<<<grid, NT, smem, L.stream>>>(md, gr, br, ws, xyz, target, out);
+  int total = 0;
+  for (int b = 0; b < br.n; ++b) total += (int)((br.off[b + 1] - br.off[b] + T - 1) / T);
+  if (total == 0) return cudaSuccess;
+  kern<<<total < L.num_sms ? total : L.num_sms, NT, smem, L.stream>>>(md, gr, br, ws, xyz, target);
   return cudaGetLastError();
 }
 
-template <int MODE>
-cudaError_t launch_mode(const Launch& L, const Model& md, const Grads& gr, const Bricks& br,
-                        const TrainWs& ws, const float* xyz, const float* target, float* out) {
+template <bool DENS>
+cudaError_t launch_mode(const Launch& L, const Model& md, const Grads& gr, const Bricks& br, const TrainWs& ws,
+                        const float* xyz, const float* target) {
   switch (md.K) {
-    case 16: return launch_k<16, MODE>(L, md, gr, br, ws, xyz, target, out);
-    case 32: return launch_k<32, MODE>(L, md, gr, br, ws, xyz, target, out);
-    case 64: return launch_k<64, MODE>(L, md, gr, br, ws, xyz, target, out);
-    case 128: return launch_k<128, MODE>(L, md, gr, br, ws, xyz, target, out);
+    case 16: return launch_k<16, DENS>(L, md, gr, br, ws, xyz, target);
+    case 32: return launch_k<32, DENS>(L, md, gr, br, ws, xyz, target);
+    case 64: return launch_k<64, DENS>(L, md, gr, br, ws, xyz, target);
+    case 128: return launch_k<128, DENS>(L, md, gr, br, ws, xyz, target);
     default: return cudaErrorInvalidValue;
   }
 }
 
 }  // namespace
 
-cudaError_t launch_query_fp32(const Launch& L, QueryMode mode, const Model& md, const Grads& gr,
-                              const Bricks& br, const TrainWs& ws, const float* xyz,
-                              const float* target, float* out) {
-  switch (mode) {
-    case kForward: return launch_mode<kForward>(L, md, gr, br, ws, xyz, target, out);
-    case kTrain: return launch_mode<kTrain>(L, md, gr, br, ws, xyz, target, out);
-    default: return launch_mode<kTrainDensity>(L, md, gr, br, ws, xyz, target, out);
-  }
+cudaError_t launch_train_fp32(const Launch& L, bool dens, const Model& md, const Grads& gr, const Bricks& br,
+                              const TrainWs& ws, const float* xyz, const float* target) {
+  return dens ? launch_mode<true>(L, md, gr, br, ws, xyz, target) : launch_mode<false>(L, md, gr, br, ws, xyz, target);
 }
 
 }  // namespace srn

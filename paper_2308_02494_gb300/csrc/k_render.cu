@@ -1,12 +1,8 @@
 // Headless neural volume renderer (Sec. 6) over a domain decomposition (Sec. 5.3).
 //
-// Per batch of rays, BF16: the forward query forms its samples itself, bundle by bundle
-// (render.h), and leaves their values in slot order.  Float32: (1) every (ray, sample)
-// computes its position, its brick through the spatial hash and its brick-local
-// coordinate, and takes a rank in its brick's bucket; (2) bucket offsets; (3) samples are
-// scattered into brick order; (4) the fused forward query runs over the buckets
-// (device-side offsets).  Then each ray reads its values in sample order and is
-// composited front to back.  Sampling and opacity: midpoints t_j = t0 + (j + 1/2) dt of the ray's
+// Per batch of rays the forward query forms its samples itself, bundle by bundle (render.h),
+// and leaves their values in slot order; then each ray reads its values in sample order and
+// is composited front to back.  Sampling and opacity: midpoints t_j = t0 + (j + 1/2) dt of the ray's
 // segment inside [-1,1]^3, alpha = 1 - exp(-a dt / (2/512)), the 256-entry RGBA
 // transfer function read with linear interpolation.
 #include <algorithm>
@@ -27,102 +23,14 @@ __device__ __forceinline__ int order_of(const RenderParams& rp, int x, int y) {
   return level_pixels(rp, l + 1) + (b >> 1) * (half + wa) + ((b & 1) ? half + a : a >> 1);
 }
 
-// Samples of a block take their rank in their brick's bucket in three levels: lanes of
-// a warp with the same brick (match), one shared-memory count per warp group, one global
-// reservation per brick per block.  A block's samples stay together in each bucket.
-__global__ void __launch_bounds__(256) k_render_gen(RenderParams rp, int pix0, int npix, float* __restrict__ loc,
-                                                    uint32_t* __restrict__ rank, uint32_t* __restrict__ bid,
-                                                    uint32_t* __restrict__ cnt) {
-  __shared__ uint32_t s_cnt[SRN_MAX_BRICKS], s_base[SRN_MAX_BRICKS];
-  const int nb = rp.grid[0] * rp.grid[1] * rp.grid[2];
-  const int total = (int)render_slots(rp, npix);
-  const int lane = threadIdx.x & 31;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < total; base += (int64_t)gridDim.x * blockDim.x) {
-    for (int k = threadIdx.x; k < nb; k += blockDim.x) s_cnt[k] = 0;
-    __syncthreads();
-    const int64_t idx = base + threadIdx.x;
-    uint32_t b = 0xffffffffu;
-    if (idx < total) {
-      const RaySlot rs = ray_slot(rp, (int)idx);
-      if (rs.ray < npix && rs.j < rp.samples) {
-        const Ray r = make_ray(rp, pixel_of(rp, pix0 + rs.ray));
-        if (r.hit) b = (uint32_t)ray_sample(rp, r, rs.j, loc[3 * idx], loc[3 * idx + 1], loc[3 * idx + 2]);
-      }
-    }
-    const unsigned grp = __match_any_sync(0xffffffffu, b);
-    const int leader = __ffs(grp) - 1;
-    const uint32_t before = __popc(grp & ((1u << lane) - 1u));
-    uint32_t wbase = 0;
-    if (b != 0xffffffffu && lane == leader) wbase = atomicAdd(s_cnt + b, (uint32_t)__popc(grp));
-    wbase = __shfl_sync(0xffffffffu, wbase, leader);
-    __syncthreads();
-    for (int k = threadIdx.x; k < nb; k += blockDim.x) s_base[k] = s_cnt[k] ? atomicAdd(cnt + k, s_cnt[k]) : 0u;
-    __syncthreads();
-    if (idx < total) {
-      bid[idx] = b;
-      if (b != 0xffffffffu) rank[idx] = s_base[b] + wbase + before;
-    }
-    __syncthreads();
-  }
-}
-
-__global__ void k_render_offsets(int nb, const uint32_t* __restrict__ cnt, int64_t* __restrict__ off) {
-  if (threadIdx.x == 0) {
-    int64_t a = 0;
-    for (int b = 0; b < nb; ++b) { off[b] = a; a += cnt[b]; }
-    off[nb] = a;
-  }
-}
-
-__global__ void k_render_scatter(int64_t total, const float* __restrict__ loc, const uint32_t* __restrict__ rank,
-                                 const uint32_t* __restrict__ bid, const int64_t* __restrict__ off,
-                                 float* __restrict__ xyz, uint32_t* __restrict__ pos) {
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t b = bid[idx];
-    if (b == 0xffffffffu) continue;
-    const int64_t dst = off[b] + rank[idx];
-    xyz[3 * dst] = loc[3 * idx];
-    xyz[3 * dst + 1] = loc[3 * idx + 1];
-    xyz[3 * dst + 2] = loc[3 * idx + 2];
-    pos[idx] = (uint32_t)dst;
-  }
-}
-
-// Decode: brick-local coordinates of a voxel block in scanline order.
-__global__ void k_decode_gen(DecodeChunk c, float* __restrict__ xyz) {
-  const int64_t n = (int64_t)c.nx * c.ny * c.nz;
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += (int64_t)gridDim.x * blockDim.x) {
-    const int x = (int)(idx % c.nx);
-    const int64_t r = idx / c.nx;
-    const int y = (int)(r % c.ny), z = (int)(r / c.ny);
-    const int v[3] = {c.x0 + x, c.y0 + y, c.z0 + z};
-#pragma unroll
-    for (int a = 0; a < 3; ++a)   // voxel index = (p + 1)/2 (vox - 1): global -> brick-local [-1, 1]
-      xyz[3 * idx + a] = ((float)v[a] - (float)c.lo[a]) / (float)(c.hi[a] - c.lo[a]) * 2.f - 1.f;
-  }
-}
-
-// Decode: the block's values (scanline order) into the volume [vox][vox][vox].
-__global__ void k_decode_store(DecodeChunk c, const float* __restrict__ val, float* __restrict__ out) {
-  const int64_t n = (int64_t)c.nx * c.ny * c.nz;
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += (int64_t)gridDim.x * blockDim.x) {
-    const int x = (int)(idx % c.nx);
-    const int64_t r = idx / c.nx;
-    const int y = (int)(r % c.ny), z = (int)(r / c.ny);
-    out[((int64_t)(c.z0 + z) * c.vox + (c.y0 + y)) * c.vox + c.x0 + x] = val[idx];
-  }
-}
-
 // Front-to-back compositing of 32 rays per block of 256 threads: thread (ray, segment)
 // composites one eighth of the ray's samples, then the segments are joined in order (the
 // compositing operator is associative).  One thread per ray left a batch of 8192 rays
 // with 54 threads per SM, each a chain of 512 dependent reads.
 constexpr int kSegs = 8;
-template <bool POS>
 __global__ void __launch_bounds__(32 * kSegs)
-k_render_composite(RenderParams rp, int pix0, int npix, const uint32_t* __restrict__ pos,
-                   const float* __restrict__ val, const float* __restrict__ lut, float* __restrict__ rgba) {
+k_render_composite(RenderParams rp, int pix0, int npix, const float* __restrict__ val,
+                   const float* __restrict__ lut, float* __restrict__ rgba) {
   __shared__ float4 part[kSegs][32];
   const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
   const int ray = blockIdx.x * 32 + lane;
@@ -137,8 +45,7 @@ k_render_composite(RenderParams rp, int pix0, int npix, const uint32_t* __restri
       const int s0 = render_slot(rp, ray, 0);
 #pragma unroll 8
       for (int j = j0; j < j1; ++j) {
-        const int slot = s0 + j * rp.rg;
-        const float f = val[POS ? pos[slot] : (uint32_t)slot];
+        const float f = val[s0 + j * rp.rg];
         const float s = fminf(fmaxf((f - rp.vmin) * inv_span, 0.f), 1.f) * 255.f;
         const int i0 = min((int)s, 254);
         const float fr = s - (float)i0;
@@ -196,46 +103,23 @@ __global__ void k_render_preview(RenderParams rp, int done, int level, const flo
   out[pix] = v;
 }
 
-int blocks_for(int64_t n, int threads, int num_sms) {
-  int64_t b = (n + threads - 1) / threads;
-  const int64_t cap = (int64_t)num_sms * 8;
-  if (b > cap) b = cap;
-  return b < 1 ? 1 : (int)b;
-}
-
 }  // namespace
 
-cudaError_t launch_render_batch(const Launch& L, const RenderParams& rp, const RenderWs& w, int pix0,
-                                int npix, const Model& md, const float* lut, float* rgba) {
-  const int64_t total = render_slots(rp, npix);
-  const int nb = rp.grid[0] * rp.grid[1] * rp.grid[2];
-  cudaError_t e;
+cudaError_t launch_render_batch(const Launch& L, const RenderParams& rp, float* val, int pix0, int npix,
+                                const Model& md, const float* lut, float* rgba) {
   Bricks br{};
-  br.n = nb;
-  if (md.F16) {
-    FwdSource src{};
-    src.kind = kFwdRender;
-    src.group = kFwdGroup;
-    src.groups = (int)((total + kFwdGroup - 1) / kFwdGroup);
-    src.pix0 = pix0;
-    src.npix = npix;
-    src.rp = rp;
-    if ((e = launch_forward_bf16(L, md, br, src, w.val)) != cudaSuccess) return e;
-    k_render_composite<false><<<(npix + 31) / 32, 32 * kSegs, 0, L.stream>>>(rp, pix0, npix, nullptr, w.val, lut, rgba);
-    return cudaGetLastError();
-  }
-  if ((e = cudaMemsetAsync(w.cnt, 0, sizeof(uint32_t) * nb, L.stream)) != cudaSuccess) return e;
-  k_render_gen<<<blocks_for(total, 256, L.num_sms), 256, 0, L.stream>>>(rp, pix0, npix, w.loc, w.rank, w.bid, w.cnt);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_render_offsets<<<1, 32, 0, L.stream>>>(nb, w.cnt, w.off);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_render_scatter<<<blocks_for(total, 256, L.num_sms), 256, 0, L.stream>>>(total, w.loc, w.rank, w.bid, w.off, w.xyz, w.pos);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  br.dev = w.off;
-  Grads gr{};
-  TrainWs tw{};
-  if ((e = launch_query_fp32(L, kForward, md, gr, br, tw, w.xyz, nullptr, w.val)) != cudaSuccess) return e;
-  k_render_composite<true><<<(npix + 31) / 32, 32 * kSegs, 0, L.stream>>>(rp, pix0, npix, w.pos, w.val, lut, rgba);
+  br.n = rp.grid[0] * rp.grid[1] * rp.grid[2];
+  FwdSource src{};
+  src.kind = kFwdRender;
+  src.boxes = 1;
+  src.group = fwd_group(!md.F16);
+  src.groups = (int)((render_slots(rp, npix) + src.group - 1) / src.group);
+  src.pix0 = pix0;
+  src.npix = npix;
+  src.rp = rp;
+  const cudaError_t e = launch_forward(L, md, br, src, val);
+  if (e != cudaSuccess) return e;
+  k_render_composite<<<(npix + 31) / 32, 32 * kSegs, 0, L.stream>>>(rp, pix0, npix, val, lut, rgba);
   return cudaGetLastError();
 }
 
@@ -247,9 +131,10 @@ cudaError_t launch_render_preview(const Launch& L, const RenderParams& rp, int d
   return cudaGetLastError();
 }
 
-cudaError_t launch_decode_bf16(const Launch& L, const RenderParams& rp, const Model& md, float* out) {
+cudaError_t launch_decode(const Launch& L, const RenderParams& rp, const Model& md, float* out) {
   FwdSource src{};
   src.kind = kFwdDecode;
+  src.boxes = 1;
   src.rp = rp;
   src.dec.vox = rp.vox;
   int n[3], nb = 1;
@@ -264,15 +149,16 @@ cudaError_t launch_decode_bf16(const Launch& L, const RenderParams& rp, const Mo
     if (n[a] == 0) return cudaSuccess;
   }
   // Blocks of at most `cap` voxels: as large as they go while there are a few for every CTA,
-  // and of the shape with the fewest 128-sample tiles over the bricks, compact ones first.
-  int cap = kFwdGroup;
-  while (cap > 128 && voxels / cap < 8 * (int64_t)L.num_sms) cap /= 2;
+  // and of the shape with the fewest tiles of samples over the bricks, compact ones first.
+  const int tile = md.F16 ? 128 : 64;
+  int cap = fwd_group(!md.F16);
+  while (cap > tile && voxels / cap < 8 * (int64_t)L.num_sms) cap /= 2;
   double best = 0.0;
   for (int x = 1; x <= std::min(16, n[0]); ++x)
     for (int y = 1; y <= std::min(16, n[1]); ++y)
       for (int z = 1; z <= std::min(16, n[2]) && x * y * z <= cap; ++z) {
         const int64_t blocks = (int64_t)((n[0] + x - 1) / x) * ((n[1] + y - 1) / y) * ((n[2] + z - 1) / z);
-        const double cost = (double)blocks * ((x * y * z + 127) / 128 + 0.25) * (1.0 + 0.01 * (x + y + z));
+        const double cost = (double)blocks * ((x * y * z + tile - 1) / tile + 0.25) * (1.0 + 0.01 * (x + y + z));
         if (best == 0.0 || cost < best) {
           best = cost;
           src.dec.blk[0] = x; src.dec.blk[1] = y; src.dec.blk[2] = z;
@@ -284,29 +170,11 @@ cudaError_t launch_decode_bf16(const Launch& L, const RenderParams& rp, const Mo
     groups *= src.dec.nblk[a];
   }
   if (groups > INT32_MAX) return cudaErrorInvalidValue;
-  src.group = (src.dec.blk[0] * src.dec.blk[1] * src.dec.blk[2] + 127) / 128 * 128;
+  src.group = (src.dec.blk[0] * src.dec.blk[1] * src.dec.blk[2] + tile - 1) / tile * tile;
   src.groups = (int)groups;
   Bricks br{};
   br.n = nb;
-  return launch_forward_bf16(L, md, br, src, out);
-}
-
-cudaError_t launch_decode_chunk(const Launch& L, const DecodeChunk& c, const RenderWs& w, const Model& md,
-                                float* out) {
-  const int64_t n = (int64_t)c.nx * c.ny * c.nz;
-  if (n == 0) return cudaSuccess;
-  k_decode_gen<<<blocks_for(n, 256, L.num_sms), 256, 0, L.stream>>>(c, w.xyz);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  Bricks br{};
-  br.n = c.n_bricks;
-  br.dev = nullptr;
-  for (int b = 0; b <= c.n_bricks; ++b) br.off[b] = b <= c.brick ? 0 : n;
-  Grads gr{};
-  TrainWs tw{};
-  if ((e = launch_query_fp32(L, kForward, md, gr, br, tw, w.xyz, nullptr, w.val)) != cudaSuccess) return e;
-  k_decode_store<<<blocks_for(n, 256, L.num_sms), 256, 0, L.stream>>>(c, w.val, out);
-  return cudaGetLastError();
+  return launch_forward(L, md, br, src, out);
 }
 
 }  // namespace srn

@@ -25,6 +25,7 @@
 //          Morton-sorted) add their corners directly.
 #include "enc_ops.cuh"
 #include "kernels.h"
+#include "sort.cuh"
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -477,123 +478,6 @@ template <int C>
 __device__ __forceinline__ uint32_t dy_bits(const __nv_bfloat16* dY, int64_t p, int M, int g) {
   if constexpr (C == 2) return __ldg(reinterpret_cast<const unsigned int*>(dY) + p * M + g);
   else return (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(dY) + p * M + g);
-}
-
-// One CTA per brick.  The brick's largest tile level lmax is the largest L <= lcap whose
-// block, mapped through any of the brick's grids, has a node box of at most capn nodes:
-// per grid axis, the image's extent in cells plus the box margin, one partial cell at
-// each end and the node past the last cell bound tile_box's count (0 when even one unit
-// is too large; such grids add their corners directly).  Units without a recorded start
-// take the next recorded one (a suffix minimum; for a sorted batch this is exact, for any
-// batch the starts become non-decreasing from 0 to n, so the tiles below always partition
-// the brick's points).  Every unit then belongs to the largest aligned range of 2^L units
-// (L <= lmax) holding at most tp (<= ST) points; each such range becomes ceil(points / tp)
-// tiles of consecutive points.
-__global__ void __launch_bounds__(1024) k_tile_list(Bricks brp, TrainWs ws, Model md, int capn, int lcap,
-                                                    int tp) {
-  constexpr int UPT = kUnits / 1024;
-  __shared__ Bricks br;
-  __shared__ int32_t st[kUnits + 1];
-  __shared__ int32_t wred[32];
-  __shared__ int32_t gbase;
-  __shared__ int32_t s_lv;
-  if (threadIdx.x == 0) s_lv = lcap;
-  load_bricks(brp, br);
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid < md.M) {
-    const float* g = md.G + (int64_t)b * md.sG + 12 * tid;
-    const float hs = 0.5f * (float)(md.R - 1) * (2.f / (float)(1 << kUnitBits));   // cells per unit
-    int lv = 0;
-    for (int L = lcap; L > 0; --L) {
-      const float ext[3] = {(float)(1 << ((L + 2) / 3)), (float)(1 << ((L + 1) / 3)), (float)(1 << (L / 3))};
-      int nodes = 1;
-      for (int d = 0; d < 3; ++d) {
-        const float e = (fabsf(g[4 * d]) * ext[0] + fabsf(g[4 * d + 1]) * ext[1] + fabsf(g[4 * d + 2]) * ext[2]) * hs;
-        nodes *= min((int)ceilf(e + 0.01f) + 2, md.R);
-      }
-      if (nodes <= capn) { lv = L; break; }
-    }
-    atomicMin(&s_lv, lv);
-  }
-  __syncthreads();
-  const int lmax = s_lv;
-  const int64_t o = br.off[b];
-  const int32_t n = (int32_t)(br.off[b + 1] - o);
-  const int32_t* us = ws.ustart + (int64_t)b * (kUnits + 1);
-  const uint32_t* bins = ws.bin_start ? ws.bin_start : ws.sorted.use() ? ws.sorted.hist : nullptr;
-  int32_t loc[UPT];
-  {
-    int32_t m = INT_MAX;
-#pragma unroll
-    for (int k = UPT - 1; k >= 0; --k) {
-      // a batch from the sampler or a sorted copy: unit u starts where its first bin starts
-      const int32_t v = bins ? (int32_t)bins[(int64_t)b * kSortBins + ((tid * UPT + k) << 3)] : us[tid * UPT + k];
-      if (v >= 0) m = min(m, v);
-      loc[k] = m;
-    }
-    int32_t incl = loc[0];   // suffix minimum over lanes >= lane
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const int32_t y = __shfl_down_sync(0xffffffffu, incl, d);
-      if (lane + d < 32) incl = min(incl, y);
-    }
-    if (lane == 0) wred[warp] = incl;
-    __syncthreads();
-    int32_t after = n;
-    for (int q = warp + 1; q < 32; ++q) after = min(after, wred[q]);
-    const int32_t next = __shfl_down_sync(0xffffffffu, incl, 1);
-    const int32_t excl = lane < 31 ? min(next, after) : after;
-#pragma unroll
-    for (int k = 0; k < UPT; ++k) st[tid * UPT + k] = min(loc[k], excl);
-    // the first point always opens a tile: in a batch that is not sorted, later points
-    // of its unit may have overwritten its recorded start
-    if (tid == 0) { st[0] = 0; st[kUnits] = n; }
-  }
-  __syncthreads();
-  int nt[UPT], lv[UPT];
-  int tot = 0;
-#pragma unroll
-  for (int k = 0; k < UPT; ++k) {
-    const int u = tid * UPT + k;
-    int L = 0;
-    for (int l = lmax; l > 0; --l) {
-      const int a = u & ~((1 << l) - 1);
-      if (st[a + (1 << l)] - st[a] <= tp) { L = l; break; }
-    }
-    lv[k] = L;
-    nt[k] = 0;
-    if ((u & ((1 << L) - 1)) == 0) nt[k] = (st[u + (1 << L)] - st[u] + tp - 1) / tp;
-    tot += nt[k];
-  }
-  int incl = tot;   // block-wide exclusive scan of the tile counts
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, incl, d);
-    if (lane >= d) incl += y;
-  }
-  __syncthreads();
-  if (lane == 31) wred[warp] = incl;
-  __syncthreads();
-  int base = incl - tot, all = 0;
-  for (int q = 0; q < 32; ++q) {
-    if (q < warp) base += wred[q];
-    all += wred[q];
-  }
-  if (tid == 0) gbase = atomicAdd(ws.tile_ctr, all);
-  __syncthreads();
-  int idx = gbase + base;
-#pragma unroll
-  for (int k = 0; k < UPT; ++k) {
-    const int u = tid * UPT + k;
-    const int c = nt[k] ? st[u + (1 << lv[k])] - st[u] : 0;
-    for (int t = 0; t < nt[k]; ++t, ++idx) {
-      ScatTile T;
-      T.start = o + st[u] + (int64_t)t * c / nt[k];
-      T.count = (int32_t)((int64_t)(t + 1) * c / nt[k] - (int64_t)t * c / nt[k]);
-      T.code = (uint32_t)b << 20 | (uint32_t)lv[k] << 16 | (uint32_t)u;
-      ws.tiles[idx] = T;
-    }
-  }
 }
 
 // Node box of the tile's block (units [u0, u0 + 2^L)) in grid g, padded by a small
@@ -1095,18 +979,13 @@ cudaError_t launch_train_k(const Launch& L, bool dens, const Model& md, const Gr
   if (tiles == 0) return cudaSuccess;
   cudaError_t e;
   {  // scatter tiles: aligned Morton blocks of each brick's points
-    int64_t nmax = 0;
-    for (int b = 0; b < br.n; ++b) nmax = std::max<int64_t>(nmax, br.off[b + 1] - br.off[b]);
-    if (nmax > INT32_MAX) return cudaErrorInvalidValue;
-    // unit starts (the sampler's histogram gives those of its batch), and a sorted copy if
-    // the batch is out of order
-    if (!ws.bin_start && (e = launch_sort(L, br, xyz, target, ws.sorted)) != cudaSuccess) return e;
+    for (int b = 0; b < br.n; ++b)
+      if (br.off[b + 1] - br.off[b] > INT32_MAX) return cudaErrorInvalidValue;
     const int cap = std::min(scat_capn(md.M, md.C), enc_capn(md.M, md.C));   // both kernels' boxes fit
     if (cap < 8) return cudaErrorInvalidConfiguration;
     if (tn.tile_points < kMinTilePoints || tn.tile_points > ST || tn.tile_level < 0 || tn.tile_level > kMaxTileLevel)
       return cudaErrorInvalidValue;
-    k_tile_list<<<br.n, 1024, 0, L.stream>>>(br, ws, md, cap, tn.tile_level, tn.tile_points);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_tiles(L, md, br, ws, xyz, target, cap, tn.tile_level, tn.tile_points)) != cudaSuccess) return e;
   }
   {
     const int capn = enc_capn(md.M, md.C);

@@ -13,9 +13,8 @@ struct Launch {
   int num_sms;
 };
 
-// BF16 path: fused forward query, and the three-kernel training pass (encoder,
-// decoder forward/backward, scatter), batched over bricks.
-// (launch_forward_bf16 is declared in render.h with the sample sources it takes.)
+// The forward queries are in render.h.  BF16 training pass: three kernels (encoder, decoder
+// forward/backward, scatter), batched over bricks.
 // Optional pair of CUDA events recorded around one kernel of the BF16 training pass
 // (which: 0 encoder, 1 decoder, 2 scatter); the measurement hook passes it.
 struct KernelMark {
@@ -51,10 +50,9 @@ cudaError_t launch_train_bf16(const Launch& L, bool dens, const Model& md, const
 // The decoder kernel of the BF16 training pass on the tcgen05 tensor cores (K = 128).
 cudaError_t launch_mlp_tc(const Launch& L, const Model& md, const Grads& gr, const Bricks& br, const TrainWs& ws,
                           const float* target);
-// FP32 path: one fused kernel per mode (encoder + SIMT decoder + per-corner scatter).
-cudaError_t launch_query_fp32(const Launch& L, QueryMode mode, const Model& md, const Grads& gr,
-                              const Bricks& br, const TrainWs& ws, const float* xyz,
-                              const float* target, float* out);
+// FP32 training pass: one fused kernel (encoder + SIMT decoder + per-corner scatter).
+cudaError_t launch_train_fp32(const Launch& L, bool dens, const Model& md, const Grads& gr, const Bricks& br,
+                              const TrainWs& ws, const float* xyz, const float* target);
 
 // Density loss (Eq. 7-9) second and third passes, and the per-brick finalisation.
 cudaError_t launch_density(const Launch& L, const Model& md, const Bricks& br, const TrainWs& ws,
@@ -120,11 +118,15 @@ cudaError_t launch_shadow(const Launch& L, const float* p, uint16_t* shadow, int
 cudaError_t launch_sample(const Launch& L, const Bricks& br, unsigned long long seed,
                           unsigned long long step, const unsigned long long* step_dev,
                           float* xyz, uint32_t* rank, uint32_t* hist);
-// The order of a batch in memory and, when more than s.limit of its points are out of it,
-// its Morton-sorted copy: the points with their targets and, first, the batch's unit starts
-// (training: s.target and s.ustart set) or with their places (queries: s.index set).
-cudaError_t launch_sort(const Launch& L, const Bricks& br, const float* xyz, const float* target,
-                        const SortedBatch& s);
+// The Morton-sorted copy of a query's points, with their places (s.index), when more than
+// s.limit of them are out of order.
+cudaError_t launch_sort_query(const Launch& L, const Bricks& br, const float* xyz, const SortedBatch& s);
+// The training pass's tiles (ws.tiles, ws.tile_ctr[0]): at most tp points each, levels up to
+// lcap with node boxes of at most capn nodes.  A batch that is not the sampler's (no
+// ws.bin_start) gets its unit starts and, if out of order, its sorted copy first
+// (ws.ustart, ws.sorted's counters and ws.tile_ctr cleared by the caller).
+cudaError_t launch_tiles(const Launch& L, const Model& md, const Bricks& br, const TrainWs& ws, const float* xyz,
+                         const float* target, int capn, int lcap, int tp);
 struct VolumeBoxes {
   int32_t lo[SRN_MAX_BRICKS][3];
   int32_t hi[SRN_MAX_BRICKS][3];

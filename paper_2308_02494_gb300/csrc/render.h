@@ -173,14 +173,15 @@ __device__ __forceinline__ void decode_voxel(const FwdBlock& k, int s, int (&v)[
   v[2] = k.v0[2] + z;
 }
 
-// Where the forward query takes its samples from, in groups of `group` (a multiple of 128,
-// at most kFwdGroup) neighbouring ones.
+// Where the forward query takes its samples from, in groups of `group` (a multiple of the
+// kernel's tile, 128 or, in float32, 64, at most fwd_group()) neighbouring ones.
 enum FwdKind { kFwdPoints = 0, kFwdRender = 1, kFwdDecode = 2 };
-constexpr int kFwdGroup = 512;
+constexpr int fwd_group(bool f32) { return f32 ? 256 : 512; }
 struct FwdSource {
   int32_t kind;
   int32_t group, groups;   // (kFwdPoints counts its groups per brick itself)
   int32_t run;             // consecutive groups of a CTA (set by the launch)
+  int32_t boxes;           // 0: read every corner from global memory (a few points: latency counts)
   const float* xyz;        // kFwdPoints, and their sorted copy, if one was made
   SortedBatch sorted;
   int32_t pix0, npix;      // kFwdRender: rays pix0 .. pix0 + npix - 1 of rp's order
@@ -188,10 +189,12 @@ struct FwdSource {
   RenderParams rp;
 };
 // The points of br in memory, in groups that leave a few for every CTA.
-inline FwdSource point_source(const Launch& L, const Bricks& br, const float* xyz) {
+inline FwdSource point_source(const Launch& L, const Bricks& br, const float* xyz, bool f32) {
   FwdSource s{};
   s.kind = kFwdPoints;
-  s.group = br.off[br.n] >= (int64_t)256 * 4 * L.num_sms ? 256 : 128;
+  s.boxes = br.off[br.n] > 16384;   // (1000 points of the 8-grid float32 model: 12.3 us with boxes)
+  s.group = 256;
+  while (s.group > (f32 ? 64 : 128) && br.off[br.n] < (int64_t)s.group * 4 * L.num_sms) s.group /= 2;
   s.xyz = xyz;
   return s;
 }
@@ -216,37 +219,20 @@ __device__ __forceinline__ int64_t decode_index(const FwdSource& src, const FwdB
 // f of every sample of the source: out[point], out[slot] (slots without a sample are left
 // alone) or out[voxel].
 cudaError_t launch_forward_bf16(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out);
+cudaError_t launch_forward_f32(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out);
+inline cudaError_t launch_forward(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
+  return md.F16 ? launch_forward_bf16(L, md, br, src, out) : launch_forward_f32(L, md, br, src, out);
+}
 
-struct RenderWs {
-  float* loc;       // [max_points][3] brick-local sample coordinates, slot order (float32 path)
-  uint32_t* rank;   // [max_points] rank inside the brick bucket (float32 path)
-  uint32_t* bid;    // [max_points] brick of the sample, all ones: no sample (float32 path)
-  uint32_t* pos;    // [max_points] bucketed position of each sample (float32 path)
-  float* xyz;       // [max_points][3] bucketed coordinates (float32 path)
-  float* val;       // [max_points] queried values: slot order (BF16), bucketed order (float32)
-  uint32_t* cnt;    // [B] bucket sizes
-  int64_t* off;     // [B + 1] bucket offsets
-};
-
-cudaError_t launch_render_batch(const Launch& L, const RenderParams& rp, const RenderWs& w, int pix0,
-                                int npix, const Model& md, const float* lut, float* rgba);
+// Rays pix0 .. pix0 + npix - 1 of rp's order; val: [max_points] scratch for their samples' values.
+cudaError_t launch_render_batch(const Launch& L, const RenderParams& rp, float* val, int pix0, int npix,
+                                const Model& md, const float* lut, float* rgba);
 // In-progress image after `done` pixels of the progressive order; `level` is the finest
 // complete hierarchy level (ignored when done = 0).
 cudaError_t launch_render_preview(const Launch& L, const RenderParams& rp, int done, int level,
                                   const float* rgba, float* preview);
 
-// The whole decode on the BF16 path: rp holds the bricks' grid, boxes and vox.
-cudaError_t launch_decode_bf16(const Launch& L, const RenderParams& rp, const Model& md, float* out);
-
-// One batch of the full-volume decode: the voxels [x0, x0+nx) x [y0, y0+ny) x [z0, z0+nz)
-// (all in brick `brick`, x fastest) queried in that brick's local coordinates (float32 path).
-struct DecodeChunk {
-  int64_t vox;
-  int32_t brick, n_bricks;
-  int32_t x0, nx, y0, ny, z0, nz;
-  int32_t lo[3], hi[3];   // the brick's voxel box (its local [-1, 1] corners)
-};
-cudaError_t launch_decode_chunk(const Launch& L, const DecodeChunk& c, const RenderWs& w, const Model& md,
-                                float* out);
+// The whole decode: rp holds the bricks' grid, boxes and vox.
+cudaError_t launch_decode(const Launch& L, const RenderParams& rp, const Model& md, float* out);
 
 }  // namespace srn

@@ -84,7 +84,7 @@ void make_layout(const srn_config* c, srn_layout* L) {
 struct WsLayout {
   size_t state, acc, gsum, rsum, rho, herr, sort_rank, sort_hist, feat, dfeat, gmax, ustart, tiles, tile_ctr;
   size_t sched, sring;
-  size_t r_loc, r_rank, r_bid, r_pos, r_xyz, r_val, r_cnt, r_off, total;
+  size_t r_val, total;
   size_t t_xyz, t_target, t_rank, t_hist, q_xyz, q_index, q_rank, q_hist;
 };
 
@@ -92,7 +92,10 @@ WsLayout ws_layout(const srn_config* c, int64_t maxp) {
   WsLayout w{};
   size_t o = 0;
   w.state = o; o += align256(sizeof(srn::StepState) + 64);
-  // (from here to r_sum's end: cleared by every backward pass)
+  const size_t hist = align256(sizeof(uint32_t) * ((size_t)srn::kSortBins * c->n_bricks + 1));   // and `moved`
+  // (from here to rsum's end: cleared by every backward pass)
+  w.ustart = o; o += c->precision == SRN_BF16 ? align256(sizeof(int32_t) * (srn::kUnits + 1) * c->n_bricks) : 0;
+  w.t_hist = o; o += hist;
   w.tile_ctr = o; o += align256(sizeof(int32_t) * 5);
   w.acc = o; o += align256(sizeof(double) * srn::kAccPerBrick * c->n_bricks);
   w.gsum = o; o += align256(sizeof(double) * 13 * c->n_grids * c->n_bricks);
@@ -112,24 +115,14 @@ WsLayout ws_layout(const srn_config* c, int64_t maxp) {
   // points (the smallest tile any tuning allows)
   const bool bf16 = c->precision == SRN_BF16;
   const int64_t max_tiles = (int64_t)c->n_bricks * (srn::kUnits + 1) + maxp / srn::kMinTilePoints + 1;
-  w.ustart = o; o += bf16 ? align256(sizeof(int32_t) * (srn::kUnits + 1) * c->n_bricks) : 0;
   w.tiles = o; o += bf16 ? align256(sizeof(srn::ScatTile) * max_tiles) : 0;
   w.sched = o; o += align256(sizeof(srn::BrickSched) * c->n_bricks);
   w.sring = o; o += align256(sizeof(double) * 2 * srn::kMaxDensityWindow * c->n_bricks);
-  w.r_loc = o; o += align256(sizeof(float) * 3 * maxp);
-  w.r_rank = o; o += align256(sizeof(uint32_t) * maxp);
-  w.r_bid = o; o += align256(sizeof(uint32_t) * maxp);
-  w.r_pos = o; o += align256(sizeof(uint32_t) * maxp);
-  w.r_xyz = o; o += align256(sizeof(float) * 3 * maxp);
-  w.r_val = o; o += align256(sizeof(float) * maxp);
-  w.r_cnt = o; o += align256(sizeof(uint32_t) * c->n_bricks);
-  w.r_off = o; o += align256(sizeof(int64_t) * (c->n_bricks + 1));
+  w.r_val = o; o += align256(sizeof(float) * maxp);   // values of a render batch's samples
   // sorted copies of a batch in memory: one of the training pass, one of the queries
-  const size_t hist = align256(sizeof(uint32_t) * ((size_t)srn::kSortBins * c->n_bricks + 1));   // and `moved`
   w.t_xyz = o; o += align256(sizeof(float) * 3 * maxp);
   w.t_target = o; o += align256(sizeof(float) * maxp);
   w.t_rank = o; o += align256(sizeof(uint32_t) * maxp);
-  w.t_hist = o; o += hist;
   w.q_xyz = o; o += align256(sizeof(float) * 3 * maxp);
   w.q_index = o; o += align256(sizeof(uint32_t) * maxp);
   w.q_rank = o; o += align256(sizeof(uint32_t) * maxp);
@@ -235,13 +228,13 @@ struct srn_handle {
     s.rank = reinterpret_cast<uint32_t*>(ws + (query ? wl.q_rank : wl.t_rank));
     s.hist = reinterpret_cast<uint32_t*>(ws + (query ? wl.q_hist : wl.t_hist));
     s.moved = s.hist + (size_t)srn::kSortBins * cfg.n_bricks;
-    if (!query) s.ustart = reinterpret_cast<int32_t*>(ws + wl.ustart);
     return s;
   }
   srn::Model model() const {
     srn::Model m{};
     const float* p = t.params_dev;
-    const __nv_bfloat16* s = reinterpret_cast<const __nv_bfloat16*>(t.shadow_dev);
+    const __nv_bfloat16* s =
+        cfg.precision == SRN_BF16 ? reinterpret_cast<const __nv_bfloat16*>(t.shadow_dev) : nullptr;
     m.G = p + lay.off_G;
     m.range = t.range_dev;
     m.F32 = p + lay.off_F;
@@ -295,32 +288,32 @@ srn_status check_training_counts(const srn::Bricks& br) {
   return SRN_OK;
 }
 
-// BF16 query of points in memory, through a sorted copy where that pays.  While `stream` is
+// Query of points in memory, through a sorted copy where that pays.  While `stream` is
 // being captured the copy is left alone: a replay could then meet another call's.
-cudaError_t forward_bf16(srn_handle* h, const srn::Launch& L, const srn::Model& md, const srn::Bricks& br,
+cudaError_t forward_points(srn_handle* h, const srn::Launch& L, const srn::Model& md, const srn::Bricks& br,
                          const float* xyz, float* out) {
-  srn::FwdSource src = srn::point_source(L, br, xyz);
+  srn::FwdSource src = srn::point_source(L, br, xyz, !md.F16);
   const int64_t n = br.off[br.n];
   // A sorted copy costs about 12 us and 0.05 ns per point.  It pays where the brick's grids
   // are well beyond L1 (random points, with it and without: 1 MB of features, 32768 points
   // 36 and 41 us; 8.4 MB, 53 and 84; 524288 points 161 and 430, 298 and 983); at 256 KB
   // from about 250 thousand points on (131072: 58 and 48; 524288: 114 and 149), below
   // that not at all (128 KB, 524288 points: 94 and 85).
-  const int64_t bytes = (int64_t)md.M * md.R * md.R * md.R * md.C * 2;
+  const int64_t bytes = (int64_t)md.M * md.R * md.R * md.R * md.C * (md.F16 ? 2 : 4);
   const int64_t least = bytes >= (512 << 10) ? 24576 : bytes >= (192 << 10) ? 262144 : INT64_MAX;
-  if (n < least || n > UINT32_MAX) return srn::launch_forward_bf16(L, md, br, src, out);
+  if (n < least || n > UINT32_MAX) return srn::launch_forward(L, md, br, src, out);
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(L.stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
     cudaGetLastError();
-    return srn::launch_forward_bf16(L, md, br, src, out);
+    return srn::launch_forward(L, md, br, src, out);
   }
   std::lock_guard<std::mutex> lock(h->query_mu);
   cudaError_t e = cudaStreamWaitEvent(L.stream, h->query_done, 0);   // (no-op before the first record)
   if (e != cudaSuccess) return e;
   src.sorted = h->sort_scratch(true);
   src.sorted.limit = (uint32_t)(n / 32);   // scan lines and other nearly sorted batches stay as they are
-  if ((e = srn::launch_sort(L, br, xyz, nullptr, src.sorted)) != cudaSuccess) return e;
-  if ((e = srn::launch_forward_bf16(L, md, br, src, out)) != cudaSuccess) return e;
+  if ((e = srn::launch_sort_query(L, br, xyz, src.sorted)) != cudaSuccess) return e;
+  if ((e = srn::launch_forward(L, md, br, src, out)) != cudaSuccess) return e;
   return cudaEventRecord(h->query_done, L.stream);
 }
 
@@ -359,10 +352,10 @@ srn_status run_query(srn_handle* h, void* stream, srn::QueryMode mode, const srn
     }
   }
   cudaError_t e;
-  if (h->cfg.precision != SRN_BF16)
-    e = srn::launch_query_fp32(L, mode, md, gr, br, ws, xyz, target, out);
-  else if (mode == srn::kForward)
-    e = forward_bf16(h, L, md, br, xyz, out);
+  if (mode == srn::kForward)
+    e = forward_points(h, L, md, br, xyz, out);
+  else if (h->cfg.precision != SRN_BF16)
+    e = srn::launch_train_fp32(L, mode == srn::kTrainDensity, md, gr, br, ws, xyz, target);
   else {
     // A caller's batch that is out of order runs through a sorted copy (random points, with
     // it and without: 2000 points 84 and 88 us at M = 8, R = 16, 162 and 293 at M = 64,
@@ -407,8 +400,8 @@ srn_status do_backward(srn_handle* h, void* stream, const float* xyz, const floa
   const bool dens = (flags & SRN_DENSITY) != 0 || sched;
   cudaError_t e = cudaMemsetAsync(h->t.grads_dev, 0, sizeof(float) * h->lay.n_params, s);
   if (e == cudaSuccess)
-    e = cudaMemsetAsync(h->ws + h->wl.tile_ctr, 0,
-                        h->wl.rsum - h->wl.tile_ctr + sizeof(double) * 12 * h->cfg.n_grids * h->cfg.n_bricks, s);
+    e = cudaMemsetAsync(h->ws + h->wl.ustart, 0,
+                        h->wl.rsum - h->wl.ustart + sizeof(double) * 12 * h->cfg.n_grids * h->cfg.n_bricks, s);
   if (e != cudaSuccess) return cuda_fail(e, "memset");
   const int rec_dg = (flags & SRN_REC_DG) ? 1 : 0;
   h->side.defer_join = split;
@@ -544,7 +537,7 @@ srn_status srn_create(const srn_config* cfg, const srn_tensors* t, void* workspa
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return cuda_fail(e, "device query");
-  e = cudaMemset(static_cast<unsigned char*>(workspace) + wl.state, 0, wl.tile_ctr - wl.state);
+  e = cudaMemset(static_cast<unsigned char*>(workspace) + wl.state, 0, wl.ustart - wl.state);
   if (e != cudaSuccess) return cuda_fail(e, "workspace init");
   srn_handle* h = new srn_handle();
   h->cfg = *cfg;
@@ -560,11 +553,15 @@ srn_status srn_create(const srn_config* cfg, const srn_tensors* t, void* workspa
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->side.fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->side.join, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->side.enc_done, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->query_done, cudaEventDisableTiming);
     if (e != cudaSuccess) {
       srn_destroy(h);
       return cuda_fail(e, "side stream");
     }
+  }
+  e = cudaEventCreateWithFlags(&h->query_done, cudaEventDisableTiming);
+  if (e != cudaSuccess) {
+    srn_destroy(h);
+    return cuda_fail(e, "event");
   }
   *out = h;
   return SRN_OK;
@@ -987,63 +984,16 @@ srn_status srn_decode(srn_handle* h, void* stream, const int32_t grid[3], const 
       const int64_t lo = boxes[6 * b + a], hi = boxes[6 * b + 3 + a];
       if (lo < 0 || hi >= vox || hi <= lo) return fail(SRN_ERR_INVALID_ARG, "box of brick %d invalid", b);
     }
-  // voxel i of an axis with I bricks belongs to brick min(floor(I i / (vox - 1)), I - 1):
-  // brick k holds [ceil(k (vox - 1) / I), ceil((k + 1)(vox - 1) / I) - 1] (the last one up to vox - 1)
-  auto first = [&](int k, int I) { return srn::decode_first(vox, k, I); };
-  unsigned char* ws = h->ws;
-  srn::RenderWs w{};
-  w.xyz = reinterpret_cast<float*>(ws + h->wl.r_xyz);
-  w.val = reinterpret_cast<float*>(ws + h->wl.r_val);
-  const srn::Model md = h->model();
-  if (h->cfg.precision == SRN_BF16) {
-    srn::RenderParams rp{};
-    rp.vox = vox;
-    for (int a = 0; a < 3; ++a) rp.grid[a] = grid[a];
-    for (int b = 0; b < h->cfg.n_bricks; ++b)
-      for (int a = 0; a < 3; ++a) {
-        rp.lo[b][a] = (int32_t)boxes[6 * b + a];
-        rp.hi[b][a] = (int32_t)boxes[6 * b + 3 + a];
-      }
-    const cudaError_t e = srn::launch_decode_bf16(h->launch(stream), rp, md, out);
-    return e == cudaSuccess ? SRN_OK : cuda_fail(e, "decode");
-  }
-  const int64_t cap = h->max_points;
-  for (int bz = 0; bz < grid[2]; ++bz)
-    for (int by = 0; by < grid[1]; ++by)
-      for (int bx = 0; bx < grid[0]; ++bx) {
-        const int b = bx + grid[0] * (by + grid[1] * bz);
-        const int bc[3] = {bx, by, bz};
-        int64_t lo[3], n[3];
-        for (int a = 0; a < 3; ++a) {
-          lo[a] = first(bc[a], grid[a]);
-          const int64_t hi = bc[a] == grid[a] - 1 ? vox - 1 : first(bc[a] + 1, grid[a]) - 1;
-          n[a] = hi - lo[a] + 1;
-        }
-        srn::DecodeChunk c{};
-        c.vox = vox;
-        c.brick = b;
-        c.n_bricks = h->cfg.n_bricks;
-        for (int a = 0; a < 3; ++a) {
-          c.lo[a] = (int32_t)boxes[6 * b + a];
-          c.hi[a] = (int32_t)boxes[6 * b + 3 + a];
-        }
-        if (n[0] <= 0 || n[1] <= 0 || n[2] <= 0) continue;
-        // chunks: whole planes if they fit, else whole rows, else parts of a row
-        const int64_t plane = n[0] * n[1];
-        const int64_t dz = plane <= cap ? std::max<int64_t>(1, cap / plane) : 1;
-        const int64_t dy = plane <= cap ? n[1] : std::max<int64_t>(1, cap / n[0]);
-        const int64_t dx = n[0] <= cap ? n[0] : cap;
-        for (int64_t z = 0; z < n[2]; z += dz)
-          for (int64_t y = 0; y < n[1]; y += dy)
-            for (int64_t x = 0; x < n[0]; x += dx) {
-              c.x0 = (int32_t)(lo[0] + x); c.nx = (int32_t)std::min(dx, n[0] - x);
-              c.y0 = (int32_t)(lo[1] + y); c.ny = (int32_t)std::min(dy, n[1] - y);
-              c.z0 = (int32_t)(lo[2] + z); c.nz = (int32_t)std::min(dz, n[2] - z);
-              cudaError_t e = srn::launch_decode_chunk(h->launch(stream), c, w, md, out);
-              if (e != cudaSuccess) return cuda_fail(e, "decode");
-            }
-      }
-  return SRN_OK;
+  srn::RenderParams rp{};
+  rp.vox = vox;
+  for (int a = 0; a < 3; ++a) rp.grid[a] = grid[a];
+  for (int b = 0; b < h->cfg.n_bricks; ++b)
+    for (int a = 0; a < 3; ++a) {
+      rp.lo[b][a] = (int32_t)boxes[6 * b + a];
+      rp.hi[b][a] = (int32_t)boxes[6 * b + 3 + a];
+    }
+  const cudaError_t e = srn::launch_decode(h->launch(stream), rp, h->model(), out);
+  return e == cudaSuccess ? SRN_OK : cuda_fail(e, "decode");
 }
 
 }  // extern "C"
@@ -1086,23 +1036,14 @@ srn_status render_params(srn_handle* h, const srn_camera* cam, const float* lut,
 // max_points samples.
 srn_status render_pixels(srn_handle* h, void* stream, const srn::RenderParams& rpi, const float* lut,
                          int64_t first, int64_t count, float* rgba) {
-  unsigned char* ws = h->ws;
-  srn::RenderWs w;
-  w.loc = reinterpret_cast<float*>(ws + h->wl.r_loc);
-  w.rank = reinterpret_cast<uint32_t*>(ws + h->wl.r_rank);
-  w.bid = reinterpret_cast<uint32_t*>(ws + h->wl.r_bid);
-  w.pos = reinterpret_cast<uint32_t*>(ws + h->wl.r_pos);
-  w.xyz = reinterpret_cast<float*>(ws + h->wl.r_xyz);
-  w.val = reinterpret_cast<float*>(ws + h->wl.r_val);
-  w.cnt = reinterpret_cast<uint32_t*>(ws + h->wl.r_cnt);
-  w.off = reinterpret_cast<int64_t*>(ws + h->wl.r_off);
+  float* val = reinterpret_cast<float*>(h->ws + h->wl.r_val);
   // Ray groups of 64 neighbouring pixels (8 x 8 of the raster order), 16 of the progressive
   // order's rows, fewer for a smaller image or workspace; a ray's samples are padded to
   // whole query groups where that adds at most an eighth.
   srn::RenderParams rp = rpi;
   rp.rg = rp.order ? 16 : 64;
   while (rp.rg > 1 && (rp.rg > count || (int64_t)rp.rg * rp.samples > h->max_points)) rp.rg /= 2;
-  const int per = srn::kFwdGroup / rp.rg;
+  const int per = srn::fwd_group(h->cfg.precision != SRN_BF16) / rp.rg;
   const int64_t pad = ((int64_t)rp.samples + per - 1) / per * per;
   rp.spr = pad * 8 <= (int64_t)rp.samples * 9 && pad * rp.rg <= h->max_points ? (int)pad : rp.samples;
   // whole ray groups whose slots fit the workspace's max_points samples (and 31 bits)
@@ -1111,7 +1052,7 @@ srn_status render_pixels(srn_handle* h, void* stream, const srn::RenderParams& r
   const srn::Model md = h->model();
   for (int64_t p0 = first; p0 < first + count; p0 += batch) {
     const int n = (int)std::min<int64_t>(batch, first + count - p0);
-    cudaError_t e = srn::launch_render_batch(h->launch(stream), rp, w, (int)p0, n, md, lut, rgba);
+    cudaError_t e = srn::launch_render_batch(h->launch(stream), rp, val, (int)p0, n, md, lut, rgba);
     if (e != cudaSuccess) return cuda_fail(e, "render");
   }
   return SRN_OK;
