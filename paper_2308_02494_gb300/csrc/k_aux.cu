@@ -218,8 +218,9 @@ __global__ void __launch_bounds__(ST) k_density_scalar(Bricks br, TrainWs ws, fl
 constexpr int DT = 128;   // points per tile
 constexpr int DNT = 256;  // threads
 
-static_assert(sizeof(TileMap) + DT * 2 * sizeof(float4) + kMaxGrids * 12 * sizeof(float) +
-                  DNT * sizeof(double) + 16 + 1024 <= kDensityCtaSmem,
+constexpr int kHalf = 7;   // of the 13 sums, staged at a time
+static_assert(kHalf * DNT >= kMaxGrids * 12, "the staging is also the transforms' place");
+static_assert(sizeof(TileMap) + DT * 2 * sizeof(float4) + kHalf * DNT * sizeof(float) + 16 + 1024 <= kDensityCtaSmem,
               "k_density_grad's shared memory must fit beside the scatter");
 // P10: the paper's p = 10 at compile time, with the x and y axes of the map, the flat
 // top and the sums carried as packed float pairs (the same arithmetic, fewer issued
@@ -229,8 +230,7 @@ __global__ void __launch_bounds__(DNT, 4)
 k_density_grad(Model md, Bricks br, TrainWs ws, const float* __restrict__ xyz, float eps) {
   __shared__ TileMap tm;
   __shared__ float4 sx[DT][2];   // (x, x, y, y), (z, z, q, 0): the pairs the packed path multiplies by
-  __shared__ float sg[kMaxGrids * 12];
-  __shared__ double red[DNT];
+  __shared__ __align__(16) float sg[kHalf * DNT];   // the brick's transforms; the sums' staging in flush
   __shared__ int s_tile;
   __shared__ float s_inv[3];
   if (ws.sorted.use()) xyz = ws.sorted.xyz;
@@ -244,20 +244,28 @@ k_density_grad(Model md, Bricks br, TrainWs ws, const float* __restrict__ xyz, f
   float s0 = 0.f, s3 = 0.f, s10 = 0.f, s11 = 0.f, s12 = 0.f;
   f2_t s12p = 0ull, s47 = 0ull, s58 = 0ull, s69 = 0ull;   // (s1, s2), (s4, s7), (s5, s8), (s6, s9)
 
+  // The threads' sums of brick b, added over the point groups in float64: one thread per
+  // (sum, grid), half of the sums at a time.  (Sum by sum, with M threads adding npg values
+  // each, it took 10 of 25 us of a 16384-point step at M = 8.)
   auto flush = [&](int b) {
     const float v[13] = {s0, f2_lo(s12p), f2_hi(s12p), s3, f2_lo(s47), f2_lo(s58), f2_lo(s69),
                          f2_hi(s47), f2_hi(s58), f2_hi(s69), s10, s11, s12};
 #pragma unroll
-    for (int j = 0; j < 13; ++j) {
-      red[tid] = (double)v[j];
+    for (int j0 = 0; j0 < 13; j0 += kHalf) {
+      const int nj = min(kHalf, 13 - j0);
       __syncthreads();
-      if (pg == 0) {
-        double s = 0.0;
-        for (int q = 0; q < npg; ++q) s += red[q * M + gi];
-        atomicAdd(ws.gsum + ((int64_t)b * M + gi) * 13 + j, s);
+#pragma unroll
+      for (int j = 0; j < kHalf; ++j)
+        if (j0 + j < 13) sg[j * DNT + tid] = v[j0 + j];
+      __syncthreads();
+      for (int o = tid; o < nj * M; o += DNT) {
+        const int j = o / M, g = o - j * M;
+        double t = 0.0;
+        for (int q = 0; q < npg; ++q) t += (double)sg[j * DNT + q * M + g];
+        atomicAdd(ws.gsum + ((int64_t)b * M + g) * 13 + j0 + j, t);
       }
-      __syncthreads();
     }
+    __syncthreads();
     s0 = s3 = s10 = s11 = s12 = 0.f;
     s12p = s47 = s58 = s69 = 0ull;
   };
