@@ -20,18 +20,45 @@ namespace {
 
 constexpr int kSortNT = 1024;
 
-// (the counters are cleared by the launch)
+// The points of this thread, first, first + step, ..., with their predecessors, four points'
+// loads in flight: f(point, bin code, predecessor's code, brick, first point of its brick).
+template <typename F>
+__device__ __forceinline__ void with_predecessors(const Bricks& br, const float* __restrict__ xyz, F f) {
+  const int64_t total = br.off[br.n], first = (int64_t)blockIdx.x * kSortNT + threadIdx.x;
+  const int64_t step = (int64_t)gridDim.x * kSortNT;
+  for (int64_t g0 = first; g0 < total; g0 += 4 * step) {
+    float q[4][6];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int64_t gi = g0 + k * step;
+#pragma unroll
+      for (int j = 0; j < 6; ++j) q[k][j] = gi < total && (gi > 0 || j > 2) ? xyz[3 * gi - 3 + j] : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int64_t gi = g0 + k * step;
+      if (gi >= total) break;
+      const int b = brick_of_point(br, gi);
+      f(gi, morton_bin(q[k][3], q[k][4], q[k][5]), morton_bin(q[k][0], q[k][1], q[k][2]), b, gi == br.off[b]);
+    }
+  }
+}
+
+// How many points come before their predecessor, first: a batch in order pays only for that.
 __global__ void __launch_bounds__(kSortNT) k_sort_query(Bricks br, const float* __restrict__ xyz, SortedBatch s) {
   cooperative_groups::grid_group grid = cooperative_groups::this_grid();
   const int64_t first = (int64_t)blockIdx.x * kSortNT + threadIdx.x;
+  uint32_t back = 0;
+  with_predecessors(br, xyz, [&](int64_t, uint32_t c, uint32_t before, int, bool head) { back += !head && before > c; });
+  back = __reduce_add_sync(0xffffffffu, back);
+  if ((threadIdx.x & 31) == 0 && back) atomicAdd(s.moved, back);   // (cleared before the launch)
   uint4* h4 = reinterpret_cast<uint4*>(s.hist);
   for (int64_t q = first; q < (int64_t)br.n * kSortBins / 4; q += (int64_t)gridDim.x * kSortNT)
     h4[q] = make_uint4(0u, 0u, 0u, 0u);
-  if (first == 0) *s.moved = 0u;
-  grid.sync();
-  sort_count<true>(br, xyz, s);
   grid.sync();
   if (*(volatile uint32_t*)s.moved <= s.limit) return;
+  sort_count(br, xyz, s);
+  grid.sync();
   for (int b = blockIdx.x; b < br.n; b += gridDim.x) {
     scan_bins(s.hist + (int64_t)b * kSortBins);
     __syncthreads();
@@ -169,33 +196,17 @@ k_sort_tiles(Bricks br, TrainWs ws, Model md, const float* __restrict__ xyz, con
              int capn, int lcap, int tp) {
   cooperative_groups::grid_group grid = cooperative_groups::this_grid();
   const SortedBatch& s = ws.sorted;
-  const int64_t total = br.off[br.n], first = (int64_t)blockIdx.x * kSortNT + threadIdx.x;
-  const int64_t step = (int64_t)gridDim.x * kSortNT;
   uint32_t back = 0;
-  for (int64_t g0 = first; g0 < total; g0 += 4 * step) {   // four points' loads in flight
-    float q[4][6];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int64_t gi = g0 + k * step;
-#pragma unroll
-      for (int j = 0; j < 6; ++j) q[k][j] = gi < total && (gi > 0 || j > 2) ? xyz[3 * gi - 3 + j] : 0.f;
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int64_t gi = g0 + k * step;
-      if (gi >= total) break;
-      const uint32_t u = morton_bin(q[k][3], q[k][4], q[k][5]) >> 3, v = morton_bin(q[k][0], q[k][1], q[k][2]) >> 3;
-      const int b = brick_of_point(br, gi);
-      const int64_t p = gi - br.off[b];
-      if (p == 0 || v != u) ws.ustart[(int64_t)b * (kUnits + 1) + u] = (int32_t)p + 1;
-      back += p != 0 && v > u;
-    }
-  }
+  with_predecessors(br, xyz, [&](int64_t gi, uint32_t c, uint32_t before, int b, bool head) {
+    const uint32_t u = c >> 3, v = before >> 3;
+    if (head || v != u) ws.ustart[(int64_t)b * (kUnits + 1) + u] = (int32_t)(gi - br.off[b]) + 1;
+    back += !head && v > u;
+  });
   back = __reduce_add_sync(0xffffffffu, back);
   if ((threadIdx.x & 31) == 0 && back) atomicAdd(s.moved, back);
   grid.sync();
   if (*(volatile uint32_t*)s.moved > s.limit) {
-    sort_count<false>(br, xyz, s);
+    sort_count(br, xyz, s);
     grid.sync();
     for (int b = blockIdx.x; b < br.n; b += gridDim.x) {
       scan_bins(s.hist + (int64_t)b * kSortBins);
@@ -220,6 +231,8 @@ int sort_blocks(int64_t n, const Launch& L) {
 
 cudaError_t launch_sort_query(const Launch& L, const Bricks& br, const float* xyz, const SortedBatch& s) {
   if (br.off[br.n] == 0) return cudaSuccess;
+  const cudaError_t e = cudaMemsetAsync(s.moved, 0, sizeof(uint32_t), L.stream);
+  if (e != cudaSuccess) return e;
   void* args[] = {(void*)&br, (void*)&xyz, (void*)&s};
   return cudaLaunchCooperativeKernel((const void*)k_sort_query, dim3(sort_blocks(br.off[br.n], L)), dim3(kSortNT), args,
                                      0, L.stream);

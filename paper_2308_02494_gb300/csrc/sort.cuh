@@ -63,14 +63,11 @@ __device__ __forceinline__ void scan_bins(uint32_t* hist) {
     h[32 * k] = make_uint4(s, s + v[k].x, s + v[k].x + v[k].y, s + v[k].x + v[k].y + v[k].z);
   }
 }
-// Ranks and bin counts (cleared before); COUNT: also the number of points whose bin comes
-// before their predecessor's.
-template <bool COUNT>
+// Ranks and bin counts (cleared before).
 __device__ __forceinline__ void sort_count(const Bricks& br, const float* __restrict__ xyz, const SortedBatch& s) {
   const int64_t total = br.off[br.n], first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
   const int lane = threadIdx.x & 31;
-  uint32_t moved = 0;
   for (int64_t gi = first; gi - lane < total; gi += step) {
     const bool in = gi < total;
     uint32_t key = 0xffffffffu;
@@ -78,7 +75,6 @@ __device__ __forceinline__ void sort_count(const Bricks& br, const float* __rest
       const int b = brick_of_point(br, gi);
       const uint32_t c = morton_bin(xyz[3 * gi], xyz[3 * gi + 1], xyz[3 * gi + 2]);
       key = (uint32_t)b * kSortBins + c;
-      if (COUNT && gi > br.off[b]) moved += morton_bin(xyz[3 * gi - 3], xyz[3 * gi - 2], xyz[3 * gi - 1]) > c;
     }
     // one atomic per distinct bin of the warp
     const unsigned grp = __match_any_sync(0xffffffffu, key);
@@ -87,10 +83,6 @@ __device__ __forceinline__ void sort_count(const Bricks& br, const float* __rest
     if (in && lane == leader) r = atomicAdd(s.hist + key, (uint32_t)__popc(grp));
     r = __shfl_sync(0xffffffffu, r, leader);
     if (in) s.rank[gi] = r + __popc(grp & ((1u << lane) - 1u));
-  }
-  if (COUNT) {
-    moved = __reduce_add_sync(0xffffffffu, moved);
-    if (lane == 0 && moved) atomicAdd(s.moved, moved);
   }
 }
 // The sorted copy (after the scan).
