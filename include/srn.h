@@ -198,7 +198,10 @@ srn_status srn_sample_target_tiled(srn_handle* h, void* stream, const float* til
                                    const float* xyz_dev, const int64_t* offsets, float* target_dev);
 
 /* Forward query f(x) = d(e(x)) (Eq. 1-3 and Sec. 4.1.2) of every brick's points:
- * out_dev[n] for xyz_dev[n].  offsets as in srn_sample_points. */
+ * out_dev[n] for xyz_dev[n].  offsets as in srn_sample_points.  A large batch whose points
+ * are in no spatial order is evaluated through a sorted copy in the workspace (the results
+ * are the same bits); calls on several streams or threads take that copy in turn, and a
+ * call on a stream that is being captured does without. */
 srn_status srn_forward(srn_handle* h, void* stream, const float* xyz_dev,
                        const int64_t* offsets, float* out_dev);
 

@@ -69,7 +69,7 @@ struct FwdLay {
   static constexpr int W2 = W1 + (F32 ? 64 * YP * 4 : 64 * K * 2);   // [64][64] bf16, or [64][HP] f32
   static constexpr int Y = W2 + (F32 ? 64 * HP * 4 : 64 * 64 * 2);   // [T][K] bf16, or [T][YP] f32 and over it,
   static constexpr int YB = F32 ? T * (YP > HP ? YP : HP) * 4 : T * K * 2;   // once read, the hidden layer [T][HP]
-  static constexpr int X = Y + YB;                   // [GROUP] float4: x, y, z, brick bits
+  static constexpr int X = Y + YB;                   // [GROUP] float4: x, y, z, bits of brick | slot << 8 (-1: no sample)
   static constexpr int W3 = X + GROUP * 16;          // [64] f32
   static constexpr int P = W3 + 64 * 4;              // [4][T] f32 partial outputs (float32)
   static constexpr int G = P + (F32 ? 4 * T * 4 : 0);   // [M][12] f32: column pairs of the x and y rows, then the z row
@@ -121,13 +121,15 @@ __device__ __forceinline__ float unord(uint32_t o) {
   return __uint_as_float(o ^ ((o & 0x80000000u) ? 0x80000000u : 0xffffffffu));
 }
 
-template <int K, int C, bool EVEN, bool F32>
+// VIEW: ray samples or voxels, else points in memory.
+template <int K, int C, bool EVEN, bool F32, bool VIEW>
 __global__ void __launch_bounds__(NT, fwd_ctas(K, F32))
-k_fwd(Model md, Bricks brp, FwdSource src, float* __restrict__ out, uint32_t pool_nodes) {
+k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> src, float* __restrict__ out,
+      uint32_t pool_nodes) {
   using L = FwdLay<K, C, F32>;
   using Node = FwdNode<C, F32>;
   constexpr int M = K / C, T = L::T;
-  constexpr int CW = F32 && K == 16 ? 4 : 8; // features per chunk
+  constexpr int CW = F32 && K == 16 ? 4 : 8;   // features per chunk
   constexpr int GPC = CW / C;                // grids per chunk
   constexpr int NCH = K / CW;                // chunks of a feature row
   constexpr int PP = K < 64 ? 1 : F32 ? 2 : 4;   // samples per thread
@@ -137,18 +139,23 @@ k_fwd(Model md, Bricks brp, FwdSource src, float* __restrict__ out, uint32_t poo
   __shared__ TileMap tm;
   __shared__ Bricks br;
   __shared__ uint32_t s_lo[3], s_hi[3], s_mask[2], s_np;
+  __shared__ float s_range[2];            // the brick's minimum and span
+  __shared__ FwdBlock blk;                // the group's voxels (kFwdDecode)
+  __shared__ uint16_t s_cnt[L::GROUP / 32];   // a mixed group's samples of a brick in each 32 slots,
+  __shared__ uint16_t s_first[SRN_MAX_BRICKS], s_end;   // where its bricks' samples start, and the last one's end
   __shared__ uint32_t s_slow[kMaxGrids / 32];   // bit i: grid i's corners come from global memory
   load_bricks(brp, br);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g8 = lane >> 2, t4 = lane & 3;
   const int R = md.R;
   const int GS = src.group;
-  if (src.kind == kFwdPoints) {
+  if constexpr (!VIEW) {
     if (tid == 0) build_tile_map(br, GS, tm);
     __syncthreads();
   }
-  const int total = src.kind == kFwdPoints ? tm.first[br.n] : src.groups;
-  const bool copied = src.sorted.use();
+  const int total = VIEW ? src.groups : tm.first[br.n];
+  const bool render = VIEW && src.kind == kFwdRender;
+  const bool copied = !VIEW && src.sorted.use();
   const float* xyz = copied ? src.sorted.xyz : src.xyz;
   float4* xs = reinterpret_cast<float4*>(sm + L::X);
   float* w3s = reinterpret_cast<float*>(sm + L::W3);
@@ -162,7 +169,6 @@ k_fwd(Model md, Bricks brp, FwdSource src, float* __restrict__ out, uint32_t poo
   const float ct = hs - 0.5f + kMagic;   // an integer when R is even (axis_cell)
 
   int cur = -1, hint = -1;
-  float span = 0.f, vmin = 0.f;
   // runs of src.run consecutive groups, dealt round robin to the CTAs: neighbouring groups
   // share a brick (and its weights), and a frame's empty corners are spread over the CTAs
   for (int r0 = blockIdx.x * src.run; r0 < total; r0 += gridDim.x * src.run) {
@@ -170,22 +176,21 @@ k_fwd(Model md, Bricks brp, FwdSource src, float* __restrict__ out, uint32_t poo
   for (int grp = r0; grp < r1; ++grp) {
     // ---- the group's samples: coordinates and brick (-1: no sample)
     if (tid < 2) s_mask[tid] = 0u;
+    if constexpr (VIEW)
+      if (tid == 2 && !render) blk = decode_block(src.dec, grp);
     __syncthreads();   // also: the previous group is done with xs, the boxes and Y
-    int64_t base;      // first point (kFwdPoints) or first slot
-    int ns;            // slots of the group that can hold samples
-    FwdBlock blk;
-    if (src.kind == kFwdPoints) {
+    // slots of the group that can hold samples, and the first one's point or slot (formed again
+    // where it is needed: a 64-bit value kept through the tiles costs registers they lack)
+    int ns = GS;
+    if (!VIEW) {
       hint = brick_of_tile(tm, br.n, grp, hint);
-      base = br.off[hint] + (int64_t)(grp - tm.first[hint]) * GS;
-      ns = (int)min((int64_t)GS, br.off[hint + 1] - base);
-    } else if (src.kind == kFwdRender) {
-      base = (int64_t)grp * GS;
-      ns = GS;
-    } else {
-      blk = decode_block(src.dec, grp);
-      base = 0;
+      ns = (int)min((int64_t)GS, br.off[hint + 1] - br.off[hint] - (int64_t)(grp - tm.first[hint]) * GS);
+    } else if (!render) {
       ns = blk.n[0] * blk.n[1] * blk.n[2];
     }
+    auto base = [&]() {
+      return VIEW ? (int64_t)grp * GS : br.off[hint] + (int64_t)(grp - tm.first[hint]) * GS;
+    };
     {
       Ray ray;
       int last = -1;
@@ -194,12 +199,12 @@ k_fwd(Model md, Bricks brp, FwdSource src, float* __restrict__ out, uint32_t poo
         float4 v = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
         if (s < ns) {
           int b;
-          if (src.kind == kFwdPoints) {
-            const float* q = xyz + 3 * (base + s);
+          if constexpr (!VIEW) {
+            const float* q = xyz + 3 * (base() + s);
             v.x = q[0]; v.y = q[1]; v.z = q[2];
             b = hint;
-          } else if (src.kind == kFwdRender) {
-            const RaySlot rs = ray_slot(src.rp, (int)base + s);
+          } else if (render) {
+            const RaySlot rs = ray_slot(src.rp, grp * GS + s);
             if (rs.ray != last) {   // slots NT apart share the ray when rg divides NT
               last = rs.ray;
               ray.hit = false;
@@ -210,28 +215,78 @@ k_fwd(Model md, Bricks brp, FwdSource src, float* __restrict__ out, uint32_t poo
             b = blk.brick;
             decode_point(src, blk, s, v.x, v.y, v.z);
           }
-          v.w = __int_as_float(b);
-          if (b >= 0) {
+          v.w = __int_as_float(b < 0 ? -1 : b | s << 8);
+          if (render && b >= 0) {
             if (b < 32) m0 |= 1u << b; else m1 |= 1u << (b - 32);
           }
         }
         xs[s] = v;
       }
-      m0 = __reduce_or_sync(0xffffffffu, m0);
-      m1 = __reduce_or_sync(0xffffffffu, m1);
-      if (lane == 0) {
-        if (m0) atomicOr(&s_mask[0], m0);
-        if (m1) atomicOr(&s_mask[1], m1);
+      if (render) {
+        m0 = __reduce_or_sync(0xffffffffu, m0);
+        m1 = __reduce_or_sync(0xffffffffu, m1);
+        if (lane == 0) {
+          if (m0) atomicOr(&s_mask[0], m0);
+          if (m1) atomicOr(&s_mask[1], m1);
+        }
       }
     }
-    __syncthreads();
-    unsigned long long mask = (unsigned long long)s_mask[0] | ((unsigned long long)s_mask[1] << 32);
+    unsigned long long mask = ns > 0 ? 1ull << (VIEW ? blk.brick : hint) : 0ull;
+    if (render) {
+      __syncthreads();
+      mask = (unsigned long long)s_mask[0] | ((unsigned long long)s_mask[1] << 32);
+    }
+    const bool mixed = VIEW && (mask & (mask - 1)) != 0;
+    if (mixed) {   // the bricks' samples one brick after the other, in order within each
+      constexpr int SPT = L::GROUP / NT;
+      float4 v[SPT];
+      int at[SPT], first = 0;
+#pragma unroll
+      for (int k = 0; k < SPT; ++k) {
+        at[k] = -1;
+        if (tid + k * NT < GS) v[k] = xs[tid + k * NT];
+      }
+      for (unsigned long long m = mask; m; m &= m - 1) {
+        const int b = __ffsll((long long)m) - 1;
+        __syncthreads();
+        uint32_t bal[SPT];
+#pragma unroll
+        for (int k = 0; k < SPT; ++k) {
+          const int s = tid + k * NT;
+          if (s >= GS) continue;   // (whole warps: GS is a multiple of 32)
+          const int w = __float_as_int(v[k].w);
+          bal[k] = __ballot_sync(0xffffffffu, w >= 0 && (w & 0xff) == b);
+          if (lane == 0) s_cnt[s / 32] = (uint16_t)__popc(bal[k]);
+        }
+        if (tid == 0) s_first[b] = (uint16_t)first;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < SPT; ++k) {
+          const int s = tid + k * NT;
+          if (s >= GS || !(bal[k] >> lane & 1u)) continue;
+          at[k] = first + __popc(bal[k] & ((1u << lane) - 1u));
+          for (int q = 0; q < s / 32; ++q) at[k] += s_cnt[q];
+        }
+        for (int q = 0; q < GS / 32; ++q) first += s_cnt[q];
+      }
+#pragma unroll
+      for (int k = 0; k < SPT; ++k)
+        if (at[k] >= 0) xs[at[k]] = v[k];
+      // (the other slots keep what they held: the bricks' ranges bound what is read)
+      if (tid == 0) s_end = (uint16_t)first;
+      __syncthreads();
+    }
     while (mask) {   // the bricks of the group (more than one only where rays cross a brick face)
       const int b = __ffsll((long long)mask) - 1;
       mask &= mask - 1;
+      // its samples: slots [i0, i1)
+      const int i0 = mixed ? s_first[b] : 0;
+      const int i1 = !mixed ? ns : mask ? s_first[__ffsll((long long)mask) - 1] : s_end;
       if (tid < 3) { s_lo[tid] = 0xffffffffu; s_hi[tid] = 0u; }
       if (tid == 3) s_np = 0u;
-      if (!src.boxes && tid < kMaxGrids / 32) s_slow[tid] = 0xffffffffu;
+      // (a mixed group's few samples of a brick are not worth the boxes' three barriers)
+      const bool stage = src.boxes && (!mixed || i1 - i0 > T);
+      if (!stage && tid < kMaxGrids / 32) s_slow[tid] = 0xffffffffu;
       if (b != cur) {
         cur = b;
         const void* w1p = F32 ? (const void*)(md.W1f + (int64_t)b * md.sW1) : (const void*)(md.W1h + (int64_t)b * md.sW1);
@@ -256,19 +311,18 @@ k_fwd(Model md, Bricks brp, FwdSource src, float* __restrict__ out, uint32_t poo
           const int i = c / 12, j = c - 12 * i;
           gs[c] = G[12 * i + (j < 8 ? (j >> 1) + 4 * (j & 1) : j)];
         }
-        vmin = md.range[2 * b];
-        span = md.range[2 * b + 1] - vmin;
+        if (tid < 2) s_range[tid] = tid ? md.range[2 * b + 1] - md.range[2 * b] : md.range[2 * b];
       }
       __syncthreads();
       const Node* Fb = F32 ? reinterpret_cast<const Node*>(md.F32 + (int64_t)b * md.sF)
                            : reinterpret_cast<const Node*>(md.F16 + (int64_t)b * md.sF);
-      if (src.boxes) {
+      if (stage) {
         {  // bounding box of the brick's samples (non-finite ones are inside no grid)
           uint32_t lo[3] = {0xffffffffu, 0xffffffffu, 0xffffffffu}, hi[3] = {0u, 0u, 0u};
           int n = 0;
-          for (int s = tid; s < ns; s += NT) {
+          for (int s = i0 + tid; s < i1; s += NT) {
             const float4 v = xs[s];
-            if (__float_as_int(v.w) == b && v.x - v.x == 0.f && v.y - v.y == 0.f && v.z - v.z == 0.f) {
+            if (__float_as_int(v.w) >= 0 && v.x - v.x == 0.f && v.y - v.y == 0.f && v.z - v.z == 0.f) {
               ++n;
               lo[0] = min(lo[0], ord(v.x)); hi[0] = max(hi[0], ord(v.x));
               lo[1] = min(lo[1], ord(v.y)); hi[1] = max(hi[1], ord(v.y));
@@ -342,16 +396,17 @@ k_fwd(Model md, Bricks brp, FwdSource src, float* __restrict__ out, uint32_t poo
         }
         __syncthreads();
       }
-      for (int t0 = 0; t0 < ns; t0 += T) {
+      for (int t0 = i0; t0 < i1; t0 += T) {
         {  // ---- encode
           const int pr = (warp / NQ) * 32 * PP + lane;   // this thread's rows: pr, pr + 32, ...
           f2_t xx[PP], yy[PP], zz[PP];
           bool valid[PP];
 #pragma unroll
           for (int p = 0; p < PP; ++p) {
-            const float4 v = xs[t0 + pr + 32 * p];
+            const int s = t0 + pr + 32 * p;
+            const float4 v = xs[min(s, GS - 1)];
             xx[p] = f2_pack(v.x, v.x); yy[p] = f2_pack(v.y, v.y); zz[p] = f2_pack(v.z, v.z);
-            valid[p] = __float_as_int(v.w) == b;
+            valid[p] = s < i1 && __float_as_int(v.w) >= 0;
           }
           // Eq. 1 and the cell of Eq. 2 of sample p in grid i
           struct Place {
@@ -412,16 +467,18 @@ k_fwd(Model md, Bricks brp, FwdSource src, float* __restrict__ out, uint32_t poo
             return c.in ? f : EncSNode<C>(0);
           };
           auto from_grid = [&](int i, const Place& c) -> EncSNode<C> {
-            if (!c.in) return EncSNode<C>(0);
+            // (a sample outside the grid reads, and drops, its first cell: no branch, so that the
+            // reads of several samples and grids are in flight together)
             constexpr uint32_t mb = (uint32_t)kMagicBits;
-            const Node* F0 = Fb + i * gsz + (((c.tz - mb) * R + (c.ty - mb)) * R + (c.tx - mb));
+            const Node* F0 = Fb + i * gsz + (c.in ? ((c.tz - mb) * R + (c.ty - mb)) * R + (c.tx - mb) : 0u);
             const Node* F2 = F0 + (uint32_t)(R * R);
             const Node n[8] = {__ldg(F0), __ldg(F0 + 1), __ldg(F0 + R), __ldg(F0 + R + 1),
                                __ldg(F2), __ldg(F2 + 1), __ldg(F2 + R), __ldg(F2 + R + 1)};
             EncSNode<C> v[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k) v[k] = widen<C, F32>(n[k]);
-            return blend(v, c);
+            const EncSNode<C> f = blend(v, c);
+            return c.in ? f : EncSNode<C>(0);
           };
           // the features of the chunk's grid j: packed pairs of bf16, or float32
           uint32_t o[PP][F32 ? CW : 4];
@@ -449,6 +506,14 @@ k_fwd(Model md, Bricks brp, FwdSource src, float* __restrict__ out, uint32_t poo
                 const FwdBox q = boxes[ch * GPC + j];
 #pragma unroll
                 for (int p = 0; p < PP; ++p) put(p, j, from_box(q, c[p]));
+              }
+            } else if (PP == 1 && unstaged == (1u << GPC) - 1u) {
+#pragma unroll
+              for (int j = 0; j < GPC; ++j) {
+                Place c[PP];
+                place(ch * GPC + j, c);
+#pragma unroll
+                for (int p = 0; p < PP; ++p) put(p, j, from_grid(ch * GPC + j, c[p]));
               }
             } else {
 #pragma unroll
@@ -482,11 +547,13 @@ k_fwd(Model md, Bricks brp, FwdSource src, float* __restrict__ out, uint32_t poo
           }
         }
         __syncthreads();
-        auto write = [&](int s, float f) {   // slot s of the group, if it holds a sample of this brick
-          if (__float_as_int(xs[s].w) != b) return;
-          f = fmaf(f, span, vmin);
-          if (src.kind == kFwdDecode) out[decode_index(src, blk, s)] = f;
-          else out[copied ? (int64_t)src.sorted.index[base + s] : base + s] = f;
+        auto write = [&](int r, float f) {   // the sample at r of the group, if there is one
+          if (r >= i1) return;
+          const int w = __float_as_int(xs[r].w), s = w >> 8;
+          if (w < 0) return;
+          f = fmaf(f, s_range[1], s_range[0]);
+          if constexpr (VIEW) out[render ? base() + s : decode_index(src, blk, s)] = f;
+          else out[copied ? (int64_t)src.sorted.index[base() + s] : base() + s] = f;
         };
         if constexpr (F32) {
           // ---- decoder in float32: warp w takes 32 rows x 16 columns of a hidden layer, lane
@@ -599,22 +666,27 @@ k_fwd(Model md, Bricks brp, FwdSource src, float* __restrict__ out, uint32_t poo
   }
 }
 
+// A CTA's dynamic shared memory: its share of the SM's (1 KB of it reserved), less the static part.
+inline int fwd_smem(const Launch& L, int K, bool F32) {
+  constexpr int kStatic = 1536;
+  return (L.smem_sm / fwd_ctas(K, F32) - 1024 - kStatic) / 128 * 128;
+}
+
 template <int K, int C, bool EVEN, bool F32>
 cudaError_t launch_k(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
   using Lay = FwdLay<K, C, F32>;
-  auto kern = k_fwd<K, C, EVEN, F32>;
-  // all of an SM's shared memory, halved (1 KB of each half is reserved), less the static part
-  int dev = 0, per_sm = 0;
-  cudaFuncAttributes fa;
-  cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess) return e;
-  if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
-  const int most = (per_sm / fwd_ctas(K, F32) - 1024 - (int)fa.sharedSizeBytes) / 128 * 128;
+  const bool view = src.kind != kFwdPoints;
+  auto points = k_fwd<K, C, EVEN, F32, false>;
+  auto views = k_fwd<K, C, EVEN, F32, true>;
+  const void* kern = view ? (const void*)views : (const void*)points;
+  const int most = fwd_smem(L, K, F32);
   if (most < Lay::POOL + 64) return cudaErrorInvalidConfiguration;
   const int smem = src.boxes ? most : Lay::POOL;   // (what is left is L1)
   const int pool = (smem - Lay::POOL) / (4 * C);
-  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return e;
+  cudaError_t e;
+  if (smem > (48 << 10) &&
+      (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess)
+    return e;
   int total = src.groups;
   if (src.kind == kFwdPoints) {
     total = 0;
@@ -624,7 +696,9 @@ cudaError_t launch_k(const Launch& L, const Model& md, const Bricks& br, const F
   FwdSource s = src;
   const int ctas = fwd_ctas(K, F32) * L.num_sms;
   s.run = std::max(1, std::min(4, total / (8 * ctas)));
-  kern<<<std::min((total + s.run - 1) / s.run, ctas), NT, smem, L.stream>>>(md, br, s, out, (uint32_t)pool);
+  const int grid = std::min((total + s.run - 1) / s.run, ctas);
+  if (view) views<<<grid, NT, smem, L.stream>>>(md, br, s, out, (uint32_t)pool);
+  else points<<<grid, NT, smem, L.stream>>>(md, br, s, out, (uint32_t)pool);
   return cudaGetLastError();
 }
 
@@ -646,6 +720,21 @@ cudaError_t SRN_FWD_LAUNCH(const Launch& L, const Model& md, const Bricks& br, c
     case 64: return launch_kc<64>(L, md, br, src, out);
     case 128: return launch_kc<128>(L, md, br, src, out);
     default: return cudaErrorInvalidValue;
+  }
+}
+
+int SRN_FWD_NODES(const Launch& L, const Model& md) {
+  auto nodes = [&](int K, int pool_at) { return (fwd_smem(L, K, kF32) - pool_at) / (4 * md.K); };
+  switch (md.K * 4 + md.C) {
+    case 16 * 4 + 1: return nodes(16, FwdLay<16, 1, kF32>::POOL);
+    case 16 * 4 + 2: return nodes(16, FwdLay<16, 2, kF32>::POOL);
+    case 32 * 4 + 1: return nodes(32, FwdLay<32, 1, kF32>::POOL);
+    case 32 * 4 + 2: return nodes(32, FwdLay<32, 2, kF32>::POOL);
+    case 64 * 4 + 1: return nodes(64, FwdLay<64, 1, kF32>::POOL);
+    case 64 * 4 + 2: return nodes(64, FwdLay<64, 2, kF32>::POOL);
+    case 128 * 4 + 1: return nodes(128, FwdLay<128, 1, kF32>::POOL);
+    case 128 * 4 + 2: return nodes(128, FwdLay<128, 2, kF32>::POOL);
+    default: return 0;
   }
 }
 

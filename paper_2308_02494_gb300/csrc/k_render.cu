@@ -7,6 +7,7 @@
 // transfer function read with linear interpolation.
 #include <algorithm>
 #include <climits>
+#include <cmath>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -111,9 +112,25 @@ cudaError_t launch_render_batch(const Launch& L, const RenderParams& rp, float* 
   br.n = rp.grid[0] * rp.grid[1] * rp.grid[2];
   FwdSource src{};
   src.kind = kFwdRender;
-  src.boxes = 1;
+  // Groups as large as they go while there is one for every CTA and a group's nodes in a grid
+  // (a cube of its samples' volume, the grids' 15% zoom, a partial cell and a node at either
+  // end) have room; where not even the smallest group's do, the corners come from L1 instead.
+  const int64_t slots = render_slots(rp, npix);
+  const int least = md.F16 ? 128 : 64, room = forward_box_nodes(L, md);
+  auto nodes = [&](int n) {
+    const float e = cbrtf((float)n * rp.cell) * 0.5f * (float)(md.R - 1) * 1.15f + 2.f;
+    return e * e * e;
+  };
   src.group = fwd_group(!md.F16);
-  src.groups = (int)((render_slots(rp, npix) + src.group - 1) / src.group);
+  while (src.group > least &&
+         (slots < (int64_t)src.group * 2 * L.num_sms || nodes(src.group) > (float)room))
+    src.group /= 2;
+  src.boxes = nodes(src.group) <= 2.f * (float)room;
+  if (!src.boxes) {
+    src.group = fwd_group(!md.F16);
+    while (src.group > least && slots < (int64_t)src.group * 2 * L.num_sms) src.group /= 2;
+  }
+  src.groups = (int)((slots + src.group - 1) / src.group);
   src.pix0 = pix0;
   src.npix = npix;
   src.rp = rp;
@@ -150,7 +167,7 @@ cudaError_t launch_decode(const Launch& L, const RenderParams& rp, const Model& 
   }
   // Blocks of at most `cap` voxels: as large as they go while there are a few for every CTA,
   // and of the shape with the fewest tiles of samples over the bricks, compact ones first.
-  const int tile = md.F16 ? 128 : 64;
+  const int tile = md.F16 ? 128 : 64;   // (the kernel's)
   int cap = fwd_group(!md.F16);
   while (cap > tile && voxels / cap < 8 * (int64_t)L.num_sms) cap /= 2;
   double best = 0.0;

@@ -1002,7 +1002,7 @@ cudaError_t launch_train_k(const Launch& L, bool dens, const Model& md, const Gr
     if (dens && side) {   // rho beside the decoder
       if ((e = cudaEventRecord(side->enc_done, L.stream)) != cudaSuccess) return e;
       if ((e = cudaStreamWaitEvent(side->stream, side->enc_done, 0)) != cudaSuccess) return e;
-      if ((e = launch_density_rho(Launch{side->stream, L.num_sms}, md, br, ws, xyz)) != cudaSuccess) return e;
+      if ((e = launch_density_rho(Launch{side->stream, L.num_sms, L.smem_sm}, md, br, ws, xyz)) != cudaSuccess) return e;
     } else if (dens && (e = launch_density_rho(L, md, br, ws, xyz)) != cudaSuccess) {
       return e;
     }
@@ -1032,7 +1032,7 @@ cudaError_t launch_train_k(const Launch& L, bool dens, const Model& md, const Gr
     const int ctas = std::min(std::max(tn.density_ctas, 1), kMaxDensityCtas);
     if ((e = cudaEventRecord(side->fork, L.stream)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(side->stream, side->fork, 0)) != cudaSuccess) return e;
-    if ((e = launch_density(Launch{side->stream, L.num_sms}, md, br, ws, xyz, ws.eps, ctas)) != cudaSuccess) return e;
+    if ((e = launch_density(Launch{side->stream, L.num_sms, L.smem_sm}, md, br, ws, xyz, ws.eps, ctas)) != cudaSuccess) return e;
     if ((e = cudaEventRecord(side->join, side->stream)) != cudaSuccess) return e;
   }
   {

@@ -11,6 +11,7 @@ enum QueryMode { kForward = 0, kTrain = 1, kTrainDensity = 2 };
 struct Launch {
   cudaStream_t stream;
   int num_sms;
+  int smem_sm;   // shared memory of an SM, bytes
 };
 
 // The forward queries are in render.h.  BF16 training pass: three kernels (encoder, decoder

@@ -15,6 +15,7 @@ struct RenderParams {
   // the other (spr per ray, the last ones empty), its rays fastest.  Consecutive slots are
   // then a compact bundle of ray segments, and a sample's slots are read coalesced over rays.
   int32_t rg, spr;
+  float cell;       // volume per sample in a brick's coordinates (about)
   int32_t grid[3];
   int64_t vox;
   float vmin, vmax;
@@ -116,7 +117,9 @@ __device__ __forceinline__ int level_pixels(const RenderParams& rp, int l) {
 // band blocks of 8 columns one after the other (the last band and block may be smaller), so
 // that 64 consecutive rays are neighbours in both directions.  Progressive order (Sec. 6):
 // the coarsest level's pixel (0, 0), then each finer level l's pixels not on level l+1's
-// grid, row by row: an even row b of the level has its odd columns, an odd row all.
+// grid, row by row: an even row b of the level has its odd columns, an odd row all.  (Taking
+// a level's rows in blocks of 8 x 8 as well, within a pass, was slower: 284 -> 308 us for the
+// 14400 pixels of a VGA view.)
 __device__ __forceinline__ int pixel_of(const RenderParams& rp, int k) {
   if (!rp.order) {
     const int band = k / (8 * rp.width), q = k - band * 8 * rp.width, hb = min(8, rp.height - 8 * band);
@@ -177,13 +180,15 @@ __device__ __forceinline__ void decode_voxel(const FwdBlock& k, int s, int (&v)[
 // kernel's tile, 128 or, in float32, 64, at most fwd_group()) neighbouring ones.
 enum FwdKind { kFwdPoints = 0, kFwdRender = 1, kFwdDecode = 2 };
 constexpr int fwd_group(bool f32) { return f32 ? 256 : 512; }
-struct FwdSource {
+struct FwdPointSource {   // what a kernel over points in memory gets (the rest is 2 KB of arguments)
   int32_t kind;
   int32_t group, groups;   // (kFwdPoints counts its groups per brick itself)
   int32_t run;             // consecutive groups of a CTA (set by the launch)
-  int32_t boxes;           // 0: read every corner from global memory (a few points: latency counts)
+  int32_t boxes;           // 0: read every corner from global memory
   const float* xyz;        // kFwdPoints, and their sorted copy, if one was made
   SortedBatch sorted;
+};
+struct FwdSource : FwdPointSource {
   int32_t pix0, npix;      // kFwdRender: rays pix0 .. pix0 + npix - 1 of rp's order
   DecodeParams dec;        // kFwdDecode; the bricks' boxes are rp.lo, rp.hi
   RenderParams rp;
@@ -192,7 +197,7 @@ struct FwdSource {
 inline FwdSource point_source(const Launch& L, const Bricks& br, const float* xyz, bool f32) {
   FwdSource s{};
   s.kind = kFwdPoints;
-  s.boxes = br.off[br.n] > 16384;   // (1000 points of the 8-grid float32 model: 12.3 us with boxes)
+  s.boxes = 0;   // (set for batches that are, or are brought, in order: boxes of random points are the whole grids)
   s.group = 256;
   while (s.group > (f32 ? 64 : 128) && br.off[br.n] < (int64_t)s.group * 4 * L.num_sms) s.group /= 2;
   s.xyz = xyz;
@@ -219,6 +224,12 @@ __device__ __forceinline__ int64_t decode_index(const FwdSource& src, const FwdB
 // f of every sample of the source: out[point], out[slot] (slots without a sample are left
 // alone) or out[voxel].
 cudaError_t launch_forward_bf16(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out);
+// Staged nodes per grid that a CTA of the forward kernel has room for.
+int forward_nodes_bf16(const Launch& L, const Model& md);
+int forward_nodes_f32(const Launch& L, const Model& md);
+inline int forward_box_nodes(const Launch& L, const Model& md) {
+  return md.F16 ? forward_nodes_bf16(L, md) : forward_nodes_f32(L, md);
+}
 cudaError_t launch_forward_f32(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out);
 inline cudaError_t launch_forward(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
   return md.F16 ? launch_forward_bf16(L, md, br, src, out) : launch_forward_f32(L, md, br, src, out);

@@ -1,5 +1,6 @@
 // C ABI of libsrn (declared in include/srn.h): argument validation, workspace
 // carving, kernel dispatch and the CUDA-graph cache of srn_train_step.
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -163,7 +164,7 @@ struct srn_handle {
   size_t ws_bytes;
   int64_t max_points;
   WsLayout wl;
-  int num_sms;
+  int num_sms, smem_sm;
   std::vector<GraphEntry> graphs;
   // training routine (srn_set_schedule)
   bool has_sched = false;
@@ -256,7 +257,7 @@ struct srn_handle {
     g.sF = lay.size_F; g.sW1 = lay.size_W1; g.sW2 = lay.size_W2; g.sw3 = lay.size_w3;
     return g;
   }
-  srn::Launch launch(void* stream) const { return srn::Launch{static_cast<cudaStream_t>(stream), num_sms}; }
+  srn::Launch launch(void* stream) const { return srn::Launch{static_cast<cudaStream_t>(stream), num_sms, smem_sm}; }
 };
 
 namespace {
@@ -294,13 +295,13 @@ cudaError_t forward_points(srn_handle* h, const srn::Launch& L, const srn::Model
                          const float* xyz, float* out) {
   srn::FwdSource src = srn::point_source(L, br, xyz, !md.F16);
   const int64_t n = br.off[br.n];
-  // A sorted copy costs about 12 us and 0.05 ns per point.  It pays where the brick's grids
-  // are well beyond L1 (random points, with it and without: 1 MB of features, 32768 points
-  // 36 and 41 us; 8.4 MB, 53 and 84; 524288 points 161 and 430, 298 and 983); at 256 KB
-  // from about 250 thousand points on (131072: 58 and 48; 524288: 114 and 149), below
-  // that not at all (128 KB, 524288 points: 94 and 85).
-  const int64_t bytes = (int64_t)md.M * md.R * md.R * md.R * md.C * (md.F16 ? 2 : 4);
-  const int64_t least = bytes >= (512 << 10) ? 24576 : bytes >= (192 << 10) ? 262144 : INT64_MAX;
+  // A sorted copy costs about 20 us and 0.05 ns per point, and pays where the brick's grids are
+  // well beyond L1, the sooner the larger they are (random points, with it and without, in us.
+  // BF16, 8.4 MB of features: 32768 points 55 and 48, 65536 73 and 80, 524288 292 and 520;
+  // 1 MB: 131072 68 and 63, 262144 99 and 119; 256 KB: 524288 114 and 109.  Float32, 17 MB:
+  // 65536 109 and 118; 2 MB: 131072 107 and 115; 512 KB: 262144 142 and 142).
+  const double bytes = (double)md.M * md.R * md.R * md.R * md.C * (md.F16 ? 2 : 4);
+  const int64_t least = bytes >= 400e3 ? (int64_t)(1.68e8 / sqrt(bytes)) : INT64_MAX;
   if (n < least || n > UINT32_MAX) return srn::launch_forward(L, md, br, src, out);
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(L.stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
@@ -310,6 +311,7 @@ cudaError_t forward_points(srn_handle* h, const srn::Launch& L, const srn::Model
   std::lock_guard<std::mutex> lock(h->query_mu);
   cudaError_t e = cudaStreamWaitEvent(L.stream, h->query_done, 0);   // (no-op before the first record)
   if (e != cudaSuccess) return e;
+  src.boxes = 1;
   src.sorted = h->sort_scratch(true);
   src.sorted.limit = (uint32_t)(n / 32);   // scan lines and other nearly sorted batches stay as they are
   if ((e = srn::launch_sort_query(L, br, xyz, src.sorted)) != cudaSuccess) return e;
@@ -533,9 +535,10 @@ srn_status srn_create(const srn_config* cfg, const srn_tensors* t, void* workspa
                         (const void*)t->adam_v_dev, (const void*)t->shadow_dev})
     if (reinterpret_cast<uintptr_t>(p) % 16 != 0)
       return fail(SRN_ERR_INVALID_ARG, "tensor pointers must be 16-byte aligned");
-  int dev = 0, sms = 0;
+  int dev = 0, sms = 0, smem_sm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   if (e != cudaSuccess) return cuda_fail(e, "device query");
   e = cudaMemset(static_cast<unsigned char*>(workspace) + wl.state, 0, wl.ustart - wl.state);
   if (e != cudaSuccess) return cuda_fail(e, "workspace init");
@@ -548,6 +551,7 @@ srn_status srn_create(const srn_config* cfg, const srn_tensors* t, void* workspa
   h->max_points = max_points;
   h->wl = wl;
   h->num_sms = sms;
+  h->smem_sm = smem_sm;
   if (cfg->precision == SRN_BF16) {
     e = cudaStreamCreateWithFlags(&h->side.stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->side.fork, cudaEventDisableTiming);
@@ -1037,13 +1041,23 @@ srn_status render_params(srn_handle* h, const srn_camera* cam, const float* lut,
 srn_status render_pixels(srn_handle* h, void* stream, const srn::RenderParams& rpi, const float* lut,
                          int64_t first, int64_t count, float* rgba) {
   float* val = reinterpret_cast<float*>(h->ws + h->wl.r_val);
-  // Ray groups of 64 neighbouring pixels (8 x 8 of the raster order), 16 of the progressive
-  // order's rows, fewer for a smaller image or workspace; a ray's samples are padded to
-  // whole query groups where that adds at most an eighth.
+  // Ray groups, so that a query group of `full` samples (rg rays x full / rg samples) is about
+  // as deep as it is wide: rays `px` apart, in blocks of the raster order (at most 64) or in
+  // rows of the progressive order's last level (at most 16), samples `dt` apart along chords
+  // of about 2.
   srn::RenderParams rp = rpi;
+  const int full = srn::fwd_group(h->cfg.precision != SRN_BF16);
+  const float* eye = rp.cam.eye;
+  const float far = rp.cam.ortho ? 1.f : std::max(0.1f, sqrtf(eye[0] * eye[0] + eye[1] * eye[1] + eye[2] * eye[2]));
+  const float stride = rp.order ? sqrtf((float)rp.width * (float)rp.height / (float)std::max<int64_t>(1, first + count)) : 1.f;
+  const float px = std::max(1e-6f, 2.f * fabsf(rp.cam.scale) * far / (float)rp.height * std::max(1.f, stride));
+  const float dt = 2.f / (float)rp.samples, ratio = (float)full * dt / px;
+  const float want = rp.order ? sqrtf(ratio) : powf(ratio, 2.f / 3.f);
   rp.rg = rp.order ? 16 : 64;
-  while (rp.rg > 1 && (rp.rg > count || (int64_t)rp.rg * rp.samples > h->max_points)) rp.rg /= 2;
-  const int per = srn::fwd_group(h->cfg.precision != SRN_BF16) / rp.rg;
+  while (rp.rg > 1 && ((float)rp.rg > 1.42f * want || rp.rg > count || (int64_t)rp.rg * rp.samples > h->max_points))
+    rp.rg /= 2;
+  rp.cell = px * px * dt * (float)(rp.grid[0] * rp.grid[1] * rp.grid[2]);
+  const int per = full / rp.rg;
   const int64_t pad = ((int64_t)rp.samples + per - 1) / per * per;
   rp.spr = pad * 8 <= (int64_t)rp.samples * 9 && pad * rp.rg <= h->max_points ? (int)pad : rp.samples;
   // whole ray groups whose slots fit the workspace's max_points samples (and 31 bits)
