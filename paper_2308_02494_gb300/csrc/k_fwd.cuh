@@ -30,12 +30,14 @@ namespace srn {
 namespace {
 
 constexpr int NT = 256;
-// CTAs per SM and samples per thread.  A thread's samples share the reads of a grid's map and
-// box (a warp-uniform 16-byte read takes two passes of the shared-memory pipe, 65% busy at
-// two samples per thread), which for K >= 64 pays for 128 registers and the two CTAs that
-// the feature tile and the boxes leave room for (frame of the paper-scale model: 157 ms at
-// two samples, 153 at four); the small models take three CTAs of one sample per thread
-// instead (progressive pass at K = 32: 318 and 292 us).
+// CTAs per SM and samples per thread.  With staged boxes a thread's samples share the reads of
+// a grid's map and box (a warp-uniform 16-byte read takes two passes of the shared-memory
+// pipe, 65% busy at two samples per thread), which for K >= 64 pays for 128 registers and
+// the two CTAs that the feature tile and the boxes leave room for (frame of the paper-scale
+// model: 157 ms at two samples, 153 at four); the small models take three CTAs of one sample
+// per thread instead (progressive pass at K = 32: 318 and 292 us).  Without boxes too: at
+// K = 128 three CTAs of one sample per thread took 593 and 31 us where two of four take 513
+// and 23 (a sparse progressive pass, a query of 5182 points).
 constexpr int fwd_ctas(int K, bool F32) { return F32 || K >= 64 ? 2 : 3; }
 
 // One grid node in global memory: C bf16 or C float32 values.
@@ -121,8 +123,8 @@ __device__ __forceinline__ float unord(uint32_t o) {
   return __uint_as_float(o ^ ((o & 0x80000000u) ? 0x80000000u : 0xffffffffu));
 }
 
-// VIEW: ray samples or voxels, else points in memory.
-template <int K, int C, bool EVEN, bool F32, bool VIEW>
+// VIEW: ray samples or voxels, else points in memory.  BOXES: with staged boxes.
+template <int K, int C, bool EVEN, bool F32, bool VIEW, bool BOXES>
 __global__ void __launch_bounds__(NT, fwd_ctas(K, F32))
 k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> src, float* __restrict__ out,
       uint32_t pool_nodes) {
@@ -285,7 +287,7 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
       if (tid < 3) { s_lo[tid] = 0xffffffffu; s_hi[tid] = 0u; }
       if (tid == 3) s_np = 0u;
       // (a mixed group's few samples of a brick are not worth the boxes' three barriers)
-      const bool stage = src.boxes && (!mixed || i1 - i0 > T);
+      const bool stage = BOXES && (!mixed || i1 - i0 > T);
       if (!stage && tid < kMaxGrids / 32) s_slow[tid] = 0xffffffffu;
       if (b != cur) {
         cur = b;
@@ -497,7 +499,7 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
           };
 #pragma unroll 1
           for (int ch = warp % NQ; ch < NCH; ch += NQ) {
-            const uint32_t unstaged = (s_slow[ch * GPC / 32] >> (ch * GPC % 32)) & ((1u << GPC) - 1u);
+            const uint32_t unstaged = !BOXES ? (1u << GPC) - 1u : (s_slow[ch * GPC / 32] >> (ch * GPC % 32)) & ((1u << GPC) - 1u);
             if (unstaged == 0u) {   // straight-line code over the chunk's grids
 #pragma unroll
               for (int j = 0; j < GPC; ++j) {
@@ -672,20 +674,20 @@ inline int fwd_smem(const Launch& L, int K, bool F32) {
   return (L.smem_sm / fwd_ctas(K, F32) - 1024 - kStatic) / 128 * 128;
 }
 
-template <int K, int C, bool EVEN, bool F32>
+template <int K, int C, bool EVEN, bool F32, bool BOXES>
 cudaError_t launch_k(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
   using Lay = FwdLay<K, C, F32>;
   const bool view = src.kind != kFwdPoints;
-  auto points = k_fwd<K, C, EVEN, F32, false>;
-  auto views = k_fwd<K, C, EVEN, F32, true>;
+  auto points = k_fwd<K, C, EVEN, F32, false, BOXES>;
+  auto views = k_fwd<K, C, EVEN, F32, true, BOXES>;
   const void* kern = view ? (const void*)views : (const void*)points;
   const int most = fwd_smem(L, K, F32);
   if (most < Lay::POOL + 64) return cudaErrorInvalidConfiguration;
-  const int smem = src.boxes ? most : Lay::POOL;   // (what is left is L1)
+  const int smem = BOXES ? most : Lay::POOL;   // (what is left is L1)
   const int pool = (smem - Lay::POOL) / (4 * C);
   cudaError_t e;
   if (smem > (48 << 10) &&
-      (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess)
+      (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
     return e;
   int total = src.groups;
   if (src.kind == kFwdPoints) {
@@ -702,40 +704,27 @@ cudaError_t launch_k(const Launch& L, const Model& md, const Bricks& br, const F
   return cudaGetLastError();
 }
 
+template <int K, int C, bool BOXES>
+cudaError_t launch_b(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
+  return md.R % 2 ? launch_k<K, C, false, kF32, BOXES>(L, md, br, src, out)
+                  : launch_k<K, C, true, kF32, BOXES>(L, md, br, src, out);
+}
 template <int K, int C>
 cudaError_t launch_c(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
-  return md.R % 2 ? launch_k<K, C, false, kF32>(L, md, br, src, out) : launch_k<K, C, true, kF32>(L, md, br, src, out);
-}
-template <int K>
-cudaError_t launch_kc(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
-  return md.C == 2 ? launch_c<K, 2>(L, md, br, src, out) : launch_c<K, 1>(L, md, br, src, out);
+  return src.boxes ? launch_b<K, C, true>(L, md, br, src, out) : launch_b<K, C, false>(L, md, br, src, out);
 }
 
 }  // namespace
 
-cudaError_t SRN_FWD_LAUNCH(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
-  switch (md.K) {
-    case 16: return launch_kc<16>(L, md, br, src, out);
-    case 32: return launch_kc<32>(L, md, br, src, out);
-    case 64: return launch_kc<64>(L, md, br, src, out);
-    case 128: return launch_kc<128>(L, md, br, src, out);
-    default: return cudaErrorInvalidValue;
-  }
+template <>
+cudaError_t launch_forward_k<kK, kF32>(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src,
+                                       float* out) {
+  return md.C == 2 ? launch_c<kK, 2>(L, md, br, src, out) : launch_c<kK, 1>(L, md, br, src, out);
 }
-
-int SRN_FWD_NODES(const Launch& L, const Model& md) {
-  auto nodes = [&](int K, int pool_at) { return (fwd_smem(L, K, kF32) - pool_at) / (4 * md.K); };
-  switch (md.K * 4 + md.C) {
-    case 16 * 4 + 1: return nodes(16, FwdLay<16, 1, kF32>::POOL);
-    case 16 * 4 + 2: return nodes(16, FwdLay<16, 2, kF32>::POOL);
-    case 32 * 4 + 1: return nodes(32, FwdLay<32, 1, kF32>::POOL);
-    case 32 * 4 + 2: return nodes(32, FwdLay<32, 2, kF32>::POOL);
-    case 64 * 4 + 1: return nodes(64, FwdLay<64, 1, kF32>::POOL);
-    case 64 * 4 + 2: return nodes(64, FwdLay<64, 2, kF32>::POOL);
-    case 128 * 4 + 1: return nodes(128, FwdLay<128, 1, kF32>::POOL);
-    case 128 * 4 + 2: return nodes(128, FwdLay<128, 2, kF32>::POOL);
-    default: return 0;
-  }
+template <>
+int forward_nodes_k<kK, kF32>(const Launch& L, const Model& md) {
+  const int at = md.C == 2 ? FwdLay<kK, 2, kF32>::POOL : FwdLay<kK, 1, kF32>::POOL;
+  return (fwd_smem(L, kK, kF32) - at) / (4 * kK);
 }
 
 }  // namespace srn

@@ -223,16 +223,38 @@ __device__ __forceinline__ int64_t decode_index(const FwdSource& src, const FwdB
 
 // f of every sample of the source: out[point], out[slot] (slots without a sample are left
 // alone) or out[voxel].
-cudaError_t launch_forward_bf16(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out);
+// (One translation unit per feature count K and precision.)
+template <int K, bool F32>
+cudaError_t launch_forward_k(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out);
 // Staged nodes per grid that a CTA of the forward kernel has room for.
-int forward_nodes_bf16(const Launch& L, const Model& md);
-int forward_nodes_f32(const Launch& L, const Model& md);
-inline int forward_box_nodes(const Launch& L, const Model& md) {
-  return md.F16 ? forward_nodes_bf16(L, md) : forward_nodes_f32(L, md);
-}
-cudaError_t launch_forward_f32(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out);
+template <int K, bool F32>
+int forward_nodes_k(const Launch& L, const Model& md);
+#define SRN_FWD(K, F32)                                                                            \
+  template <>                                                                                      \
+  cudaError_t launch_forward_k<K, F32>(const Launch&, const Model&, const Bricks&, const FwdSource&, float*); \
+  template <>                                                                                      \
+  int forward_nodes_k<K, F32>(const Launch&, const Model&);
+SRN_FWD(16, false) SRN_FWD(32, false) SRN_FWD(64, false) SRN_FWD(128, false)
+SRN_FWD(16, true) SRN_FWD(32, true) SRN_FWD(64, true) SRN_FWD(128, true)
+#undef SRN_FWD
 inline cudaError_t launch_forward(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
-  return md.F16 ? launch_forward_bf16(L, md, br, src, out) : launch_forward_f32(L, md, br, src, out);
+  const bool f32 = !md.F16;
+  switch (md.K) {
+    case 16: return f32 ? launch_forward_k<16, true>(L, md, br, src, out) : launch_forward_k<16, false>(L, md, br, src, out);
+    case 32: return f32 ? launch_forward_k<32, true>(L, md, br, src, out) : launch_forward_k<32, false>(L, md, br, src, out);
+    case 64: return f32 ? launch_forward_k<64, true>(L, md, br, src, out) : launch_forward_k<64, false>(L, md, br, src, out);
+    case 128: return f32 ? launch_forward_k<128, true>(L, md, br, src, out) : launch_forward_k<128, false>(L, md, br, src, out);
+    default: return cudaErrorInvalidValue;
+  }
+}
+inline int forward_box_nodes(const Launch& L, const Model& md) {
+  const bool f32 = !md.F16;
+  switch (md.K) {
+    case 16: return f32 ? forward_nodes_k<16, true>(L, md) : forward_nodes_k<16, false>(L, md);
+    case 32: return f32 ? forward_nodes_k<32, true>(L, md) : forward_nodes_k<32, false>(L, md);
+    case 64: return f32 ? forward_nodes_k<64, true>(L, md) : forward_nodes_k<64, false>(L, md);
+    default: return f32 ? forward_nodes_k<128, true>(L, md) : forward_nodes_k<128, false>(L, md);
+  }
 }
 
 // Rays pix0 .. pix0 + npix - 1 of rp's order; val: [max_points] scratch for their samples' values.

@@ -137,3 +137,35 @@ def test_training_batch_in_no_order(shape, n, density):
         assert rel_l2(gb[k], ga[k]) < 2e-3, k
     if density:
         assert rel_l2(gb["G"], ga["G"]) < 2e-3
+
+
+@pytest.mark.parametrize("ordered", [True, False])
+def test_captured_backward_follows_its_batch(ordered):
+    """A captured backward pass decides on the device, at each replay, whether the points
+    then in its buffer need the sorted copy."""
+    import torch
+
+    ensure_built()
+    n = 40_000
+    r = np.random.default_rng(5)
+    x = r.uniform(-1, 1, (n, 3)).astype(np.float32)
+    t = r.uniform(0, 1, n).astype(np.float32)
+    o = morton_order(x)
+    first, then = (np.arange(n), o) if ordered else (o, np.arange(n))
+    net = _model((32, 20, 2), 1, n)
+    xs, ts = torch.as_tensor(x[first], device="cuda"), torch.as_tensor(t[first], device="cuda")
+    net.backward(xs, ts, [0, n], density=True)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        net.backward(xs, ts, [0, n], density=True)
+    xs.copy_(torch.as_tensor(x[then], device="cuda"))
+    ts.copy_(torch.as_tensor(t[then], device="cuda"))
+    g.replay()
+    torch.cuda.synchronize()
+    got, losses = net.get("grads")[0], net.losses.cpu().numpy().copy()
+    want_l = net.backward(xs, ts, [0, n], density=True).cpu().numpy()
+    want = net.get("grads")[0]
+    np.testing.assert_allclose(losses, want_l, rtol=1e-6)
+    for k in ("F", "W1", "W2", "w3", "G"):
+        assert rel_l2(got[k], want[k]) < 1e-5, k
