@@ -685,6 +685,11 @@ int blocks_for(int64_t n, int threads, int num_sms, int per_sm) {
 cudaError_t launch_density_rho(const Launch& L, const Model& md, const Bricks& br, const TrainWs& ws,
                                const float* xyz) {
   if (br.off[br.n] == 0) return cudaSuccess;
+  // The counter is clear already: the node holds this pass back until the decoder, ready at the
+  // same moment, has its two CTAs on every SM.  Where this pass's CTA came first, only one of
+  // them found registers, and the decoder took 0.645 ms beside it instead of 0.42.
+  const cudaError_t e = cudaMemsetAsync(ws.tile_ctr + 4, 0, sizeof(int32_t), L.stream);
+  if (e != cudaSuccess) return e;
   if (md.p == 10) k_density_rho<true><<<L.num_sms, RHT, 0, L.stream>>>(md, br, ws, xyz);
   else k_density_rho<false><<<L.num_sms, RHT, 0, L.stream>>>(md, br, ws, xyz);
   return cudaGetLastError();
