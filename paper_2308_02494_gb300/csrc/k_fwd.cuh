@@ -234,11 +234,11 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
         }
       }
     }
-    unsigned long long mask = ns > 0 ? 1ull << (VIEW ? blk.brick : hint) : 0ull;
-    if (render) {
-      __syncthreads();
-      mask = (unsigned long long)s_mask[0] | ((unsigned long long)s_mask[1] << 32);
-    }
+    unsigned long long mask = render || ns <= 0 ? 0ull : 1ull << (VIEW ? blk.brick : hint);
+    // (a decode's block that is empty, at the end of a shorter brick, comes to no other barrier
+    // before `blk` is written again)
+    if constexpr (VIEW) __syncthreads();
+    if (render) mask = (unsigned long long)s_mask[0] | ((unsigned long long)s_mask[1] << 32);
     const bool mixed = VIEW && (mask & (mask - 1)) != 0;
     if (mixed) {   // the bricks' samples one brick after the other, in order within each
       constexpr int SPT = L::GROUP / NT;
