@@ -23,23 +23,13 @@
 // The blend is rounded as the global read's was, so the features are the same bits.
 #include <algorithm>
 
-#include "enc_ops.cuh"
+#include "fwd_box.cuh"
 #include "kernels.h"
-#include "render.h"
 
 namespace srn {
 namespace {
 
 constexpr int NT = 256;
-// CTAs per SM and samples per thread.  With staged boxes a thread's samples share the reads of
-// a grid's map and box (a warp-uniform 16-byte read takes two passes of the shared-memory
-// pipe, 65% busy at two samples per thread), which for K >= 64 pays for 128 registers and
-// the two CTAs that the feature tile and the boxes leave room for (frame of the paper-scale
-// model: 157 ms at two samples, 153 at four); the small models take three CTAs of one sample
-// per thread instead (progressive pass at K = 32: 318 and 292 us).  Without boxes too: at
-// K = 128 three CTAs of one sample per thread took 593 and 31 us where two of four take 513
-// and 23 (a sparse progressive pass, a query of 5182 points).
-constexpr int fwd_ctas(int K, bool F32) { return F32 || K >= 64 ? 2 : 3; }
 
 // One grid node in global memory: C bf16 or C float32 values.
 template <int C, bool F32>
@@ -49,70 +39,6 @@ __device__ __forceinline__ EncSNode<C> widen(FwdNode<C, F32> v) {   // as C floa
   if constexpr (F32) return v;
   else if constexpr (C == 2) return bf2_bits(v);
   else return __uint_as_float((uint32_t)v << 16);
-}
-
-// One grid's staged box as the encoder sees it.  With t the cell's float bits of
-// axis_cell (cell + kMagicBits) per axis, the byte address of the cell's first corner is
-// at + tz oz + ty oy + tx (node bytes), all modulo 2^32.
-struct __align__(16) FwdBox {
-  uint32_t at, oy, oz, pad;
-};
-// What staging needs: lo | nodes per axis as in block_box, and the pool offset in nodes.
-struct FwdStage {
-  uint32_t lo, n, at;
-};
-
-template <int K, int C, bool F32>
-struct FwdLay {
-  static constexpr int M = K / C;
-  static constexpr int T = F32 ? 64 : 128;           // samples per feature tile
-  static constexpr int GROUP = fwd_group(F32);       // samples per group, at most
-  static constexpr int YP = K + 4, HP = 64 + 4;      // row pitches of the float32 tiles (floats)
-  static constexpr int W1 = 0;                       // [64][K] bf16 swizzled, or [64][YP] f32
-  static constexpr int W2 = W1 + (F32 ? 64 * YP * 4 : 64 * K * 2);   // [64][64] bf16, or [64][HP] f32
-  static constexpr int Y = W2 + (F32 ? 64 * HP * 4 : 64 * 64 * 2);   // [T][K] bf16, or [T][YP] f32 and over it,
-  static constexpr int YB = F32 ? T * (YP > HP ? YP : HP) * 4 : T * K * 2;   // once read, the hidden layer [T][HP]
-  static constexpr int X = Y + YB;                   // [GROUP] float4: x, y, z, bits of brick | slot << 8 (-1: no sample)
-  static constexpr int W3 = X + GROUP * 16;          // [64] f32
-  static constexpr int P = W3 + 64 * 4;              // [4][T] f32 partial outputs (float32)
-  static constexpr int G = P + (F32 ? 4 * T * 4 : 0);   // [M][12] f32: column pairs of the x and y rows, then the z row
-  static constexpr int BOX = G + M * 48;             // [M] FwdBox
-  static constexpr int STG = BOX + M * 16;           // [M] FwdStage
-  static constexpr int POOL = (STG + M * 12 + 15) / 16 * 16;   // staged nodes, C float32 each
-};
-
-// Node box of grid g over the block [lo, hi]: block_box with a margin that covers the
-// rounding of the per-sample map for any transform, so that every sample of the block
-// inside the grid has its cell in the box (no per-sample test is needed).
-// gp: the grid's map as load order keeps it, the column pairs of its x and y rows, then
-// its z row.
-__device__ __forceinline__ bool sample_box(const float (&lo)[3], const float (&hi)[3], const float* gp, int R,
-                                           uint32_t& blo, uint32_t& bn) {
-  const float h = 0.5f * (float)(R - 1), top = (float)(R - 1);
-  blo = 0;
-  bn = 0;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    auto g = [&](int k) { return d < 2 ? gp[2 * k + d] : gp[8 + k]; };
-    float umin = g(3), umax = umin, mag = fabsf(umin);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const float a = g(k), p = a * lo[k], q = a * hi[k];
-      umin += fminf(p, q);
-      umax += fmaxf(p, q);
-      mag += fmaxf(fabsf(p), fabsf(q));
-    }
-    // per sample and here: at most 5 roundings of sums of at most mag, each 2^-24 of them
-    const float pu = mag * 1e-6f, ps = fmaf(h, pu, 1e-3f);
-    if (umax + pu < -1.f || umin - pu > 1.f) return false;
-    const float a = fmaf(umin, h, h) - ps, b = fmaf(umax, h, h) + ps;
-    const float s0 = a >= 0.f ? fminf(a, top) : 0.f;     // (a NaN bound takes the whole axis)
-    const float s1 = b <= top ? fmaxf(b, 0.f) : top;
-    const int c0 = min((int)s0, R - 2), c1 = min((int)s1, R - 2);
-    blo |= (uint32_t)c0 << (8 * d);
-    bn |= (uint32_t)(c1 - c0 + 2) << (8 * d);
-  }
-  return true;
 }
 
 // Float order as unsigned integer order (for min/max reductions).
@@ -367,13 +293,7 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
             const uint32_t at = used + incl - nodes;
             const bool fits = nodes && at + nodes <= pool_nodes;
             if (i < M) {
-              FwdBox q;
-              q.oy = nx * kNB;
-              q.oz = nx * ny * kNB;
-              q.at = spool + at * kNB - ((blo >> 16 & 0xffu) + (uint32_t)kMagicBits) * q.oz -
-                     ((blo >> 8 & 0xffu) + (uint32_t)kMagicBits) * q.oy - ((blo & 0xffu) + (uint32_t)kMagicBits) * kNB;
-              q.pad = 0u;
-              boxes[i] = q;
+              boxes[i] = fwd_box<C>(blo, fits ? bn : 0u, spool + at * kNB);
               stg[i] = FwdStage{blo, fits ? bn : 0u, at};
             }
             const uint32_t slow = __ballot_sync(0xffffffffu, any && !fits);
@@ -460,7 +380,7 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
             }
           };
           // from a staged box (a sample outside the grid reads, and drops, nodes at the pool's
-          // start: the offsets to a cell's last corner are less than the box's size)
+          // start, see fwd_box)
           auto from_box = [&](const FwdBox& q, const Place& c) -> EncSNode<C> {
             const uint32_t a = q.at + c.tz * q.oz + c.ty * q.oy + c.tx * kNB, a0 = c.in ? a : spool;
             const uint32_t a1 = a0 + q.oy, a2 = a0 + q.oz, a3 = a2 + q.oy;
@@ -669,12 +589,6 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
   }
 }
 
-// A CTA's dynamic shared memory: its share of the SM's (1 KB of it reserved), less the static part.
-inline int fwd_smem(const Launch& L, int K, bool F32) {
-  constexpr int kStatic = 1536;
-  return (L.smem_sm / fwd_ctas(K, F32) - 1024 - kStatic) / 128 * 128;
-}
-
 template <int K, int C, bool EVEN, bool F32, bool BOXES>
 cudaError_t launch_k(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
   using Lay = FwdLay<K, C, F32>;
@@ -682,8 +596,8 @@ cudaError_t launch_k(const Launch& L, const Model& md, const Bricks& br, const F
   auto points = k_fwd<K, C, EVEN, F32, false, BOXES>;
   auto views = k_fwd<K, C, EVEN, F32, true, BOXES>;
   const void* kern = view ? (const void*)views : (const void*)points;
-  const int most = fwd_smem(L, K, F32);
-  if (most < Lay::POOL + 64) return cudaErrorInvalidConfiguration;
+  const int most = fwd_smem(L.smem_sm, K, F32);
+  if (most < Lay::POOL + 64) return cudaErrorInvalidConfiguration;   // room for dropped reads (fwd_box)
   const int smem = BOXES ? most : Lay::POOL;   // (what is left is L1)
   const int pool = (smem - Lay::POOL) / (4 * C);
   cudaError_t e;
@@ -725,7 +639,7 @@ cudaError_t launch_forward_k<kK, kF32>(const Launch& L, const Model& md, const B
 template <>
 int forward_nodes_k<kK, kF32>(const Launch& L, const Model& md) {
   const int at = md.C == 2 ? FwdLay<kK, 2, kF32>::POOL : FwdLay<kK, 1, kF32>::POOL;
-  return (fwd_smem(L, kK, kF32) - at) / (4 * kK);
+  return (fwd_smem(L.smem_sm, kK, kF32) - at) / (4 * kK);
 }
 
 }  // namespace srn
