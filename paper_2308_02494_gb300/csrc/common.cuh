@@ -65,6 +65,7 @@ struct SortedBatch {
   uint32_t* rank;      // [N] scratch: rank inside the bin
   uint32_t* hist;      // [B][kSortBins] bin starts within the brick (written with the copy)
   uint32_t* moved;
+  uint32_t* next;      // (queries) the next call's `moved`
   uint32_t limit;
   __device__ __forceinline__ bool use() const { return moved && *moved > limit; }
 };
@@ -287,6 +288,15 @@ __device__ __forceinline__ void build_tile_map(const Bricks& br, int T, TileMap&
   for (int b = 0; b < br.n; ++b) {
     tm.first[b] = acc;
     acc += (int)((br.off[b + 1] - br.off[b] + T - 1) / T);
+  }
+  tm.first[br.n] = acc;
+}
+// Tiles of 2^lt points.
+__device__ __forceinline__ void build_tile_map_log2(const Bricks& br, int lt, TileMap& tm) {
+  int acc = 0;
+  for (int b = 0; b < br.n; ++b) {
+    tm.first[b] = acc;
+    acc += (int)((br.off[b + 1] - br.off[b] + (1 << lt) - 1) >> lt);
   }
   tm.first[br.n] = acc;
 }

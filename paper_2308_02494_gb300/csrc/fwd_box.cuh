@@ -10,10 +10,13 @@ namespace srn {
 // pipe, 65% busy at two samples per thread), which for K >= 64 pays for 128 registers and
 // the two CTAs that the feature tile and the boxes leave room for (frame of the paper-scale
 // model: 157 ms at two samples, 153 at four); the small models take three CTAs of one sample
-// per thread instead (progressive pass at K = 32: 318 and 292 us).  Without boxes too: at
-// K = 128 three CTAs of one sample per thread took 593 and 31 us where two of four take 513
-// and 23 (a sparse progressive pass, a query of 5182 points).
-constexpr int fwd_ctas(int K, bool F32) { return F32 || K >= 64 ? 2 : 3; }
+// per thread instead (progressive pass at K = 32: 318 and 292 us).  Without boxes what is left
+// of shared memory is L1, the corners' latency asks for warps, and three CTAs of one sample
+// per thread, of two at K = 128, are best (BF16 queries at two CTAs of four samples, three of
+// two, three of one: K = 128, 500000 points in order 198, 189 and 197 us; K = 64, 60000 points
+// in no order 46.5, 40.7 and 40.5).  Float32 has the registers for two (K = 128, 20000 points
+// in no order: 63.5 us at two samples per thread, 57.0 at one).
+constexpr int fwd_ctas(int K, bool F32, bool boxes) { return F32 || (boxes && K >= 64) ? 2 : 3; }
 
 // One grid's staged box as the encoder sees it.  With t the cell's float bits of
 // axis_cell (cell + kMagicBits) per axis, the byte address of the cell's first corner is
@@ -26,11 +29,11 @@ struct FwdStage {
   uint32_t lo, n, at;
 };
 
-template <int K, int C, bool F32>
+template <int K, int C, bool F32, bool BOXES>
 struct FwdLay {
   static constexpr int M = K / C;
   static constexpr int T = F32 ? 64 : 128;           // samples per feature tile
-  static constexpr int GROUP = fwd_group(F32);       // samples per group, at most
+  static constexpr int GROUP = fwd_group(F32, BOXES);   // samples per group, at most
   static constexpr int YP = K + 4, HP = 64 + 4;      // row pitches of the float32 tiles (floats)
   static constexpr int W1 = 0;                       // [64][K] bf16 swizzled, or [64][YP] f32
   static constexpr int W2 = W1 + (F32 ? 64 * YP * 4 : 64 * K * 2);   // [64][64] bf16, or [64][HP] f32
@@ -43,6 +46,7 @@ struct FwdLay {
   static constexpr int BOX = G + M * 48;             // [M] FwdBox
   static constexpr int STG = BOX + M * 16;           // [M] FwdStage
   static constexpr int POOL = (STG + M * 12 + 15) / 16 * 16;   // staged nodes, C float32 each
+  // (without boxes the layout ends at BOX)
 };
 
 // The box of the nodes blo | bn (as sample_box gives them) whose staged nodes start at byte
@@ -97,10 +101,10 @@ __host__ __device__ inline bool sample_box(const float (&lo)[3], const float (&h
   return true;
 }
 
-// A CTA's dynamic shared memory: its share of the SM's (1 KB of it reserved), less the static part.
+// The dynamic shared memory of a CTA with boxes: its share of the SM's (1 KB of it reserved), less the static part.
 inline int fwd_smem(int smem_sm, int K, bool F32) {
   constexpr int kStatic = 1536;
-  return (smem_sm / fwd_ctas(K, F32) - 1024 - kStatic) / 128 * 128;
+  return (smem_sm / fwd_ctas(K, F32, true) - 1024 - kStatic) / 128 * 128;
 }
 
 }  // namespace srn

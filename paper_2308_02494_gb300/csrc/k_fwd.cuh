@@ -1,25 +1,27 @@
 // Forward query f(x) = d(e(x)) (Eq. 1-3 and Sec. 4.1.2), BF16 or float32, for srn_forward, the
-// renderer and the full-volume decode.
+// renderer and the full-volume decode.  Included by one translation unit per feature count
+// and precision, which sets kK and kF32 first.
 //
 // A CTA takes groups of up to 512 neighbouring samples: consecutive points of a brick, a
-// bundle of ray samples (8 x 8 pixels x 8 samples), or a block of voxels, whose
-// coordinates it forms itself, so the renderer and the decode keep no coordinates in
-// memory.  Per group and brick the samples' bounding box, mapped through each grid's
-// Eq. 1, bounds the nodes that the grid can read; boxes that are worth it and fit are
-// staged in shared memory as the float32 values of their nodes.  Then 128 samples at a
-// time: a thread evaluates Eq. 1-2 for one or four samples and four grids (C = 2) before
-// it stores one 16-byte chunk of features (BF16, swizzled) each, and warp w runs the two hidden
-// layers for rows 16w..16w+15 on the tensor cores (m16n8k16, FP32 accumulate) and the
-// 64 -> 1 output layer in FP32.
+// bundle of ray samples, or a block of voxels, whose coordinates it forms itself, so the
+// renderer and the decode keep no coordinates in memory.  Dense views (boxes_pay) stage nodes
+// in shared memory: per group and brick the samples' bounding box, mapped through each grid's
+// Eq. 1, bounds the nodes that the grid can read, and boxes that are worth it and fit are
+// kept as the float32 values of their nodes.  All others read the corners from global memory.
+// Then 128 samples (float32: 64) at a time: a thread evaluates Eq. 1-2 for one to four samples
+// and the grids of eight features (float32 at K = 16: four) before it stores them.  BF16: warp w
+// runs the two hidden layers for rows 16w..16w+15 on the tensor cores (m16n8k16, FP32
+// accumulate) and the 64 -> 1 output layer in FP32; float32: packed FMAs, 32 rows x 16 columns
+// a warp.
 //
-// What bounds it: instruction issue and the shared-memory pipe (55% and 65% busy in a
-// decode).  Reading the corners from global memory took 116 warp instructions per 32
-// (sample, grid) pairs (unpacking BF16 nodes, float-int conversions, clamps) with the L1
-// pipe at 55-59%; staged float32 nodes need no unpacking, one address for eight reads and
-// packed f32x2 blends: 88.  319^3 decode of the paper-scale model 11.65 -> 8.53 ms, frame
-// of 1024^2 x 512 samples 220 -> 143 ms, progressive pass 425 -> 283 us (with the
-// coordinates, the brick sort and the serial compositing taken out of memory).  Float32:
-// 200 003-point query 192 -> 173 us, progressive pass of 20 832 rays 1290 -> 989 us.
+// What bounds it: with boxes, instruction issue and the shared-memory pipe (55% and 65% busy
+// in a decode); without, the L1 pipe.  Reading the corners from global memory takes 116 warp
+// instructions per 32 (sample, grid) pairs (unpacking BF16 nodes, float-int conversions,
+// clamps); staged float32 nodes need no unpacking, one address for eight reads and packed
+// f32x2 blends: 88.  A sample outside a grid reads nothing, by predicated loads: reading, and
+// dropping, some cell took 110.9 us where it takes 102.0 (200003 points in no order, K = 64).
+// Boxes of points in memory did not pay at any density: 1500000 points in order of the
+// paper-scale model took 568 us with them and 470 without, 60000 59 and 46.
 // The blend is rounded as the global read's was, so the features are the same bits.
 #include <algorithm>
 
@@ -41,6 +43,28 @@ __device__ __forceinline__ EncSNode<C> widen(FwdNode<C, F32> v) {   // as C floa
   else return __uint_as_float((uint32_t)v << 16);
 }
 
+// The node at a, or 0.
+__device__ __forceinline__ uint16_t load_if(bool p, const uint16_t* a) {
+  uint16_t v;
+  asm("{.reg .pred q;\n setp.ne.s32 q, %2, 0;\n mov.b16 %0, 0;\n @q ld.global.nc.u16 %0, [%1];}" : "=h"(v) : "l"(a), "r"((int)p));
+  return v;
+}
+__device__ __forceinline__ uint32_t load_if(bool p, const uint32_t* a) {
+  uint32_t v;
+  asm("{.reg .pred q;\n setp.ne.s32 q, %2, 0;\n mov.b32 %0, 0;\n @q ld.global.nc.u32 %0, [%1];}" : "=r"(v) : "l"(a), "r"((int)p));
+  return v;
+}
+__device__ __forceinline__ float load_if(bool p, const float* a) {
+  float v;
+  asm("{.reg .pred q;\n setp.ne.s32 q, %2, 0;\n mov.b32 %0, 0;\n @q ld.global.nc.f32 %0, [%1];}" : "=f"(v) : "l"(a), "r"((int)p));
+  return v;
+}
+__device__ __forceinline__ unsigned long long load_if(bool p, const unsigned long long* a) {
+  unsigned long long v;
+  asm("{.reg .pred q;\n setp.ne.s32 q, %2, 0;\n mov.b64 %0, 0;\n @q ld.global.nc.u64 %0, [%1];}" : "=l"(v) : "l"(a), "r"((int)p));
+  return v;
+}
+
 // Float order as unsigned integer order (for min/max reductions).
 __device__ __forceinline__ uint32_t ord(float v) {
   const uint32_t b = __float_as_uint(v);
@@ -52,16 +76,16 @@ __device__ __forceinline__ float unord(uint32_t o) {
 
 // VIEW: ray samples or voxels, else points in memory.  BOXES: with staged boxes.
 template <int K, int C, bool EVEN, bool F32, bool VIEW, bool BOXES>
-__global__ void __launch_bounds__(NT, fwd_ctas(K, F32))
+__global__ void __launch_bounds__(NT, fwd_ctas(K, F32, BOXES))
 k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> src, float* __restrict__ out,
       uint32_t pool_nodes) {
-  using L = FwdLay<K, C, F32>;
+  using L = FwdLay<K, C, F32, BOXES>;
   using Node = FwdNode<C, F32>;
   constexpr int M = K / C, T = L::T;
   constexpr int CW = F32 && K == 16 ? 4 : 8;   // features per chunk
   constexpr int GPC = CW / C;                // grids per chunk
   constexpr int NCH = K / CW;                // chunks of a feature row
-  constexpr int PP = K < 64 ? 1 : F32 ? 2 : 4;   // samples per thread
+  constexpr int PP = K < 64 || (!BOXES && (F32 || K < 128)) ? 1 : F32 || !BOXES ? 2 : 4;   // samples per thread
   constexpr int NQ = 8 / (T / (32 * PP));    // warps sharing the same samples, each its own chunks
   constexpr uint32_t kNB = 4 * C;            // bytes of a staged node
   extern __shared__ __align__(128) unsigned char sm[];
@@ -79,7 +103,7 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
   const int R = md.R;
   const int GS = src.group;
   if constexpr (!VIEW) {
-    if (tid == 0) build_tile_map(br, GS, tm);
+    if (tid == 0) build_tile_map_log2(br, __ffs(GS) - 1, tm);   // (a power of two: 64-bit divisions took 0.1 us a brick)
     __syncthreads();
   }
   const int total = VIEW ? src.groups : tm.first[br.n];
@@ -390,13 +414,13 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
             return c.in ? f : EncSNode<C>(0);
           };
           auto from_grid = [&](int i, const Place& c) -> EncSNode<C> {
-            // (a sample outside the grid reads, and drops, its first cell: no branch, so that the
-            // reads of several samples and grids are in flight together)
+            // (predicated loads and no branch, so that the reads of several samples and grids are
+            // in flight together; a sample outside the grid reads nothing)
             constexpr uint32_t mb = (uint32_t)kMagicBits;
-            const Node* F0 = Fb + i * gsz + (c.in ? ((c.tz - mb) * R + (c.ty - mb)) * R + (c.tx - mb) : 0u);
+            const Node* F0 = Fb + i * gsz + ((c.tz - mb) * R + (c.ty - mb)) * R + (c.tx - mb);
             const Node* F2 = F0 + (uint32_t)(R * R);
-            const Node n[8] = {__ldg(F0), __ldg(F0 + 1), __ldg(F0 + R), __ldg(F0 + R + 1),
-                               __ldg(F2), __ldg(F2 + 1), __ldg(F2 + R), __ldg(F2 + R + 1)};
+            const Node n[8] = {load_if(c.in, F0), load_if(c.in, F0 + 1), load_if(c.in, F0 + R), load_if(c.in, F0 + R + 1),
+                               load_if(c.in, F2), load_if(c.in, F2 + 1), load_if(c.in, F2 + R), load_if(c.in, F2 + R + 1)};
             EncSNode<C> v[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k) v[k] = widen<C, F32>(n[k]);
@@ -404,7 +428,7 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
             return c.in ? f : EncSNode<C>(0);
           };
           // the features of the chunk's grid j: packed pairs of bf16, or float32
-          uint32_t o[PP][F32 ? CW : 4];
+          uint32_t o[PP][F32 ? CW : CW / 2];
           auto put = [&](int p, int j, EncSNode<C> f) {
             if constexpr (F32 && C == 2) {
               o[p][2 * j] = (uint32_t)f;
@@ -463,8 +487,9 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
 #pragma unroll
                 for (int q = 0; q < CW / 4; ++q) y[q] = make_uint4(o[p][4 * q], o[p][4 * q + 1], o[p][4 * q + 2], o[p][4 * q + 3]);
               } else {
-                *reinterpret_cast<uint4*>(sm + L::Y + swz<K>(pr + 32 * p, 8 * ch)) =
-                    make_uint4(o[p][0], o[p][1], o[p][2], o[p][3]);
+                unsigned char* y = sm + L::Y + swz<K>(pr + 32 * p, CW * ch);
+                if constexpr (CW == 8) *reinterpret_cast<uint4*>(y) = make_uint4(o[p][0], o[p][1], o[p][2], o[p][3]);
+                else *reinterpret_cast<uint2*>(y) = make_uint2(o[p][0], o[p][1]);
               }
             }
           }
@@ -589,44 +614,40 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
   }
 }
 
-template <int K, int C, bool EVEN, bool F32, bool BOXES>
+template <int K, int C, bool EVEN, bool F32, bool VIEW, bool BOXES>
 cudaError_t launch_k(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
-  using Lay = FwdLay<K, C, F32>;
-  const bool view = src.kind != kFwdPoints;
-  auto points = k_fwd<K, C, EVEN, F32, false, BOXES>;
-  auto views = k_fwd<K, C, EVEN, F32, true, BOXES>;
-  const void* kern = view ? (const void*)views : (const void*)points;
-  const int most = fwd_smem(L.smem_sm, K, F32);
-  if (most < Lay::POOL + 64) return cudaErrorInvalidConfiguration;   // room for dropped reads (fwd_box)
-  const int smem = BOXES ? most : Lay::POOL;   // (what is left is L1)
-  const int pool = (smem - Lay::POOL) / (4 * C);
+  using Lay = FwdLay<K, C, F32, BOXES>;
+  auto kern = k_fwd<K, C, EVEN, F32, VIEW, BOXES>;
+  const int smem = BOXES ? fwd_smem(L.smem_sm, K, F32) : Lay::BOX;   // (what is left is L1)
+  if (BOXES && smem < Lay::POOL + 64) return cudaErrorInvalidConfiguration;   // room for dropped reads (fwd_box)
+  const int pool = BOXES ? (smem - Lay::POOL) / (4 * C) : 0;
   cudaError_t e;
   if (smem > (48 << 10) &&
       (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
     return e;
   int total = src.groups;
-  if (src.kind == kFwdPoints) {
+  if (!VIEW) {
     total = 0;
     for (int b = 0; b < br.n; ++b) total += (int)((br.off[b + 1] - br.off[b] + src.group - 1) / src.group);
   }
   if (total == 0) return cudaSuccess;
   FwdSource s = src;
-  const int ctas = fwd_ctas(K, F32) * L.num_sms;
+  const int ctas = fwd_ctas(K, F32, BOXES) * L.num_sms;
   s.run = std::max(1, std::min(4, total / (8 * ctas)));
   const int grid = std::min((total + s.run - 1) / s.run, ctas);
-  if (view) views<<<grid, NT, smem, L.stream>>>(md, br, s, out, (uint32_t)pool);
-  else points<<<grid, NT, smem, L.stream>>>(md, br, s, out, (uint32_t)pool);
+  kern<<<grid, NT, smem, L.stream>>>(md, br, s, out, (uint32_t)pool);
   return cudaGetLastError();
 }
 
-template <int K, int C, bool BOXES>
-cudaError_t launch_b(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
-  return md.R % 2 ? launch_k<K, C, false, kF32, BOXES>(L, md, br, src, out)
-                  : launch_k<K, C, true, kF32, BOXES>(L, md, br, src, out);
+template <int K, int C, bool EVEN>
+cudaError_t launch_e(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
+  if (src.kind == kFwdPoints) return launch_k<K, C, EVEN, kF32, false, false>(L, md, br, src, out);
+  return src.boxes ? launch_k<K, C, EVEN, kF32, true, true>(L, md, br, src, out)
+                   : launch_k<K, C, EVEN, kF32, true, false>(L, md, br, src, out);
 }
 template <int K, int C>
 cudaError_t launch_c(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
-  return src.boxes ? launch_b<K, C, true>(L, md, br, src, out) : launch_b<K, C, false>(L, md, br, src, out);
+  return md.R % 2 ? launch_e<K, C, false>(L, md, br, src, out) : launch_e<K, C, true>(L, md, br, src, out);
 }
 
 }  // namespace
@@ -638,7 +659,7 @@ cudaError_t launch_forward_k<kK, kF32>(const Launch& L, const Model& md, const B
 }
 template <>
 int forward_nodes_k<kK, kF32>(const Launch& L, const Model& md) {
-  const int at = md.C == 2 ? FwdLay<kK, 2, kF32>::POOL : FwdLay<kK, 1, kF32>::POOL;
+  const int at = md.C == 2 ? FwdLay<kK, 2, kF32, true>::POOL : FwdLay<kK, 1, kF32, true>::POOL;
   return (fwd_smem(L.smem_sm, kK, kF32) - at) / (4 * kK);
 }
 

@@ -121,13 +121,13 @@ cudaError_t launch_render_batch(const Launch& L, const RenderParams& rp, float* 
     const float e = cbrtf((float)n * rp.cell) * 0.5f * (float)(md.R - 1) * 1.15f + 2.f;
     return e * e * e;
   };
-  src.group = fwd_group(!md.F16);
+  src.group = fwd_group(!md.F16, true);
   while (src.group > least &&
          (slots < (int64_t)src.group * 2 * L.num_sms || nodes(src.group) > (float)room))
     src.group /= 2;
   src.boxes = nodes(src.group) <= 2.f * (float)room;
   if (!src.boxes) {
-    src.group = fwd_group(!md.F16);
+    src.group = fwd_group(!md.F16, false);
     while (src.group > least && slots < (int64_t)src.group * 2 * L.num_sms) src.group /= 2;
   }
   src.groups = (int)((slots + src.group - 1) / src.group);
@@ -168,7 +168,7 @@ cudaError_t launch_decode(const Launch& L, const RenderParams& rp, const Model& 
   // Blocks of at most `cap` voxels: as large as they go while there are a few for every CTA,
   // and of the shape with the fewest tiles of samples over the bricks, compact ones first.
   const int tile = md.F16 ? 128 : 64;   // (the kernel's)
-  int cap = fwd_group(!md.F16);
+  int cap = fwd_group(!md.F16, true);
   while (cap > tile && voxels / cap < 8 * (int64_t)L.num_sms) cap /= 2;
   double best = 0.0;
   for (int x = 1; x <= std::min(16, n[0]); ++x)

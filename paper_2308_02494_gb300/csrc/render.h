@@ -179,12 +179,12 @@ __device__ __forceinline__ void decode_voxel(const FwdBlock& k, int s, int (&v)[
 // Where the forward query takes its samples from, in groups of `group` (a multiple of the
 // kernel's tile, 128 or, in float32, 64, at most fwd_group()) neighbouring ones.
 enum FwdKind { kFwdPoints = 0, kFwdRender = 1, kFwdDecode = 2 };
-constexpr int fwd_group(bool f32) { return f32 ? 256 : 512; }
+constexpr int fwd_group(bool f32, bool boxes) { return f32 || !boxes ? 256 : 512; }
 struct FwdPointSource {   // what a kernel over points in memory gets (the rest is 2 KB of arguments)
   int32_t kind;
   int32_t group, groups;   // (kFwdPoints counts its groups per brick itself)
   int32_t run;             // consecutive groups of a CTA (set by the launch)
-  int32_t boxes;           // 0: read every corner from global memory
+  int32_t boxes;           // 0 (always for points in memory): read every corner from global memory
   const float* xyz;        // kFwdPoints, and their sorted copy, if one was made
   SortedBatch sorted;
 };
@@ -197,7 +197,6 @@ struct FwdSource : FwdPointSource {
 inline FwdSource point_source(const Launch& L, const Bricks& br, const float* xyz, bool f32) {
   FwdSource s{};
   s.kind = kFwdPoints;
-  s.boxes = 0;   // (set for batches that are, or are brought, in order: boxes of random points are the whole grids)
   s.group = 256;
   while (s.group > (f32 ? 64 : 128) && br.off[br.n] < (int64_t)s.group * 4 * L.num_sms) s.group /= 2;
   s.xyz = xyz;

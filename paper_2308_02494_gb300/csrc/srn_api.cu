@@ -93,7 +93,7 @@ WsLayout ws_layout(const srn_config* c, int64_t maxp) {
   WsLayout w{};
   size_t o = 0;
   w.state = o; o += align256(sizeof(srn::StepState) + 64);
-  const size_t hist = align256(sizeof(uint32_t) * ((size_t)srn::kSortBins * c->n_bricks + 1));   // and `moved`
+  const size_t hist = align256(sizeof(uint32_t) * ((size_t)srn::kSortBins * c->n_bricks + 2));   // and `moved`
   // (from here to rsum's end: cleared by every backward pass)
   w.ustart = o; o += c->precision == SRN_BF16 ? align256(sizeof(int32_t) * (srn::kUnits + 1) * c->n_bricks) : 0;
   w.t_hist = o; o += hist;
@@ -185,6 +185,7 @@ struct srn_handle {
   // handle's one sorted copy in turn (query_done: the last one has read it)
   std::mutex query_mu;
   cudaEvent_t query_done = nullptr;
+  uint32_t query_turn = 0;   // how many have sorted, or looked whether to
   // launch shape of the BF16 training pass (srn_set_tuning / srn_autotune)
   srn::Tuning tune = srn::kDefaultTuning;
 
@@ -229,6 +230,11 @@ struct srn_handle {
     s.rank = reinterpret_cast<uint32_t*>(ws + (query ? wl.q_rank : wl.t_rank));
     s.hist = reinterpret_cast<uint32_t*>(ws + (query ? wl.q_hist : wl.t_hist));
     s.moved = s.hist + (size_t)srn::kSortBins * cfg.n_bricks;
+    s.next = nullptr;
+    if (query) {   // each call counts in one word, and clears the next call's
+      s.next = s.moved + ((query_turn + 1) & 1);
+      s.moved += query_turn & 1;
+    }
     return s;
   }
   srn::Model model() const {
@@ -295,13 +301,16 @@ cudaError_t forward_points(srn_handle* h, const srn::Launch& L, const srn::Model
                          const float* xyz, float* out) {
   srn::FwdSource src = srn::point_source(L, br, xyz, !md.F16);
   const int64_t n = br.off[br.n];
-  // A sorted copy costs about 20 us and 0.05 ns per point, and pays where the brick's grids are
-  // well beyond L1, the sooner the larger they are (random points, with it and without, in us.
-  // BF16, 8.4 MB of features: 32768 points 55 and 48, 65536 73 and 80, 524288 292 and 520;
-  // 1 MB: 131072 68 and 63, 262144 99 and 119; 256 KB: 524288 114 and 109.  Float32, 17 MB:
-  // 65536 109 and 118; 2 MB: 131072 107 and 115; 512 KB: 262144 142 and 142).
+  // A sorted copy costs about 16 us and 0.05 ns per point, and looking whether the points need
+  // one 6 us.  It pays where the brick's grids are well beyond L1, the sooner the larger they are
+  // (random points, with it and without, in us.  BF16, 8.4 MB of features: 20000 points 47 and
+  // 50, 60000 66 and 96, 500000 223 and 625; 1 MB: 60000 38 and 38, 100000 44 and 55; 256 KB:
+  // 200003 56 and 51.  Float32, 17 MB: 20000 61 and 57, 60000 101 and 127; 2 MB: 60000 65 and
+  // 64, 100000 92 and 105; 512 KB: 130000 87 and 85).  Points in order gain nothing and pay for
+  // the look, so the line lies somewhat above (BF16, 8.4 MB, points in order, with the look and
+  // without: 70000 53 and 50, 100000 65 and 59).
   const double bytes = (double)md.M * md.R * md.R * md.R * md.C * (md.F16 ? 2 : 4);
-  const int64_t least = bytes >= 400e3 ? (int64_t)(1.68e8 / sqrt(bytes)) : INT64_MAX;
+  const int64_t least = bytes >= 400e3 ? (int64_t)(3.4e6 / pow(bytes, 0.25)) : INT64_MAX;
   if (n < least || n > UINT32_MAX) return srn::launch_forward(L, md, br, src, out);
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(L.stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
@@ -311,10 +320,10 @@ cudaError_t forward_points(srn_handle* h, const srn::Launch& L, const srn::Model
   std::lock_guard<std::mutex> lock(h->query_mu);
   cudaError_t e = cudaStreamWaitEvent(L.stream, h->query_done, 0);   // (no-op before the first record)
   if (e != cudaSuccess) return e;
-  src.boxes = 1;
   src.sorted = h->sort_scratch(true);
   src.sorted.limit = (uint32_t)(n / 32);   // scan lines and other nearly sorted batches stay as they are
   if ((e = srn::launch_sort_query(L, br, xyz, src.sorted)) != cudaSuccess) return e;
+  ++h->query_turn;
   if ((e = srn::launch_forward(L, md, br, src, out)) != cudaSuccess) return e;
   return cudaEventRecord(h->query_done, L.stream);
 }
@@ -541,6 +550,7 @@ srn_status srn_create(const srn_config* cfg, const srn_tensors* t, void* workspa
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   if (e != cudaSuccess) return cuda_fail(e, "device query");
   e = cudaMemset(static_cast<unsigned char*>(workspace) + wl.state, 0, wl.ustart - wl.state);
+  if (e == cudaSuccess) e = cudaMemset(static_cast<unsigned char*>(workspace) + wl.q_hist, 0, wl.total - wl.q_hist);
   if (e != cudaSuccess) return cuda_fail(e, "workspace init");
   srn_handle* h = new srn_handle();
   h->cfg = *cfg;
@@ -1046,7 +1056,7 @@ srn_status render_pixels(srn_handle* h, void* stream, const srn::RenderParams& r
   // rows of the progressive order's last level (at most 16), samples `dt` apart along chords
   // of about 2.
   srn::RenderParams rp = rpi;
-  const int full = srn::fwd_group(h->cfg.precision != SRN_BF16);
+  const int full = srn::fwd_group(h->cfg.precision != SRN_BF16, true);
   const float* eye = rp.cam.eye;
   const float far = rp.cam.ortho ? 1.f : std::max(0.1f, sqrtf(eye[0] * eye[0] + eye[1] * eye[1] + eye[2] * eye[2]));
   const float stride = rp.order ? sqrtf((float)rp.width * (float)rp.height / (float)std::max<int64_t>(1, first + count)) : 1.f;

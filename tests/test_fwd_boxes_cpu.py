@@ -16,7 +16,7 @@ using namespace srn;
 template <int K, int C, bool F32>
 int check() {
   const int smem = fwd_smem(233472, K, F32);   // an SM has 228 KB
-  const uint32_t pool = (uint32_t)(smem - FwdLay<K, C, F32>::POOL) / (4 * C) * (4 * C);
+  const uint32_t pool = (uint32_t)(smem - FwdLay<K, C, F32, true>::POOL) / (4 * C) * (4 * C);
   int bad = 0;
   for (int R = 2; R <= 64; ++R)
     for (int miss = 0; miss < 8; ++miss)
