@@ -200,8 +200,9 @@ srn_status srn_sample_target_tiled(srn_handle* h, void* stream, const float* til
 /* Forward query f(x) = d(e(x)) (Eq. 1-3 and Sec. 4.1.2) of every brick's points:
  * out_dev[n] for xyz_dev[n].  offsets as in srn_sample_points.  A large batch whose points
  * are in no spatial order is evaluated through a sorted copy in the workspace (the results
- * are the same bits); calls on several streams or threads take that copy in turn, and a
- * call on a stream that is being captured does without. */
+ * are the same bits).  Calls may come from several threads and overlap on several streams:
+ * while one stream's call is at that copy, another stream's does without it, as does a call
+ * on a stream that is being captured. */
 srn_status srn_forward(srn_handle* h, void* stream, const float* xyz_dev,
                        const int64_t* offsets, float* out_dev);
 
@@ -337,8 +338,7 @@ srn_status srn_load_state(srn_handle* h, void* stream, const void* src, size_t b
  * to brick min(floor(n i / (vox - 1)), n - 1) of the grid[3] = (I, J, K) bricks (the
  * Sec. 5.3 hash at that position), and is queried in that brick's local [-1, 1]^3
  * given by boxes[B][6] (lo xyz, hi xyz voxels, as in srn_render).  out_dev receives
- * [vox][vox][vox] float32, z slowest.  Batches of at most max_points voxels; FP32 or
- * BF16 as the handle. */
+ * [vox][vox][vox] float32, z slowest.  FP32 or BF16 as the handle. */
 srn_status srn_decode(srn_handle* h, void* stream, const int32_t grid[3], const int64_t* boxes, int64_t vox,
                       float* out_dev);
 

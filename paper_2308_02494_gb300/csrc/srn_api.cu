@@ -181,11 +181,13 @@ struct srn_handle {
   // set by the training step around its backward pass: the batch is the sampler's, whose
   // histogram holds the bin starts the BF16 tile list needs
   const uint32_t* batch_bins = nullptr;
-  // srn_forward calls may come from several threads and streams: those that sort take the
-  // handle's one sorted copy in turn (query_done: the last one has read it)
+  // srn_forward calls may come from several threads and streams: the handle's one sorted copy
+  // is a call's if no other stream's is at it (query_done: the last one has read it), and the
+  // others do without
   std::mutex query_mu;
   cudaEvent_t query_done = nullptr;
-  uint32_t query_turn = 0;   // how many have sorted, or looked whether to
+  cudaStream_t query_stream = nullptr;
+  uint64_t query_turn = 0;   // how many have sorted, or looked whether to
   // launch shape of the BF16 training pass (srn_set_tuning / srn_autotune)
   srn::Tuning tune = srn::kDefaultTuning;
 
@@ -318,14 +320,29 @@ cudaError_t forward_points(srn_handle* h, const srn::Launch& L, const srn::Model
     return srn::launch_forward(L, md, br, src, out);
   }
   std::lock_guard<std::mutex> lock(h->query_mu);
-  cudaError_t e = cudaStreamWaitEvent(L.stream, h->query_done, 0);   // (no-op before the first record)
+  if (h->query_turn && h->query_stream != L.stream) {
+    // (relaxed: the question must not end a capture that another thread has begun)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const bool busy = cudaEventQuery(h->query_done) != cudaSuccess;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (busy) {
+      cudaGetLastError();
+      return srn::launch_forward(L, md, br, src, out);
+    }
+  }
+  // (the same stream's calls are in order anyway; the wait is for a handle that named another
+  // stream before: a stream destroyed since, or another thread's per-thread default stream)
+  cudaError_t e = h->query_turn ? cudaStreamWaitEvent(L.stream, h->query_done, 0) : cudaSuccess;
   if (e != cudaSuccess) return e;
   src.sorted = h->sort_scratch(true);
   src.sorted.limit = (uint32_t)(n / 32);   // scan lines and other nearly sorted batches stay as they are
   if ((e = srn::launch_sort_query(L, br, xyz, src.sorted)) != cudaSuccess) return e;
   ++h->query_turn;
-  if ((e = srn::launch_forward(L, md, br, src, out)) != cudaSuccess) return e;
-  return cudaEventRecord(h->query_done, L.stream);
+  h->query_stream = L.stream;
+  e = srn::launch_forward(L, md, br, src, out);
+  const cudaError_t r = cudaEventRecord(h->query_done, L.stream);   // (also where the launch failed: the sort runs)
+  return e != cudaSuccess ? e : r;
 }
 
 srn_status run_query(srn_handle* h, void* stream, srn::QueryMode mode, const srn::Bricks& br,

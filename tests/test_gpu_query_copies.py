@@ -62,3 +62,27 @@ def test_sorted_copy_gives_the_same_bits(shape, precision, n_bricks):
     torch.cuda.synchronize()
     assert torch.equal(out, want)
 
+
+@pytest.mark.parametrize("precision", ["bf16", "fp32"])
+def test_a_query_does_not_wait_for_another_streams(precision):
+    """Work that one stream has queued before its query holds that query, not another stream's."""
+    import torch
+
+    ensure_built()
+    n = 200_003
+    net = _model((32, 20, 2), 1, n, precision)
+    x = [torch.rand((n, 3), device="cuda") * 2 - 1 for _ in range(2)]
+    want = [net.forward(v, [0, n]).clone() for v in x]
+    out = [torch.zeros(n, device="cuda") for _ in range(2)]
+    torch.cuda.synchronize()
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    with torch.cuda.stream(a):
+        torch.cuda._sleep(400_000_000)   # about 0.2 s
+    net.forward(x[0], [0, n], out=out[0], stream=a)
+    done = torch.cuda.Event()
+    done.record(a)
+    net.forward(x[1], [0, n], out=out[1], stream=b)
+    b.synchronize()
+    assert not done.query()
+    torch.cuda.synchronize()
+    assert torch.equal(out[0], want[0]) and torch.equal(out[1], want[1])
