@@ -501,7 +501,8 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
           if (w < 0) return;
           f = fmaf(f, s_range[1], s_range[0]);
           if constexpr (VIEW) out[render ? base() + s : decode_index(src, blk, s)] = f;
-          else out[copied ? (int64_t)src.sorted.index[base() + s] : base() + s] = f;
+          else if (!copied) out[base() + s] = f;
+          else if (const int64_t at = src.sorted.index[base() + s]; at < br.off[br.n]) out[at] = f;   // (sort_scatter)
         };
         if constexpr (F32) {
           // ---- decoder in float32: warp w takes 32 rows x 16 columns of a hidden layer, lane

@@ -85,14 +85,16 @@ __device__ __forceinline__ void sort_count(const Bricks& br, const float* __rest
     if (in) s.rank[gi] = r + __popc(grp & ((1u << lane) - 1u));
   }
 }
-// The sorted copy (after the scan).
+// The sorted copy (after the scan).  (Points that another stream is writing meanwhile may have
+// another bin than they were counted in: their places stay within their brick.)
 __device__ __forceinline__ void sort_scatter(const Bricks& br, const float* __restrict__ xyz,
                                              const float* __restrict__ target, const SortedBatch& s) {
   const int64_t total = br.off[br.n];
   for (int64_t gi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gi < total; gi += (int64_t)gridDim.x * blockDim.x) {
     const int b = brick_of_point(br, gi);
     const float x = xyz[3 * gi], y = xyz[3 * gi + 1], z = xyz[3 * gi + 2];
-    const int64_t dst = br.off[b] + s.hist[(int64_t)b * kSortBins + morton_bin(x, y, z)] + s.rank[gi];
+    const int64_t dst = min(br.off[b] + (int64_t)s.hist[(int64_t)b * kSortBins + morton_bin(x, y, z)] + s.rank[gi],
+                            br.off[b + 1] - 1);
     s.xyz[3 * dst] = x; s.xyz[3 * dst + 1] = y; s.xyz[3 * dst + 2] = z;
     if (s.target) s.target[dst] = target[gi];
     if (s.index) s.index[dst] = (uint32_t)gi;

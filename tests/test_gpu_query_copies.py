@@ -86,3 +86,28 @@ def test_a_query_does_not_wait_for_another_streams(precision):
     assert not done.query()
     torch.cuda.synchronize()
     assert torch.equal(out[0], want[0]) and torch.equal(out[1], want[1])
+
+
+@pytest.mark.parametrize("n_bricks", [1, 3])
+def test_points_written_during_a_query_cost_only_their_values(n_bricks):
+    """Points that another stream overwrites while they are being sorted may come out as anything,
+    but nothing beyond the batch's outputs is written."""
+    import torch
+
+    ensure_built()
+    n, most = 200_003, 400_000
+    net = _model((32, 20, 2), n_bricks, most, "bf16")
+    big = torch.rand((most, 3), device="cuda") * 2 - 1
+    net.forward(big, [0] + [most * (b + 1) // n_bricks for b in range(n_bricks)])   # places beyond n, from before
+    x = big[:n].clone()
+    other = torch.rand((n, 3), device="cuda") * 2 - 1
+    out = torch.full((n + 2 * 65536,), 7.5, device="cuda")
+    off = [0] + [n * (b + 1) // n_bricks for b in range(n_bricks)]
+    torch.cuda.synchronize()
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    for k in range(40):
+        with torch.cuda.stream(b):
+            x.copy_(other if k % 2 else big[:n])
+        net.forward(x, off, out=out[65536:65536 + n], stream=a)
+    torch.cuda.synchronize()
+    assert bool((out[:65536] == 7.5).all()) and bool((out[65536 + n:] == 7.5).all())
