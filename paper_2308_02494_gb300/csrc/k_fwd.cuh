@@ -93,6 +93,7 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
   __shared__ Bricks br;
   __shared__ uint32_t s_lo[3], s_hi[3], s_mask[2], s_np;
   __shared__ float s_range[2];            // the brick's minimum and span
+  __shared__ int s_run[2];                // the next run of groups
   __shared__ FwdBlock blk;                // the group's voxels (kFwdDecode)
   __shared__ uint16_t s_cnt[L::GROUP / 32];   // a mixed group's samples of a brick in each 32 slots,
   __shared__ uint16_t s_first[SRN_MAX_BRICKS], s_end;   // where its bricks' samples start, and the last one's end
@@ -122,10 +123,14 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
   const float ct = hs - 0.5f + kMagic;   // an integer when R is even (axis_cell)
 
   int cur = -1, hint = -1;
-  // runs of src.run consecutive groups, dealt round robin to the CTAs: neighbouring groups
-  // share a brick (and its weights), and a frame's empty corners are spread over the CTAs
-  for (int r0 = blockIdx.x * src.run; r0 < total; r0 += gridDim.x * src.run) {
-  const int r1 = min(total, r0 + src.run);
+  // Runs of src.run consecutive groups (they share a brick and its weights): one for every CTA,
+  // and then in turn, or where the groups differ as CTAs are done (src.next; the next run is
+  // taken one ahead).  Dealt in turn, the rows of a view's groups could divide the CTAs evenly,
+  // and some had the volume's middle in every round and others its empty sides (a progressive
+  // pass with a third of its rays on the volume: 473 us, and 293 taken as they come).
+  for (int r = blockIdx.x, k = 0; r * src.run < total; ++k) {
+  if (VIEW && src.next && tid == 0) s_run[k & 1] = (int)gridDim.x + atomicAdd(src.next, 1);
+  const int r0 = r * src.run, r1 = min(total, r0 + src.run);
   for (int grp = r0; grp < r1; ++grp) {
     // ---- the group's samples: coordinates and brick (-1: no sample)
     if (tid < 2) s_mask[tid] = 0u;
@@ -612,6 +617,8 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
       }
     }
   }
+  // (a group has a barrier at least, so s_run[k & 1] is not written again before it is read)
+  r = VIEW && src.next ? s_run[k & 1] : r + (int)gridDim.x;
   }
 }
 
@@ -657,11 +664,6 @@ template <>
 cudaError_t launch_forward_k<kK, kF32>(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src,
                                        float* out) {
   return md.C == 2 ? launch_c<kK, 2>(L, md, br, src, out) : launch_c<kK, 1>(L, md, br, src, out);
-}
-template <>
-int forward_nodes_k<kK, kF32>(const Launch& L, const Model& md) {
-  const int at = md.C == 2 ? FwdLay<kK, 2, kF32, true>::POOL : FwdLay<kK, 1, kF32, true>::POOL;
-  return (fwd_smem(L.smem_sm, kK, kF32) - at) / (4 * kK);
 }
 
 }  // namespace srn

@@ -31,7 +31,8 @@ __device__ __forceinline__ int order_of(const RenderParams& rp, int x, int y) {
 constexpr int kSegs = 8;
 __global__ void __launch_bounds__(32 * kSegs)
 k_render_composite(RenderParams rp, int pix0, int npix, const float* __restrict__ val,
-                   const float* __restrict__ lut, float* __restrict__ rgba) {
+                   const float* __restrict__ lut, float* __restrict__ rgba, int32_t* __restrict__ next) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *next = 0;   // for the next batch's groups
   __shared__ float4 part[kSegs][32];
   const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
   const int ray = blockIdx.x * 32 + lane;
@@ -106,37 +107,34 @@ __global__ void k_render_preview(RenderParams rp, int done, int level, const flo
 
 }  // namespace
 
-cudaError_t launch_render_batch(const Launch& L, const RenderParams& rp, float* val, int pix0, int npix,
+bool boxes_pay(const Model& md, int group, float x, float y, float z) {
+  const float cells = 0.5f * (float)(md.R - 1) * 1.15f, e = cbrtf((float)group);
+  const float nodes = (e * x * cells + 2.f) * (e * y * cells + 2.f) * (e * z * cells + 2.f);
+  return nodes * (md.F16 ? 8.f : 16.f) <= (float)group;
+}
+
+cudaError_t launch_render_batch(const Launch& L, const RenderParams& rp, float* val, int32_t* next, int pix0, int npix,
                                 const Model& md, const float* lut, float* rgba) {
   Bricks br{};
   br.n = rp.grid[0] * rp.grid[1] * rp.grid[2];
   FwdSource src{};
   src.kind = kFwdRender;
-  // Groups as large as they go while there is one for every CTA and a group's nodes in a grid
-  // (a cube of its samples' volume, the grids' 15% zoom, a partial cell and a node at either
-  // end) have room; where not even the smallest group's do, the corners come from L1 instead.
+  // Groups as large as they go while there are two for every SM; a group is about a cube.
   const int64_t slots = render_slots(rp, npix);
-  const int least = md.F16 ? 128 : 64, room = forward_box_nodes(L, md);
-  auto nodes = [&](int n) {
-    const float e = cbrtf((float)n * rp.cell) * 0.5f * (float)(md.R - 1) * 1.15f + 2.f;
-    return e * e * e;
-  };
+  const int least = md.F16 ? 128 : 64;
+  const float edge = cbrtf(rp.cell);
   src.group = fwd_group(!md.F16, true);
-  while (src.group > least &&
-         (slots < (int64_t)src.group * 2 * L.num_sms || nodes(src.group) > (float)room))
-    src.group /= 2;
-  src.boxes = nodes(src.group) <= 2.f * (float)room;
-  if (!src.boxes) {
-    src.group = fwd_group(!md.F16, false);
-    while (src.group > least && slots < (int64_t)src.group * 2 * L.num_sms) src.group /= 2;
-  }
+  while (src.group > least && slots < (int64_t)src.group * 2 * L.num_sms) src.group /= 2;
+  src.boxes = boxes_pay(md, src.group, edge, edge, edge);
+  if (!src.boxes) src.group = std::min(src.group, fwd_group(!md.F16, false));
   src.groups = (int)((slots + src.group - 1) / src.group);
+  src.next = next;
   src.pix0 = pix0;
   src.npix = npix;
   src.rp = rp;
   const cudaError_t e = launch_forward(L, md, br, src, val);
   if (e != cudaSuccess) return e;
-  k_render_composite<<<(npix + 31) / 32, 32 * kSegs, 0, L.stream>>>(rp, pix0, npix, val, lut, rgba);
+  k_render_composite<<<(npix + 31) / 32, 32 * kSegs, 0, L.stream>>>(rp, pix0, npix, val, lut, rgba, next);
   return cudaGetLastError();
 }
 
@@ -151,7 +149,6 @@ cudaError_t launch_render_preview(const Launch& L, const RenderParams& rp, int d
 cudaError_t launch_decode(const Launch& L, const RenderParams& rp, const Model& md, float* out) {
   FwdSource src{};
   src.kind = kFwdDecode;
-  src.boxes = 1;
   src.rp = rp;
   src.dec.vox = rp.vox;
   int n[3], nb = 1;
@@ -170,6 +167,8 @@ cudaError_t launch_decode(const Launch& L, const RenderParams& rp, const Model& 
   const int tile = md.F16 ? 128 : 64;   // (the kernel's)
   int cap = fwd_group(!md.F16, true);
   while (cap > tile && voxels / cap < 8 * (int64_t)L.num_sms) cap /= 2;
+  src.boxes = boxes_pay(md, cap, 2.f / (float)n[0], 2.f / (float)n[1], 2.f / (float)n[2]);
+  if (!src.boxes) cap = std::min(cap, fwd_group(!md.F16, false));
   double best = 0.0;
   for (int x = 1; x <= std::min(16, n[0]); ++x)
     for (int y = 1; y <= std::min(16, n[1]); ++y)

@@ -184,6 +184,7 @@ struct FwdPointSource {   // what a kernel over points in memory gets (the rest 
   int32_t kind;
   int32_t group, groups;   // (kFwdPoints counts its groups per brick itself)
   int32_t run;             // consecutive groups of a CTA (set by the launch)
+  int32_t* next;           // kFwdRender: zero; runs of groups taken beyond the CTAs' first
   int32_t boxes;           // 0 (always for points in memory): read every corner from global memory
   const float* xyz;        // kFwdPoints, and their sorted copy, if one was made
   SortedBatch sorted;
@@ -225,14 +226,9 @@ __device__ __forceinline__ int64_t decode_index(const FwdSource& src, const FwdB
 // (One translation unit per feature count K and precision.)
 template <int K, bool F32>
 cudaError_t launch_forward_k(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out);
-// Staged nodes per grid that a CTA of the forward kernel has room for.
-template <int K, bool F32>
-int forward_nodes_k(const Launch& L, const Model& md);
 #define SRN_FWD(K, F32)                                                                            \
   template <>                                                                                      \
-  cudaError_t launch_forward_k<K, F32>(const Launch&, const Model&, const Bricks&, const FwdSource&, float*); \
-  template <>                                                                                      \
-  int forward_nodes_k<K, F32>(const Launch&, const Model&);
+  cudaError_t launch_forward_k<K, F32>(const Launch&, const Model&, const Bricks&, const FwdSource&, float*);
 SRN_FWD(16, false) SRN_FWD(32, false) SRN_FWD(64, false) SRN_FWD(128, false)
 SRN_FWD(16, true) SRN_FWD(32, true) SRN_FWD(64, true) SRN_FWD(128, true)
 #undef SRN_FWD
@@ -246,18 +242,20 @@ inline cudaError_t launch_forward(const Launch& L, const Model& md, const Bricks
     default: return cudaErrorInvalidValue;
   }
 }
-inline int forward_box_nodes(const Launch& L, const Model& md) {
-  const bool f32 = !md.F16;
-  switch (md.K) {
-    case 16: return f32 ? forward_nodes_k<16, true>(L, md) : forward_nodes_k<16, false>(L, md);
-    case 32: return f32 ? forward_nodes_k<32, true>(L, md) : forward_nodes_k<32, false>(L, md);
-    case 64: return f32 ? forward_nodes_k<64, true>(L, md) : forward_nodes_k<64, false>(L, md);
-    default: return f32 ? forward_nodes_k<128, true>(L, md) : forward_nodes_k<128, false>(L, md);
-  }
-}
 
-// Rays pix0 .. pix0 + npix - 1 of rp's order; val: [max_points] scratch for their samples' values.
-cudaError_t launch_render_batch(const Launch& L, const RenderParams& rp, float* val, int pix0, int npix,
+// Whether staged boxes pay for groups of `group` of a brick's samples, x, y and z apart in its
+// coordinates: a cube's nodes in a grid are those of its extent in cells (the maps are on the
+// device: they are taken to zoom by 15%), a partial cell and a node at either end, and a node
+// should serve eight samples or more, sixteen in float32.  With boxes and without, in us, at
+// samples per node by this count: BF16, 64 grids, 11 (frame of 512^2 x 256 rays through 8 bricks)
+// 20300 and 23600, 6.6 (progressive pass of 9000 x 256) 967 and 925, 2.9 (the same, 4 bricks)
+// 1475 and 1059; 32 grids, 13 460 and 459; 16 grids, 14 (14400 x 256) 258 and 283.  Float32, 64
+// grids, 7 (frame of 160^2 x 320) 7036 and 7548, 2.6 (8 bricks) 10780 and 8910; 16 grids of 9^3,
+// 20 2805 and 2600.
+bool boxes_pay(const Model& md, int group, float x, float y, float z);
+// Rays pix0 .. pix0 + npix - 1 of rp's order; val: [max_points] scratch for their samples'
+// values, next: a counter that is zero, and again after a batch whose launches succeed.
+cudaError_t launch_render_batch(const Launch& L, const RenderParams& rp, float* val, int32_t* next, int pix0, int npix,
                                 const Model& md, const float* lut, float* rgba);
 // In-progress image after `done` pixels of the progressive order; `level` is the finest
 // complete hierarchy level (ignored when done = 0).

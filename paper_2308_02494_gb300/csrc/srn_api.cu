@@ -85,7 +85,7 @@ void make_layout(const srn_config* c, srn_layout* L) {
 struct WsLayout {
   size_t state, acc, gsum, rsum, rho, herr, sort_rank, sort_hist, feat, dfeat, gmax, ustart, tiles, tile_ctr;
   size_t sched, sring;
-  size_t r_val, total;
+  size_t r_val, r_next, total;
   size_t t_xyz, t_target, t_rank, t_hist, q_xyz, q_index, q_rank, q_hist;
 };
 
@@ -120,6 +120,7 @@ WsLayout ws_layout(const srn_config* c, int64_t maxp) {
   w.sched = o; o += align256(sizeof(srn::BrickSched) * c->n_bricks);
   w.sring = o; o += align256(sizeof(double) * 2 * srn::kMaxDensityWindow * c->n_bricks);
   w.r_val = o; o += align256(sizeof(float) * maxp);   // values of a render batch's samples
+  w.r_next = o; o += align256(sizeof(int32_t));
   // sorted copies of a batch in memory: one of the training pass, one of the queries
   w.t_xyz = o; o += align256(sizeof(float) * 3 * maxp);
   w.t_target = o; o += align256(sizeof(float) * maxp);
@@ -186,6 +187,7 @@ struct srn_handle {
   // others do without
   std::mutex query_mu;
   cudaEvent_t query_done = nullptr;
+  bool render_failed = false;   // a render batch's launches did: its counter may not be zero
   cudaStream_t query_stream = nullptr;
   uint64_t query_turn = 0;   // how many have sorted, or looked whether to
   // launch shape of the BF16 training pass (srn_set_tuning / srn_autotune)
@@ -568,6 +570,7 @@ srn_status srn_create(const srn_config* cfg, const srn_tensors* t, void* workspa
   if (e != cudaSuccess) return cuda_fail(e, "device query");
   e = cudaMemset(static_cast<unsigned char*>(workspace) + wl.state, 0, wl.ustart - wl.state);
   if (e == cudaSuccess) e = cudaMemset(static_cast<unsigned char*>(workspace) + wl.q_hist, 0, wl.total - wl.q_hist);
+  if (e == cudaSuccess) e = cudaMemset(static_cast<unsigned char*>(workspace) + wl.r_next, 0, sizeof(int32_t));
   if (e != cudaSuccess) return cuda_fail(e, "workspace init");
   srn_handle* h = new srn_handle();
   h->cfg = *cfg;
@@ -1068,33 +1071,40 @@ srn_status render_params(srn_handle* h, const srn_camera* cam, const float* lut,
 srn_status render_pixels(srn_handle* h, void* stream, const srn::RenderParams& rpi, const float* lut,
                          int64_t first, int64_t count, float* rgba) {
   float* val = reinterpret_cast<float*>(h->ws + h->wl.r_val);
-  // Ray groups, so that a query group of `full` samples (rg rays x full / rg samples) is about
-  // as deep as it is wide: rays `px` apart, in blocks of the raster order (at most 64) or in
-  // rows of the progressive order's last level (at most 16), samples `dt` apart along chords
-  // of about 2.
+  int32_t* next = reinterpret_cast<int32_t*>(h->ws + h->wl.r_next);
+  // Ray groups, so that `full` samples (rg rays x full / rg samples), a query group with staged
+  // boxes or a feature tile without, are about as deep as they are wide: rays `px` apart, in
+  // blocks of the raster order (at most 64) or in rows of the progressive order's last level (at
+  // most 16), samples `dt` apart along chords of about 2.
   srn::RenderParams rp = rpi;
-  const int full = srn::fwd_group(h->cfg.precision != SRN_BF16, true);
+  const srn::Model md = h->model();
+  const bool f32 = h->cfg.precision != SRN_BF16;
   const float* eye = rp.cam.eye;
   const float far = rp.cam.ortho ? 1.f : std::max(0.1f, sqrtf(eye[0] * eye[0] + eye[1] * eye[1] + eye[2] * eye[2]));
   const float stride = rp.order ? sqrtf((float)rp.width * (float)rp.height / (float)std::max<int64_t>(1, first + count)) : 1.f;
   const float px = std::max(1e-6f, 2.f * fabsf(rp.cam.scale) * far / (float)rp.height * std::max(1.f, stride));
-  const float dt = 2.f / (float)rp.samples, ratio = (float)full * dt / px;
-  const float want = rp.order ? sqrtf(ratio) : powf(ratio, 2.f / 3.f);
+  const float dt = 2.f / (float)rp.samples;
+  rp.cell = px * px * dt * (float)(rp.grid[0] * rp.grid[1] * rp.grid[2]);
+  const float edge = cbrtf(rp.cell);
+  const int full = srn::boxes_pay(md, srn::fwd_group(f32, true), edge, edge, edge) ? srn::fwd_group(f32, true) : f32 ? 64 : 128;
+  const float ratio = (float)full * dt / px, want = rp.order ? sqrtf(ratio) : powf(ratio, 2.f / 3.f);
   rp.rg = rp.order ? 16 : 64;
   while (rp.rg > 1 && ((float)rp.rg > 1.42f * want || rp.rg > count || (int64_t)rp.rg * rp.samples > h->max_points))
     rp.rg /= 2;
-  rp.cell = px * px * dt * (float)(rp.grid[0] * rp.grid[1] * rp.grid[2]);
   const int per = full / rp.rg;
   const int64_t pad = ((int64_t)rp.samples + per - 1) / per * per;
   rp.spr = pad * 8 <= (int64_t)rp.samples * 9 && pad * rp.rg <= h->max_points ? (int)pad : rp.samples;
   // whole ray groups whose slots fit the workspace's max_points samples (and 31 bits)
   const int64_t cap = std::min<int64_t>(h->max_points, (int64_t)1 << 30);
   const int64_t batch = std::max<int64_t>(1, cap / rp.spr / rp.rg) * rp.rg;
-  const srn::Model md = h->model();
   for (int64_t p0 = first; p0 < first + count; p0 += batch) {
     const int n = (int)std::min<int64_t>(batch, first + count - p0);
-    cudaError_t e = srn::launch_render_batch(h->launch(stream), rp, val, (int)p0, n, md, lut, rgba);
+    cudaError_t e = cudaSuccess;
+    if (h->render_failed) e = cudaMemsetAsync(next, 0, sizeof(int32_t), static_cast<cudaStream_t>(stream));
+    h->render_failed = true;
+    if (e == cudaSuccess) e = srn::launch_render_batch(h->launch(stream), rp, val, next, (int)p0, n, md, lut, rgba);
     if (e != cudaSuccess) return cuda_fail(e, "render");
+    h->render_failed = false;
   }
   return SRN_OK;
 }
