@@ -55,11 +55,11 @@ struct Grads {
   int64_t sF, sW1, sW2, sw3;
 };
 
-// A batch of the caller's points and its Morton-sorted copy (launch_sort), which stands in
-// for it when more than `limit` of its points come before their predecessor: *moved is
-// counted on the device, so the choice needs no host round trip.  moved == NULL: no copy.
+// A batch of the caller's points and its Morton-sorted copy (launch_sort_query, launch_tiles),
+// which stands in for it when more than `limit` of its points come before their predecessor:
+// *moved is counted on the device, so the choice needs no host round trip.  xyz == NULL: no copy.
 struct SortedBatch {
-  float* xyz;          // [N][3] in bin order within each brick
+  float* xyz;          // [N][3] in bin order within each brick, or NULL
   float* target;       // [N] the targets in that order (training), or NULL
   uint32_t* index;     // [N] the points' places in the caller's batch (queries), or NULL
   uint32_t* rank;      // [N] scratch: rank inside the bin
@@ -67,7 +67,7 @@ struct SortedBatch {
   uint32_t* moved;
   uint32_t* next;      // (queries) the next call's `moved`
   uint32_t limit;
-  __device__ __forceinline__ bool use() const { return moved && *moved > limit; }
+  __device__ __forceinline__ bool use() const { return xyz && *moved > limit; }
 };
 
 // Workspace pieces the training kernels write.
@@ -100,7 +100,8 @@ struct TrainWs {
 // A tile of the encoder and the scatter: `count` (<= the tuning's tile_points, at most
 // 1024) consecutive points of one brick, all in the aligned Morton range of 2^L units
 // starting at unit u0 when the brick's points are sorted by Morton bin.
-// code = brick << 20 | L << 16 | u0.
+// code = brick << 20 | L << 16 | u0; L = kNoBlock: points in no order, in no block.
+constexpr uint32_t kNoBlock = 15;
 struct ScatTile {
   int64_t start;
   int32_t count;

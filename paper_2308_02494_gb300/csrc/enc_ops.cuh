@@ -158,7 +158,7 @@ __device__ __forceinline__ void enc_stage(const EncBox& e, const EncNode<C>* __r
 // C bf16 (0 outside the grid: Eq. 2's inclusive mask), from the staged box when the
 // point's cell lies in it, else from global memory.  gi is the grid's transform, hs =
 // (R-1)/2, ct = hs - 1/2 + kMagic (used when R is even), Fi the grid's BF16 nodes.
-// PROD: the blend as trilinear_bf16's products ((1 - w) a + w b), else a + w (b - a).
+// PROD: the blend as enc_global's products ((1 - w) a + w b), to its bits, else a + w (b - a).
 template <int C, bool EVEN_R, bool PROD>
 __device__ __forceinline__ uint32_t encode_point(const float (&gi)[12], float x, float y, float z, const EncBox& e,
                                                  float hs, float ct, int R, const __nv_bfloat16* Fi) {
@@ -209,7 +209,10 @@ __device__ __forceinline__ uint32_t encode_point(const float (&gi)[12], float x,
         const float v2 = enc_node<C, 0>(a1), v3 = enc_node<C, kRow>(a1);
         const float v4 = enc_node<C, 0>(a2), v5 = enc_node<C, kRow>(a2);
         const float v6 = enc_node<C, 0>(a3), v7 = enc_node<C, kRow>(a3);
-        auto mix = [](float a, float b, float w) { return PROD ? blend1(a, b, w, 1.f - w) : fmaf(w, b - a, a); };
+        // (enc_global's expression is compiled to the product of a and the FMA of b with one channel)
+        auto mix = [](float a, float b, float w) {
+          return PROD ? fmaf(w, b, __fmul_rn(1.f - w, a)) : fmaf(w, b - a, a);
+        };
         const float e0 = mix(v0, v1, wx), e1 = mix(v2, v3, wx), e2 = mix(v4, v5, wx), e3 = mix(v6, v7, wx);
         yv = __bfloat16_as_ushort(__float2bfloat16_rn(mix(mix(e0, e1, wy), mix(e2, e3, wy), wz)));
       }

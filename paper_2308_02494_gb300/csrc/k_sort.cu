@@ -54,9 +54,7 @@ __global__ void __launch_bounds__(kSortNT) k_sort_query(Bricks br, const float* 
   with_predecessors(br, xyz, [&](int64_t, uint32_t c, uint32_t before, int, bool head) { back += !head && before > c; });
   back = __reduce_add_sync(0xffffffffu, back);
   if ((threadIdx.x & 31) == 0 && back) atomicAdd(s.moved, back);   // (cleared by the call before)
-  uint4* h4 = reinterpret_cast<uint4*>(s.hist);
-  for (int64_t q = first; q < (int64_t)br.n * kSortBins / 4; q += (int64_t)gridDim.x * kSortNT)
-    h4[q] = make_uint4(0u, 0u, 0u, 0u);
+  sort_clear(br, s);   // (here, so that a copy has one barrier less)
   grid.sync();
   if (*(volatile uint32_t*)s.moved <= s.limit) return;
   sort_count(br, xyz, s);
@@ -182,6 +180,23 @@ __device__ __forceinline__ void tile_list(const Bricks& br, int b, const TrainWs
   }
 }
 
+// The tiles of brick b of a batch in no order, by a block: runs of at most `run` points.
+__device__ __forceinline__ void run_list(const Bricks& br, int b, const TrainWs& ws, int run) {
+  __shared__ int32_t s_first;
+  const int64_t o = br.off[b], n = br.off[b + 1] - o;
+  const int32_t nt = (int32_t)((n + run - 1) / run);
+  if (threadIdx.x == 0) s_first = atomicAdd(ws.tile_ctr, nt);
+  __syncthreads();
+  for (int t = threadIdx.x; t < nt; t += blockDim.x) {
+    const int64_t from = t * n / nt;
+    ScatTile T;
+    T.start = o + from;
+    T.count = (int32_t)((t + 1) * n / nt - from);
+    T.code = (uint32_t)b << 20 | kNoBlock << 16;
+    ws.tiles[s_first + t] = T;
+  }
+}
+
 // The sampler's batch: its histogram gives the unit starts.
 __global__ void __launch_bounds__(kSortNT) k_tile_list(Bricks brp, TrainWs ws, Model md, int capn, int lcap, int tp) {
   __shared__ Bricks br;
@@ -192,10 +207,10 @@ __global__ void __launch_bounds__(kSortNT) k_tile_list(Bricks brp, TrainWs ws, M
 // A caller's batch: the first point of every Morton unit (2 x 2 x 2 bins) that starts a run of
 // that unit in its brick (plus one; 0, as cleared with the accumulators, for the others) and
 // the number of points whose unit comes before their predecessor's; the sorted copy if the
-// batch needs one; the tiles.
+// batch needs one and has room for it; the tiles.
 __global__ void __launch_bounds__(kSortNT)
 k_sort_tiles(Bricks br, TrainWs ws, Model md, const float* __restrict__ xyz, const float* __restrict__ target,
-             int capn, int lcap, int tp) {
+             int capn, int capw, int lcap, int tp, int run) {
   cooperative_groups::grid_group grid = cooperative_groups::this_grid();
   const SortedBatch& s = ws.sorted;
   uint32_t back = 0;
@@ -207,7 +222,10 @@ k_sort_tiles(Bricks br, TrainWs ws, Model md, const float* __restrict__ xyz, con
   back = __reduce_add_sync(0xffffffffu, back);
   if ((threadIdx.x & 31) == 0 && back) atomicAdd(s.moved, back);
   grid.sync();
-  if (*(volatile uint32_t*)s.moved > s.limit) {
+  const bool none = *(volatile uint32_t*)s.moved > s.limit;   // in no order
+  if (none && s.xyz) {
+    sort_clear(br, s);
+    grid.sync();
     sort_count(br, xyz, s);
     grid.sync();
     for (int b = blockIdx.x; b < br.n; b += gridDim.x) {
@@ -219,7 +237,8 @@ k_sort_tiles(Bricks br, TrainWs ws, Model md, const float* __restrict__ xyz, con
   }
   for (int b = blockIdx.x; b < br.n; b += gridDim.x) {
     __syncthreads();
-    tile_list(br, b, ws, md, capn, lcap, tp);
+    if (none && !s.xyz) run_list(br, b, ws, run);
+    else tile_list(br, b, ws, md, none ? capw : capn, lcap, tp);
   }
 }
 
@@ -239,13 +258,13 @@ cudaError_t launch_sort_query(const Launch& L, const Bricks& br, const float* xy
 }
 
 cudaError_t launch_tiles(const Launch& L, const Model& md, const Bricks& br, const TrainWs& ws, const float* xyz,
-                         const float* target, int capn, int lcap, int tp) {
+                         const float* target, int capn, int capw, int lcap, int tp, int run) {
   if (ws.bin_start) {
     k_tile_list<<<br.n, kSortNT, 0, L.stream>>>(br, ws, md, capn, lcap, tp);
     return cudaGetLastError();
   }
-  void* args[] = {(void*)&br,     (void*)&ws,   (void*)&md,   (void*)&xyz,
-                  (void*)&target, (void*)&capn, (void*)&lcap, (void*)&tp};
+  void* args[] = {(void*)&br,   (void*)&ws,   (void*)&md,   (void*)&xyz, (void*)&target,
+                  (void*)&capn, (void*)&capw, (void*)&lcap, (void*)&tp,  (void*)&run};
   return cudaLaunchCooperativeKernel((const void*)k_sort_tiles, dim3(sort_blocks(br.off[br.n], L)), dim3(kSortNT), args,
                                      0, L.stream);
 }

@@ -473,6 +473,58 @@ __device__ __forceinline__ void red_cell(uint32_t a0, uint32_t oy, uint32_t oz, 
   }
 }
 
+// The same with 21 more bits below each sum's unit, for batches whose sums were float32 ones
+// (scat_units): the rounding's remainder, exact but for its last bits, goes to a second word.
+constexpr float kLowScale = 2097152.f;   // 2^21: a remainder of at most 1/2 stays below 2^20, and 1024 of them below 2^30
+template <int C>
+__device__ __forceinline__ void red_cell_wide(uint32_t a0, uint32_t oy, uint32_t oz, float wx, float wy, float wz,
+                                              uint32_t d, float scale) {
+  constexpr int kX = 2 * C * 128;   // the next x node
+  const uint32_t a[4] = {a0, a0 + oy, a0 + oz, a0 + oy + oz};
+  if constexpr (C == 2) {
+    const unsigned long long one = f2_bits(1.f, 1.f), mm = f2_bits(kMagic, kMagic), ls = f2_bits(kLowScale, kLowScale);
+    const unsigned long long wx2 = f2_bits(wx, wx), wy2 = f2_bits(wy, wy), wz2 = f2_bits(wz, wz);
+    auto sub2 = [](unsigned long long p, unsigned long long q) {
+      unsigned long long r;
+      asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(p), "l"(q));
+      return r;
+    };
+    const unsigned long long ax2 = sub2(one, wx2), ay2 = sub2(one, wy2), az2 = sub2(one, wz2);
+    const unsigned long long gs = mul2(bf2_bits(d), f2_bits(scale, scale));
+    const unsigned long long z0 = mul2(az2, gs), z1 = mul2(wz2, gs);
+    const unsigned long long yz[4] = {mul2(ay2, z0), mul2(wy2, z0), mul2(ay2, z1), mul2(wy2, z1)};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const unsigned long long va = fma2(ax2, yz[j], mm), vb = fma2(wx2, yz[j], mm);
+      const unsigned long long la = fma2(fma2(ax2, yz[j], sub2(mm, va)), ls, mm);
+      const unsigned long long lb = fma2(fma2(wx2, yz[j], sub2(mm, vb)), ls, mm);
+      red_s32<0>(a[j], (int32_t)(uint32_t)va - kMagicBits);
+      red_s32<128>(a[j], (int32_t)(uint32_t)la - kMagicBits);
+      red_s32<256>(a[j], (int32_t)(uint32_t)(va >> 32) - kMagicBits);
+      red_s32<384>(a[j], (int32_t)(uint32_t)(la >> 32) - kMagicBits);
+      red_s32<kX>(a[j], (int32_t)(uint32_t)vb - kMagicBits);
+      red_s32<kX + 128>(a[j], (int32_t)(uint32_t)lb - kMagicBits);
+      red_s32<kX + 256>(a[j], (int32_t)(uint32_t)(vb >> 32) - kMagicBits);
+      red_s32<kX + 384>(a[j], (int32_t)(uint32_t)(lb >> 32) - kMagicBits);
+    }
+  } else {
+    const float ax = 1.f - wx, ay = 1.f - wy, az = 1.f - wz;
+    const float zy[4] = {az * ay, az * wy, wz * ay, wz * wy};
+    const float gs = __uint_as_float(d << 16) * scale;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float wa = zy[j] * ax, wb = zy[j] * wx;
+      const float va = fmaf(wa, gs, kMagic), vb = fmaf(wb, gs, kMagic);
+      const float la = fmaf(fmaf(wa, gs, kMagic - va), kLowScale, kMagic);
+      const float lb = fmaf(fmaf(wb, gs, kMagic - vb), kLowScale, kMagic);
+      red_s32<0>(a[j], __float_as_int(va) - kMagicBits);
+      red_s32<128>(a[j], __float_as_int(la) - kMagicBits);
+      red_s32<kX>(a[j], __float_as_int(vb) - kMagicBits);
+      red_s32<kX + 128>(a[j], __float_as_int(lb) - kMagicBits);
+    }
+  }
+}
+
 // dL/dy of point p (global index) for grid g: C bf16 values in the low bits.
 template <int C>
 __device__ __forceinline__ uint32_t dy_bits(const __nv_bfloat16* dY, int64_t p, int M, int g) {
@@ -485,6 +537,7 @@ __device__ __forceinline__ uint32_t dy_bits(const __nv_bfloat16* dY, int64_t p, 
 // block is inside the grid).
 __device__ uint2 tile_box(uint32_t code, const float* __restrict__ g, int R) {
   const int L = (code >> 16) & 15;
+  if (L == kNoBlock) return make_uint2(0u, 0u);
   const uint32_t u0 = code & 0xffffu;
   const int ext[3] = {1 << ((L + 2) / 3), 1 << ((L + 1) / 3), 1 << (L / 3)};
   const uint32_t uc[3] = {compact3(u0), compact3(u0 >> 1), compact3(u0 >> 2)};
@@ -498,25 +551,21 @@ __device__ uint2 tile_box(uint32_t code, const float* __restrict__ g, int R) {
   return block_box(lo, hi, g, R);
 }
 
-// Two CTAs of 8 warps per SM, each on its own units, so that one CTA's barriers and
-// flushes overlap the other's reductions.  At most 96 registers: with them a CTA of the
-// density pass (8 warps x 64) fits beside the scatter's 16 warps in one SM's register file.
-template <int C, bool EVEN_R>
-__global__ void __maxnreg__(96)
-k_scat(Model md, Grads gr, Bricks brp, TrainWs ws, const float* __restrict__ xyz, int capn) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  ScatHead& h = *reinterpret_cast<ScatHead*>(smraw);
-  int32_t* acc = reinterpret_cast<int32_t*>(smraw + sizeof(ScatHead));
-  __shared__ Bricks br;
-  __shared__ TileMap dtm;   // the decoder's 128-point tiles (ws.gmax_blk)
-  load_bricks(brp, br);
-  if (ws.sorted.use()) xyz = ws.sorted.xyz;
-  if (threadIdx.x == 0) build_tile_map(br, 128, dtm);
+// The units of k_scat.  WIDE: the batch is a sorted copy of one in no order, whose products
+// were added in float32 one by one.  Its boxes take those within 2^-17 of the tile's largest
+// dL/dy with 41 bits or more below that (red_cell_wide), so that the rounding of a product is
+// below 2^-25 of its point's dL/dy (float32's own weights are off by 2^-20); smaller ones, and
+// tiles with an infinity or a NaN, are added one by one as before.  capn: nodes that fit.
+template <int C, bool EVEN_R, bool WIDE>
+__device__ __forceinline__ void scat_units(const Model& md, const Grads& gr, const Bricks& br, const TileMap& dtm,
+                                           const TrainWs& ws, const float* __restrict__ xyz, int capn, ScatHead& h,
+                                           int32_t* acc) {
   const int tid = threadIdx.x, lane = tid & 31;
   const int M = md.M, R = md.R;
   const int ngrp = M >= 32 ? M >> 5 : 1;
   const int gper = M >= 32 ? 32 : M;             // grids of a unit
-  constexpr int kNode = C * 32;                  // words of one node of a column group
+  constexpr int kLimbs = WIDE ? 2 : 1;           // words of a sum
+  constexpr int kNode = C * 32 * kLimbs;         // words of one node of a column group
   constexpr uint32_t kNodeBytes = kNode * 4;
   {  // the boxes start zeroed; every flush leaves them zeroed again
     uint4* a4 = reinterpret_cast<uint4*>(acc);
@@ -564,8 +613,8 @@ k_scat(Model md, Grads gr, Bricks brp, TrainWs ws, const float* __restrict__ xyz
     const int64_t p0 = T.start;
     const int np = T.count;
     const float* Gb = md.G + (int64_t)b * md.sG;
-    const int lvl = (int)((T.code >> 16) & 15u);
-    bool mine_in = true;   // every point of this thread lies in the tile's block
+    const uint32_t lvl = (T.code >> 16) & 15u;
+    bool mine_in = lvl != kNoBlock;   // every point of this thread lies in the tile's block
     for (int p = tid; p < np; p += SCT) {
       const float x = xyz[3 * (p0 + p)], y = xyz[3 * (p0 + p) + 1], z = xyz[3 * (p0 + p) + 2];
       h.xs[p] = make_float4(x, y, z, 0.f);
@@ -606,8 +655,9 @@ k_scat(Model md, Grads gr, Bricks brp, TrainWs ws, const float* __restrict__ xyz
     const int nxb = (int)(bx.y & 0xffu), nyb = (int)((bx.y >> 8) & 0xffu), nzb = (int)((bx.y >> 16) & 0xffu);
     const int lox = (int)(bx.x & 0xffu), loy = (int)((bx.x >> 8) & 0xffu), loz = (int)((bx.x >> 16) & 0xffu);
     const int nodes = nxb * nyb * nzb;
-    const bool boxed = nodes > 0 && nodes <= capn;
     const uint32_t mb = h.gmax[mp.g - g0u];
+    const bool boxed = nodes > 0 && nodes <= capn && (!WIDE || mb < 0x7f80u);
+    const uint32_t least = mb > (17u << 7) ? mb - (17u << 7) : 1u;   // (WIDE) bits of the smallest boxed dL/dy
     float inv;
     const float scale = fixed_scale(mb, np, inv);
     float* dFi = gr.dF + (int64_t)b * gr.sF + mp.g * gsz;
@@ -678,14 +728,20 @@ k_scat(Model md, Grads gr, Bricks brp, TrainWs ws, const float* __restrict__ xyz
           // mask): the box's cells lie in [0, R-2], and beyond a face the cell on that
           // axis is -1 or R-1.  With R odd the cell is a truncation: test the mask.
           if constexpr (!EVEN_R) inbox = inbox && (fabsf(ux) <= 1.f) & (fabsf(uy) <= 1.f) & (fabsf(uz) <= 1.f);
+          if constexpr (WIDE) {   // (0 - 1 is no small number)
+            const uint32_t m = dc[u] & kNz;
+            inbox = inbox && (m & 0xffffu) - 1u >= least - 1u;
+            if constexpr (C == 2) inbox = inbox && (m >> 16) - 1u >= least - 1u;
+          }
           ad[u] = nz && inbox ? col_s + ((lz * (unsigned)nyb + ly) * (unsigned)nxb + lx) * kNodeBytes : ~0u;
           live |= (uint32_t)(nz && !inbox) << u;
         }
 #pragma unroll
         for (int u = 0; u < SU; ++u) {
           if (ad[u] != ~0u) {
-            red_cell<C>(ad[u], oy, oz, wxs[u], wys[u], wzs[u], dc[u], scale);
-          } else if (live & (1u << u)) {   // outside the tile's box (rounding at its faces, or an unsorted batch)
+            if constexpr (WIDE) red_cell_wide<C>(ad[u], oy, oz, wxs[u], wys[u], wzs[u], dc[u], scale);
+            else red_cell<C>(ad[u], oy, oz, wxs[u], wys[u], wzs[u], dc[u], scale);
+          } else if (live & (1u << u)) {   // outside the tile's box (rounding at its faces, or a batch in no order)
             const float4 x = h.xs[p + u * mp.npg];
             float ux, uy, uz;
             affine(gi, x.x, x.y, x.z, ux, uy, uz);
@@ -706,18 +762,25 @@ k_scat(Model md, Grads gr, Bricks brp, TrainWs ws, const float* __restrict__ xyz
       int qz = n0 / (nxb * nyb), qr = n0 - qz * nxb * nyb;
       int qy = qr / nxb, qx = qr - qy * nxb;
       for (int n = n0; n < nodes; n += step) {
-        int32_t s0 = 0, s1 = 0;
+        int32_t s[C * kLimbs] = {};
         int32_t* q = acc + n * kNode + lane;   // column lane = grid g's first
+        int32_t any = 0;
         for (int sub = 0; sub < (M >= 32 ? 1 : 32 / M); ++sub) {
           int32_t* qs = q + sub * M;
-          s0 += qs[0];
-          qs[0] = 0;
-          if (C == 2) { s1 += qs[32]; qs[32] = 0; }
+#pragma unroll
+          for (int w = 0; w < C * kLimbs; ++w) { s[w] += qs[32 * w]; qs[32 * w] = 0; }
         }
-        if (s0 | s1) {
+#pragma unroll
+        for (int w = 0; w < C * kLimbs; ++w) any |= s[w];
+        if (any) {
           const int node = ((loz + qz) * R + (loy + qy)) * R + lox + qx;   // < R^3 <= 2^18
-          if (C == 2) atomicAdd(reinterpret_cast<float2*>(dFi) + node, make_float2((float)s0 * inv, (float)s1 * inv));
-          else atomicAdd(dFi + node, (float)s0 * inv);
+          auto sum = [&](int c) {
+            if constexpr (WIDE)   // (one rounding)
+              return __ll2float_rn(((long long)s[2 * c] << 21) + s[2 * c + 1]) * (1.f / kLowScale) * inv;
+            else return (float)s[c] * inv;
+          };
+          if constexpr (C == 2) atomicAdd(reinterpret_cast<float2*>(dFi) + node, make_float2(sum(0), sum(1)));
+          else atomicAdd(dFi + node, sum(0));
         }
         qx += step;
         while (qx >= nxb) {
@@ -727,6 +790,23 @@ k_scat(Model md, Grads gr, Bricks brp, TrainWs ws, const float* __restrict__ xyz
       }
     }
   }
+}
+
+// Two CTAs of 8 warps per SM, each on its own units, so that one CTA's barriers and
+// flushes overlap the other's reductions.  At most 96 registers: with them a CTA of the
+// density pass (8 warps x 64) fits beside the scatter's 16 warps in one SM's register file.
+template <int C, bool EVEN_R>
+__global__ void __maxnreg__(96)
+k_scat(Model md, Grads gr, Bricks brp, TrainWs ws, const float* __restrict__ xyz, int capn) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  ScatHead& h = *reinterpret_cast<ScatHead*>(smraw);
+  int32_t* acc = reinterpret_cast<int32_t*>(smraw + sizeof(ScatHead));
+  __shared__ Bricks br;
+  __shared__ TileMap dtm;   // the decoder's 128-point tiles (ws.gmax_blk)
+  load_bricks(brp, br);
+  if (threadIdx.x == 0) build_tile_map(br, 128, dtm);
+  if (ws.sorted.use()) scat_units<C, EVEN_R, true>(md, gr, br, dtm, ws, ws.sorted.xyz, capn / 2, h, acc);
+  else scat_units<C, EVEN_R, false>(md, gr, br, dtm, ws, xyz, capn, h, acc);
 }
 
 // =============================================================================== k_enc
@@ -755,8 +835,8 @@ k_enc(Model md, Bricks brp, TrainWs ws, const float* __restrict__ xyz, int capn)
   SE* boxes = reinterpret_cast<SE*>(smraw + sizeof(EncHead));   // [capn][32 columns]
   __shared__ Bricks br;
   load_bricks(brp, br);
-  // a batch that was not sorted reads Eq. 2 in the form that its points used to take (all
-  // of them outside their tiles' boxes), so that the features keep their bits
+  // a sorted copy reads Eq. 2 as products, the form that the points of a batch in no order
+  // take elsewhere (outside their tiles' boxes): the same bits, however the batch is run
   const bool copied = ws.sorted.use();
   if (copied) xyz = ws.sorted.xyz;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -985,7 +1065,12 @@ cudaError_t launch_train_k(const Launch& L, bool dens, const Model& md, const Gr
     if (cap < 8) return cudaErrorInvalidConfiguration;
     if (tn.tile_points < kMinTilePoints || tn.tile_points > ST || tn.tile_level < 0 || tn.tile_level > kMaxTileLevel)
       return cudaErrorInvalidValue;
-    if ((e = launch_tiles(L, md, br, ws, xyz, target, cap, tn.tile_level, tn.tile_points)) != cudaSuccess) return e;
+    const int capw = std::min(scat_capn(md.M, md.C) / 2, enc_capn(md.M, md.C));   // (two words a sum: scat_units)
+    // a batch in no blocks: two units for each CTA of the encoder and the scatter
+    const int64_t units = 4 * (int64_t)L.num_sms, groups = std::max(1, md.M / 32);
+    const int run = (int)std::min<int64_t>(std::max<int64_t>(br.off[br.n] * groups / units, 32), tn.tile_points);
+    if ((e = launch_tiles(L, md, br, ws, xyz, target, cap, capw, tn.tile_level, tn.tile_points, run)) != cudaSuccess)
+      return e;
   }
   {
     const int capn = enc_capn(md.M, md.C);

@@ -35,6 +35,12 @@ struct SideStream {
 // A tile is a run of Morton-consecutive points of one brick inside one aligned Morton
 // block of at most 2^tile_level units, holding at most tile_points points; the block's
 // node box in every grid is what the encoder stages and the scatter accumulates.
+// Points per brick from which a training batch in no order gets a sorted copy, whose tiles have
+// boxes; a smaller one runs as it is, every corner's sum in memory (runs and copy, in us, without
+// the density loss: 64 grids of 32^3, 100003 points 638 and 328, zoomed by up to 1.4 415 and 472,
+// 8 bricks of 125000 5209 and 2250, zoomed 3142 and 3455; 32 grids of 20^3, 100003 points 343 and
+// 168; 8 grids of 16^3, 143 and 127).
+constexpr int64_t kSortPoints = 50000;
 constexpr int kMinTilePoints = 128;
 constexpr int kMaxTilePoints = 1024;   // the encoder's and the scatter's point staging
 constexpr int kMaxTileLevel = 9;
@@ -124,10 +130,11 @@ cudaError_t launch_sample(const Launch& L, const Bricks& br, unsigned long long 
 cudaError_t launch_sort_query(const Launch& L, const Bricks& br, const float* xyz, const SortedBatch& s);
 // The training pass's tiles (ws.tiles, ws.tile_ctr[0]): at most tp points each, levels up to
 // lcap with node boxes of at most capn nodes.  A batch that is not the sampler's (no
-// ws.bin_start) gets its unit starts and, if out of order, its sorted copy first
-// (ws.ustart, ws.sorted's counters and ws.tile_ctr cleared by the caller).
+// ws.bin_start) gets its unit starts first; one that is out of order gets a sorted copy and
+// boxes of at most capw nodes, or, where it has no room for one (ws.sorted.xyz), runs of `run`
+// points in no blocks (ws.ustart and ws.tile_ctr cleared by the caller).
 cudaError_t launch_tiles(const Launch& L, const Model& md, const Bricks& br, const TrainWs& ws, const float* xyz,
-                         const float* target, int capn, int lcap, int tp);
+                         const float* target, int capn, int capw, int lcap, int tp, int run);
 struct VolumeBoxes {
   int32_t lo[SRN_MAX_BRICKS][3];
   int32_t hi[SRN_MAX_BRICKS][3];

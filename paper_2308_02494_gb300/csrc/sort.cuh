@@ -63,7 +63,14 @@ __device__ __forceinline__ void scan_bins(uint32_t* hist) {
     h[32 * k] = make_uint4(s, s + v[k].x, s + v[k].x + v[k].y, s + v[k].x + v[k].y + v[k].z);
   }
 }
-// Ranks and bin counts (cleared before).
+// The bins' counts, cleared by the whole grid.
+__device__ __forceinline__ void sort_clear(const Bricks& br, const SortedBatch& s) {
+  uint4* h4 = reinterpret_cast<uint4*>(s.hist);
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < (int64_t)br.n * kSortBins / 4;
+       q += (int64_t)gridDim.x * blockDim.x)
+    h4[q] = make_uint4(0u, 0u, 0u, 0u);
+}
+// Ranks and bin counts.
 __device__ __forceinline__ void sort_count(const Bricks& br, const float* __restrict__ xyz, const SortedBatch& s) {
   const int64_t total = br.off[br.n], first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t step = (int64_t)gridDim.x * blockDim.x;

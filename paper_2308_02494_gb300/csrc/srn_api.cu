@@ -84,7 +84,7 @@ void make_layout(const srn_config* c, srn_layout* L) {
 // Workspace carving (every piece 256-byte aligned).
 struct WsLayout {
   size_t state, acc, gsum, rsum, rho, herr, sort_rank, sort_hist, feat, dfeat, gmax, ustart, tiles, tile_ctr;
-  size_t sched, sring;
+  size_t sched, sring, moved;
   size_t r_val, r_next, total;
   size_t t_xyz, t_target, t_rank, t_hist, q_xyz, q_index, q_rank, q_hist;
 };
@@ -93,10 +93,11 @@ WsLayout ws_layout(const srn_config* c, int64_t maxp) {
   WsLayout w{};
   size_t o = 0;
   w.state = o; o += align256(sizeof(srn::StepState) + 64);
+  const bool bf16 = c->precision == SRN_BF16;
   const size_t hist = align256(sizeof(uint32_t) * ((size_t)srn::kSortBins * c->n_bricks + 2));   // and `moved`
   // (from here to rsum's end: cleared by every backward pass)
-  w.ustart = o; o += c->precision == SRN_BF16 ? align256(sizeof(int32_t) * (srn::kUnits + 1) * c->n_bricks) : 0;
-  w.t_hist = o; o += hist;
+  w.ustart = o; o += bf16 ? align256(sizeof(int32_t) * (srn::kUnits + 1) * c->n_bricks) : 0;
+  w.moved = o; o += align256(sizeof(uint32_t));   // (on a line of its own: beside the tile counters it took 15 us)
   w.tile_ctr = o; o += align256(sizeof(int32_t) * 5);
   w.acc = o; o += align256(sizeof(double) * srn::kAccPerBrick * c->n_bricks);
   w.gsum = o; o += align256(sizeof(double) * 13 * c->n_grids * c->n_bricks);
@@ -106,15 +107,14 @@ WsLayout ws_layout(const srn_config* c, int64_t maxp) {
   w.sort_rank = o; o += align256(sizeof(uint32_t) * maxp);
   w.sort_hist = o; o += align256(sizeof(uint32_t) * srn::kSortBins * c->n_bricks);
   // BF16 training pass: features Y [N][K] and dL/dy [M][N][C], both bfloat16
-  const size_t kbytes = c->precision == SRN_BF16 ? sizeof(uint16_t) * c->n_grids * c->channels : 0;
+  const size_t kbytes = bf16 ? sizeof(uint16_t) * c->n_grids * c->channels : 0;
   w.feat = o; o += align256(kbytes * maxp);
   w.dfeat = o; o += align256(kbytes * maxp);
   // largest |dL/dy| per grid and 128-point decoder tile (tcgen05 decoder, K = 128)
   const int64_t dec_tiles = maxp / 128 + c->n_bricks + 1;
-  w.gmax = o; o += c->precision == SRN_BF16 ? align256(sizeof(uint16_t) * srn::kMaxGrids * dec_tiles) : 0;
+  w.gmax = o; o += bf16 ? align256(sizeof(uint16_t) * srn::kMaxGrids * dec_tiles) : 0;
   // BF16 tiles: unit starts, and at most one tile per unit plus one per kMinTilePoints
   // points (the smallest tile any tuning allows)
-  const bool bf16 = c->precision == SRN_BF16;
   const int64_t max_tiles = (int64_t)c->n_bricks * (srn::kUnits + 1) + maxp / srn::kMinTilePoints + 1;
   w.tiles = o; o += bf16 ? align256(sizeof(srn::ScatTile) * max_tiles) : 0;
   w.sched = o; o += align256(sizeof(srn::BrickSched) * c->n_bricks);
@@ -125,6 +125,7 @@ WsLayout ws_layout(const srn_config* c, int64_t maxp) {
   w.t_xyz = o; o += align256(sizeof(float) * 3 * maxp);
   w.t_target = o; o += align256(sizeof(float) * maxp);
   w.t_rank = o; o += align256(sizeof(uint32_t) * maxp);
+  w.t_hist = o; o += hist;
   w.q_xyz = o; o += align256(sizeof(float) * 3 * maxp);
   w.q_index = o; o += align256(sizeof(uint32_t) * maxp);
   w.q_rank = o; o += align256(sizeof(uint32_t) * maxp);
@@ -225,19 +226,32 @@ struct srn_handle {
     w.sorted = srn::SortedBatch{};
     return w;
   }
-  // Scratch of a training batch's (query's) sorted copy.
-  srn::SortedBatch sort_scratch(bool query) const {
+  // Scratch of a query's sorted copy.
+  srn::SortedBatch query_scratch() const {
     srn::SortedBatch s{};
-    s.xyz = reinterpret_cast<float*>(ws + (query ? wl.q_xyz : wl.t_xyz));
-    if (query) s.index = reinterpret_cast<uint32_t*>(ws + wl.q_index);
-    else s.target = reinterpret_cast<float*>(ws + wl.t_target);
-    s.rank = reinterpret_cast<uint32_t*>(ws + (query ? wl.q_rank : wl.t_rank));
-    s.hist = reinterpret_cast<uint32_t*>(ws + (query ? wl.q_hist : wl.t_hist));
+    s.xyz = reinterpret_cast<float*>(ws + wl.q_xyz);
+    s.index = reinterpret_cast<uint32_t*>(ws + wl.q_index);
+    s.rank = reinterpret_cast<uint32_t*>(ws + wl.q_rank);
+    s.hist = reinterpret_cast<uint32_t*>(ws + wl.q_hist);
     s.moved = s.hist + (size_t)srn::kSortBins * cfg.n_bricks;
-    s.next = nullptr;
-    if (query) {   // each call counts in one word, and clears the next call's
-      s.next = s.moved + ((query_turn + 1) & 1);
-      s.moved += query_turn & 1;
+    s.next = s.moved + ((query_turn + 1) & 1);   // each call counts in one word, and clears the next call's
+    s.moved += query_turn & 1;
+    return s;
+  }
+  // A caller's training batch: where it counts the points out of order, and its sorted copy if
+  // it is large enough for one (srn::kSortPoints).  One point in 1024 is the limit: with as many
+  // out of place the tiles of a batch left as it is find few points in their blocks (2^18 points,
+  // 64 grids of 32^3, one in 1000 moved: 1413 us, and 441 with a copy).
+  srn::SortedBatch batch_scratch(const srn::Bricks& br) const {
+    srn::SortedBatch s{};
+    const int64_t n = br.off[br.n];
+    s.moved = reinterpret_cast<uint32_t*>(ws + wl.moved);
+    s.limit = n <= UINT32_MAX ? (uint32_t)(n / 1024) : UINT32_MAX;
+    if (n >= srn::kSortPoints * br.n && n <= UINT32_MAX) {
+      s.xyz = reinterpret_cast<float*>(ws + wl.t_xyz);
+      s.target = reinterpret_cast<float*>(ws + wl.t_target);
+      s.rank = reinterpret_cast<uint32_t*>(ws + wl.t_rank);
+      s.hist = reinterpret_cast<uint32_t*>(ws + wl.t_hist);
     }
     return s;
   }
@@ -337,7 +351,7 @@ cudaError_t forward_points(srn_handle* h, const srn::Launch& L, const srn::Model
   // stream before: a stream destroyed since, or another thread's per-thread default stream)
   cudaError_t e = h->query_turn ? cudaStreamWaitEvent(L.stream, h->query_done, 0) : cudaSuccess;
   if (e != cudaSuccess) return e;
-  src.sorted = h->sort_scratch(true);
+  src.sorted = h->query_scratch();
   src.sorted.limit = (uint32_t)(n / 32);   // scan lines and other nearly sorted batches stay as they are
   if ((e = srn::launch_sort_query(L, br, xyz, src.sorted)) != cudaSuccess) return e;
   ++h->query_turn;
@@ -387,14 +401,7 @@ srn_status run_query(srn_handle* h, void* stream, srn::QueryMode mode, const srn
   else if (h->cfg.precision != SRN_BF16)
     e = srn::launch_train_fp32(L, mode == srn::kTrainDensity, md, gr, br, ws, xyz, target);
   else {
-    // A caller's batch that is out of order runs through a sorted copy (random points, with
-    // it and without: 2000 points 84 and 88 us at M = 8, R = 16, 162 and 293 at M = 64,
-    // R = 32; 131072 points 138 and 222, 271 and 720)
-    const int64_t n = br.off[br.n];
-    if (!ws.bin_start) {
-      ws.sorted = h->sort_scratch(false);
-      ws.sorted.limit = n >= 1024 && n <= UINT32_MAX ? (uint32_t)(n / 1024) : UINT32_MAX;
-    }
+    if (!ws.bin_start) ws.sorted = h->batch_scratch(br);
     e = srn::launch_train_bf16(L, mode == srn::kTrainDensity, md, gr, br, ws, xyz, target, h->tune,
                                timed && time_kernel ? &mark : nullptr, h->side.stream ? &h->side : nullptr);
   }
@@ -429,9 +436,9 @@ srn_status do_backward(srn_handle* h, void* stream, const float* xyz, const floa
   const srn::BrickSched* sched = (flags & SRN_SCHEDULE) ? h->sched() : nullptr;
   const bool dens = (flags & SRN_DENSITY) != 0 || sched;
   cudaError_t e = cudaMemsetAsync(h->t.grads_dev, 0, sizeof(float) * h->lay.n_params, s);
+  const size_t from = h->wl.ustart;
   if (e == cudaSuccess)
-    e = cudaMemsetAsync(h->ws + h->wl.ustart, 0,
-                        h->wl.rsum - h->wl.ustart + sizeof(double) * 12 * h->cfg.n_grids * h->cfg.n_bricks, s);
+    e = cudaMemsetAsync(h->ws + from, 0, h->wl.rsum - from + sizeof(double) * 12 * h->cfg.n_grids * h->cfg.n_bricks, s);
   if (e != cudaSuccess) return cuda_fail(e, "memset");
   const int rec_dg = (flags & SRN_REC_DG) ? 1 : 0;
   h->side.defer_join = split;
