@@ -95,7 +95,7 @@ WsLayout ws_layout(const srn_config* c, int64_t maxp) {
   w.state = o; o += align256(sizeof(srn::StepState) + 64);
   const bool bf16 = c->precision == SRN_BF16;
   const size_t hist = align256(sizeof(uint32_t) * ((size_t)srn::kSortBins * c->n_bricks + 2));   // and `moved`
-  // (from here to rsum's end: cleared by every backward pass)
+  // cleared by every backward pass up to rsum's end: from ustart where it is read
   w.ustart = o; o += bf16 ? align256(sizeof(int32_t) * (srn::kUnits + 1) * c->n_bricks) : 0;
   w.moved = o; o += align256(sizeof(uint32_t));   // (on a line of its own: beside the tile counters it took 15 us)
   w.tile_ctr = o; o += align256(sizeof(int32_t) * 5);
@@ -121,11 +121,11 @@ WsLayout ws_layout(const srn_config* c, int64_t maxp) {
   w.sring = o; o += align256(sizeof(double) * 2 * srn::kMaxDensityWindow * c->n_bricks);
   w.r_val = o; o += align256(sizeof(float) * maxp);   // values of a render batch's samples
   w.r_next = o; o += align256(sizeof(int32_t));
-  // sorted copies of a batch in memory: one of the training pass, one of the queries
-  w.t_xyz = o; o += align256(sizeof(float) * 3 * maxp);
-  w.t_target = o; o += align256(sizeof(float) * maxp);
-  w.t_rank = o; o += align256(sizeof(uint32_t) * maxp);
-  w.t_hist = o; o += hist;
+  // sorted copies of a batch in memory: one of the BF16 training pass, one of the queries
+  w.t_xyz = o; o += bf16 ? align256(sizeof(float) * 3 * maxp) : 0;
+  w.t_target = o; o += bf16 ? align256(sizeof(float) * maxp) : 0;
+  w.t_rank = o; o += bf16 ? align256(sizeof(uint32_t) * maxp) : 0;
+  w.t_hist = o; o += bf16 ? hist : 0;
   w.q_xyz = o; o += align256(sizeof(float) * 3 * maxp);
   w.q_index = o; o += align256(sizeof(uint32_t) * maxp);
   w.q_rank = o; o += align256(sizeof(uint32_t) * maxp);
@@ -436,7 +436,7 @@ srn_status do_backward(srn_handle* h, void* stream, const float* xyz, const floa
   const srn::BrickSched* sched = (flags & SRN_SCHEDULE) ? h->sched() : nullptr;
   const bool dens = (flags & SRN_DENSITY) != 0 || sched;
   cudaError_t e = cudaMemsetAsync(h->t.grads_dev, 0, sizeof(float) * h->lay.n_params, s);
-  const size_t from = h->wl.ustart;
+  const size_t from = h->batch_bins ? h->wl.tile_ctr : h->wl.ustart;   // (the sampler's bins give the unit starts)
   if (e == cudaSuccess)
     e = cudaMemsetAsync(h->ws + from, 0, h->wl.rsum - from + sizeof(double) * 12 * h->cfg.n_grids * h->cfg.n_bricks, s);
   if (e != cudaSuccess) return cuda_fail(e, "memset");
