@@ -19,11 +19,8 @@ constexpr int kUnitBits = kSortBits - 1;          // a unit is 2 x 2 x 2 bins
 constexpr int kUnits = 1 << (3 * kUnitBits);
 
 // Per-launch description of the bricks: points of brick b are [off[b], off[b+1]).
-// When `dev` is non-NULL the offsets are read from device memory at kernel start
-// (counts produced on the device, e.g. by the renderer's bucketing).
 struct Bricks {
   int32_t n;
-  const int64_t* dev;
   int64_t off[SRN_MAX_BRICKS + 1];
 };
 
@@ -32,8 +29,7 @@ struct Bricks {
 __device__ __forceinline__ void load_bricks(const Bricks& in, Bricks& sh) {
   if (threadIdx.x == 0) {
     sh.n = in.n;
-    sh.dev = nullptr;
-    for (int b = 0; b <= in.n; ++b) sh.off[b] = in.dev ? in.dev[b] : in.off[b];
+    for (int b = 0; b <= in.n; ++b) sh.off[b] = in.off[b];
   }
   __syncthreads();
 }

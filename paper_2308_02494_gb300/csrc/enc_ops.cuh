@@ -32,12 +32,8 @@ using EncNode = std::conditional_t<C == 2, uint32_t, uint16_t>;   // one node in
 template <int C>
 using EncSNode = std::conditional_t<C == 2, unsigned long long, float>;   // one staged node: C float32
 
-// Packed float pairs (two channels at once).
-__device__ __forceinline__ unsigned long long f2_bits(float lo, float hi) {
-  return (unsigned long long)__float_as_uint(lo) | ((unsigned long long)__float_as_uint(hi) << 32);
-}
 __device__ __forceinline__ unsigned long long bf2_bits(uint32_t v) {   // bf16x2 -> f32x2
-  return f2_bits(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
+  return f2_pack(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
 }
 // a + w (b - a) on both halves
 __device__ __forceinline__ unsigned long long lerp2(unsigned long long a, unsigned long long b,
@@ -48,23 +44,11 @@ __device__ __forceinline__ unsigned long long lerp2(unsigned long long a, unsign
   return r;
 }
 
-__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
-  unsigned long long r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b,
-                                                   unsigned long long c) {
-  unsigned long long r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-
-// (1 - w) a + w b, rounded as trilinear_bf16's expression is (one product, one FMA):
+// (1 - w) a + w b as one product and one FMA, as a query always rounded it:
 // packed over two channels, v = 1 - w, and for one.
 __device__ __forceinline__ unsigned long long blend2(unsigned long long a, unsigned long long b,
                                                      unsigned long long w, unsigned long long v) {
-  return fma2(v, a, mul2(w, b));
+  return f2_fma(v, a, f2_mul(w, b));
 }
 __device__ __forceinline__ float blend1(float a, float b, float w, float v) { return fmaf(v, a, __fmul_rn(w, b)); }
 
@@ -72,7 +56,7 @@ __device__ __forceinline__ float blend1(float a, float b, float w, float v) { re
 // ct2 = (ct, ct), m2 = (kMagic, kMagic): the same roundings as two axis_cell calls.
 __device__ __forceinline__ void axis_cell2(unsigned long long u, unsigned long long hs2, unsigned long long ct2,
                                            unsigned long long m2, int32_t& ta, int32_t& tb, float& wa, float& wb) {
-  const unsigned long long t = fma2(u, hs2, ct2), s = fma2(u, hs2, hs2);
+  const unsigned long long t = f2_fma(u, hs2, ct2), s = f2_fma(u, hs2, hs2);
   unsigned long long tm, w;
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(tm) : "l"(t), "l"(m2));
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(w) : "l"(s), "l"(tm));
@@ -179,7 +163,7 @@ __device__ __forceinline__ uint32_t encode_point(const float (&gi)[12], float x,
     unsigned lx, ly, lz;   // cell relative to the box
     if constexpr (EVEN_R) {
       int32_t tx, ty;   // x and y as one packed pair
-      axis_cell2(f2_bits(ux, uy), f2_bits(hs, hs), f2_bits(ct, ct), f2_bits(kMagic, kMagic), tx, ty, wx, wy);
+      axis_cell2(f2_pack(ux, uy), f2_pack(hs, hs), f2_pack(ct, ct), f2_pack(kMagic, kMagic), tx, ty, wx, wy);
       lx = (unsigned)(tx - e.mlox);
       ly = (unsigned)(ty - e.mloy);
       lz = (unsigned)(axis_cell(uz, hs, ct, wz) - e.mloz);
@@ -193,9 +177,9 @@ __device__ __forceinline__ uint32_t encode_point(const float (&gi)[12], float x,
       const uint32_t a0 = e.col_s + ((lz * (unsigned)e.nyb + ly) * (unsigned)e.nxb + lx) * kRow;
       const uint32_t a1 = a0 + e.oy, a2 = a0 + e.oz, a3 = a2 + e.oy;
       if constexpr (C == 2) {
-        const unsigned long long px = f2_bits(wx, wx), py = f2_bits(wy, wy), pz = f2_bits(wz, wz);
+        const unsigned long long px = f2_pack(wx, wx), py = f2_pack(wy, wy), pz = f2_pack(wz, wz);
         auto mix = [](unsigned long long a, unsigned long long b, float w, unsigned long long w2) {
-          if constexpr (PROD) return blend2(a, b, w2, f2_bits(1.f - w, 1.f - w));
+          if constexpr (PROD) return blend2(a, b, w2, f2_pack(1.f - w, 1.f - w));
           else return lerp2(a, b, w2);
         };
         const unsigned long long e0 = mix(enc_node<C, 0>(a0), enc_node<C, kRow>(a0), wx, px);

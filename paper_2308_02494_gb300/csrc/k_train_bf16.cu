@@ -12,7 +12,7 @@
 //          K = 128 runs on tcgen05 instead (k_mlp_tc.cu).
 //  k_scat  adjoint of Eq. 2.  A tile is up to tile_points (<= 1024) points of one brick
 //          lying in one aligned Morton range of the sampler's bins (a small
-//          axis-aligned block of the brick), listed by k_tile_list.
+//          axis-aligned block of the brick), listed by k_tile_list or k_sort_tiles.
 //          Two CTAs per SM take (tile, group of 32 grids) units.  Lane l of a warp
 //          takes grid l of the group: the block, mapped through the grid's Eq. 1,
 //          bounds a node box that the tile's level keeps within shared memory, and the
@@ -21,8 +21,9 @@
 //          its largest |dL/dy|: for K = 128 the decoder's maxima per 128 points) with
 //          shared-memory integer reductions, one bank per lane.
 //          Each box node then goes into the float32 gradient grid with one atomic.
-//          Points outside their tile's box (rounding at its faces; a batch that is not
-//          Morton-sorted) add their corners directly.
+//          Points outside their tile's box (rounding at its faces) add their corners
+//          directly, as all do of a batch in no order; a large one is sorted first, and
+//          its boxes hold two words per sum (scat_units).
 #include "enc_ops.cuh"
 #include "kernels.h"
 #include "sort.cuh"
@@ -444,19 +445,19 @@ template <int C>
 __device__ __forceinline__ void red_cell(uint32_t a0, uint32_t oy, uint32_t oz, float wx, float wy, float wz,
                                          uint32_t d, float scale) {
   if constexpr (C == 2) {
-    const unsigned long long one = f2_bits(1.f, 1.f), mm = f2_bits(kMagic, kMagic);
-    const unsigned long long wx2 = f2_bits(wx, wx), wy2 = f2_bits(wy, wy), wz2 = f2_bits(wz, wz);
+    const unsigned long long one = f2_pack(1.f, 1.f), mm = f2_pack(kMagic, kMagic);
+    const unsigned long long wx2 = f2_pack(wx, wx), wy2 = f2_pack(wy, wy), wz2 = f2_pack(wz, wz);
     unsigned long long ax2, ay2, az2;
     asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(ax2) : "l"(one), "l"(wx2));
     asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(ay2) : "l"(one), "l"(wy2));
     asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(az2) : "l"(one), "l"(wz2));
-    const unsigned long long gs = mul2(bf2_bits(d), f2_bits(scale, scale));
-    const unsigned long long z0 = mul2(az2, gs), z1 = mul2(wz2, gs);
-    const unsigned long long yz[4] = {mul2(ay2, z0), mul2(wy2, z0), mul2(ay2, z1), mul2(wy2, z1)};
+    const unsigned long long gs = f2_mul(bf2_bits(d), f2_pack(scale, scale));
+    const unsigned long long z0 = f2_mul(az2, gs), z1 = f2_mul(wz2, gs);
+    const unsigned long long yz[4] = {f2_mul(ay2, z0), f2_mul(wy2, z0), f2_mul(ay2, z1), f2_mul(wy2, z1)};
     const uint32_t a[4] = {a0, a0 + oy, a0 + oz, a0 + oy + oz};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const unsigned long long va = fma2(ax2, yz[j], mm), vb = fma2(wx2, yz[j], mm);
+      const unsigned long long va = f2_fma(ax2, yz[j], mm), vb = f2_fma(wx2, yz[j], mm);
       red_s32<0>(a[j], (int32_t)(uint32_t)va - kMagicBits);
       red_s32<128>(a[j], (int32_t)(uint32_t)(va >> 32) - kMagicBits);
       red_s32<256>(a[j], (int32_t)(uint32_t)vb - kMagicBits);
@@ -482,22 +483,22 @@ __device__ __forceinline__ void red_cell_wide(uint32_t a0, uint32_t oy, uint32_t
   constexpr int kX = 2 * C * 128;   // the next x node
   const uint32_t a[4] = {a0, a0 + oy, a0 + oz, a0 + oy + oz};
   if constexpr (C == 2) {
-    const unsigned long long one = f2_bits(1.f, 1.f), mm = f2_bits(kMagic, kMagic), ls = f2_bits(kLowScale, kLowScale);
-    const unsigned long long wx2 = f2_bits(wx, wx), wy2 = f2_bits(wy, wy), wz2 = f2_bits(wz, wz);
+    const unsigned long long one = f2_pack(1.f, 1.f), mm = f2_pack(kMagic, kMagic), ls = f2_pack(kLowScale, kLowScale);
+    const unsigned long long wx2 = f2_pack(wx, wx), wy2 = f2_pack(wy, wy), wz2 = f2_pack(wz, wz);
     auto sub2 = [](unsigned long long p, unsigned long long q) {
       unsigned long long r;
       asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(p), "l"(q));
       return r;
     };
     const unsigned long long ax2 = sub2(one, wx2), ay2 = sub2(one, wy2), az2 = sub2(one, wz2);
-    const unsigned long long gs = mul2(bf2_bits(d), f2_bits(scale, scale));
-    const unsigned long long z0 = mul2(az2, gs), z1 = mul2(wz2, gs);
-    const unsigned long long yz[4] = {mul2(ay2, z0), mul2(wy2, z0), mul2(ay2, z1), mul2(wy2, z1)};
+    const unsigned long long gs = f2_mul(bf2_bits(d), f2_pack(scale, scale));
+    const unsigned long long z0 = f2_mul(az2, gs), z1 = f2_mul(wz2, gs);
+    const unsigned long long yz[4] = {f2_mul(ay2, z0), f2_mul(wy2, z0), f2_mul(ay2, z1), f2_mul(wy2, z1)};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const unsigned long long va = fma2(ax2, yz[j], mm), vb = fma2(wx2, yz[j], mm);
-      const unsigned long long la = fma2(fma2(ax2, yz[j], sub2(mm, va)), ls, mm);
-      const unsigned long long lb = fma2(fma2(wx2, yz[j], sub2(mm, vb)), ls, mm);
+      const unsigned long long va = f2_fma(ax2, yz[j], mm), vb = f2_fma(wx2, yz[j], mm);
+      const unsigned long long la = f2_fma(f2_fma(ax2, yz[j], sub2(mm, va)), ls, mm);
+      const unsigned long long lb = f2_fma(f2_fma(wx2, yz[j], sub2(mm, vb)), ls, mm);
       red_s32<0>(a[j], (int32_t)(uint32_t)va - kMagicBits);
       red_s32<128>(a[j], (int32_t)(uint32_t)la - kMagicBits);
       red_s32<256>(a[j], (int32_t)(uint32_t)(va >> 32) - kMagicBits);
@@ -672,7 +673,7 @@ __device__ __forceinline__ void scat_units(const Model& md, const Grads& gr, con
       const uint32_t oy = (uint32_t)nxb * kNodeBytes, oz = (uint32_t)(nxb * nyb) * kNodeBytes;
       const float hs = 0.5f * (float)(R - 1);
       const float ct = hs - 0.5f + kMagic;   // an integer when R is even (axis_cell)
-      const unsigned long long hs2 = f2_bits(hs, hs), ct2 = f2_bits(ct, ct), mm2 = f2_bits(kMagic, kMagic);
+      const unsigned long long hs2 = f2_pack(hs, hs), ct2 = f2_pack(ct, ct), mm2 = f2_pack(kMagic, kMagic);
       const int32_t mlox = kMagicBits + lox, mloy = kMagicBits + loy, mloz = kMagicBits + loz;
       // dL/dy of the next SU points is requested while the current SU are processed
       constexpr int SU = 4;
@@ -713,7 +714,7 @@ __device__ __forceinline__ void scat_units(const Model& md, const Grads& gr, con
           unsigned lx, ly, lz;   // cell relative to the box
           if constexpr (EVEN_R) {
             int32_t tx, ty;   // x and y as one packed pair
-            axis_cell2(f2_bits(ux, uy), hs2, ct2, mm2, tx, ty, wxs[u], wys[u]);
+            axis_cell2(f2_pack(ux, uy), hs2, ct2, mm2, tx, ty, wxs[u], wys[u]);
             lx = (unsigned)(tx - mlox);
             ly = (unsigned)(ty - mloy);
             lz = (unsigned)(axis_cell(uz, hs, ct, wzs[u]) - mloz);

@@ -13,8 +13,9 @@ __device__ __forceinline__ int brick_of_point(const Bricks& br, int64_t g) {
   return lo;
 }
 
-// Exclusive scan of one brick's kSortBins counters by a block of 1024 threads: each warp scans 1024 consecutive counters, 128 at a time (a lane reads four, so every
-// load of a warp is one line), with shuffles, and one warp scans the 32 warp totals.
+// Exclusive scan of one brick's kSortBins counters by a block of 1024 threads: each warp scans
+// 1024 consecutive counters, 128 at a time (a lane reads four, so every load of a warp is one
+// line), with shuffles, and one warp scans the 32 warp totals.
 // (With 32 consecutive counters per thread every load touched 32 lines: 11 us.)
 __device__ __forceinline__ void scan_bins(uint32_t* hist) {
   constexpr int rounds = kSortBins / 32 / 128;

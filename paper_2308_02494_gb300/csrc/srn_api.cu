@@ -301,7 +301,6 @@ srn_status make_bricks(const srn_handle* h, const int64_t* offsets, srn::Bricks*
     return fail(SRN_ERR_INVALID_ARG, "%lld points exceed max_points %lld", (long long)offsets[B],
                 (long long)h->max_points);
   br->n = B;
-  br->dev = nullptr;
   for (int b = 0; b <= B; ++b) br->off[b] = offsets[b];
   return SRN_OK;
 }

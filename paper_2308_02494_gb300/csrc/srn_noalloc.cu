@@ -52,7 +52,6 @@ extern "C" srn_status srn_sample_points_static(void* stream, uint64_t seed, uint
   if (offsets[0] != 0) return srn::report(SRN_ERR_INVALID_ARG, "srn_sample_points_static: offsets[0] must be 0");
   srn::Bricks br{};
   br.n = n_bricks;
-  br.dev = nullptr;
   for (int b = 0; b <= n_bricks; ++b) {
     if (b > 0 && offsets[b] < offsets[b - 1])
       return srn::report(SRN_ERR_INVALID_ARG, "srn_sample_points_static: offsets decrease");
