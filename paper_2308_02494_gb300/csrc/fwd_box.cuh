@@ -14,9 +14,11 @@ namespace srn {
 // of shared memory is L1, the corners' latency asks for warps, and three CTAs of one sample
 // per thread, of two at K = 128, are best (BF16 queries at two CTAs of four samples, three of
 // two, three of one: K = 128, 500000 points in order 198, 189 and 197 us; K = 64, 60000 points
-// in no order 46.5, 40.7 and 40.5).  Float32 has the registers for two (K = 128, 20000 points
-// in no order: 63.5 us at two samples per thread, 57.0 at one).
-constexpr int fwd_ctas(int K, bool F32, bool boxes) { return F32 || (boxes && K >= 64) ? 2 : 3; }
+// in no order 46.5, 40.7 and 40.5).  Points far apart in K = 128's grids, whose corners come from
+// far, want four samples' reads in flight instead (`far`: point_source).  Float32 has the
+// registers for two (K = 128, 20000 points in no order: 63.5 us at two samples per thread, 57.0
+// at one).
+constexpr int fwd_ctas(int K, bool F32, bool four) { return F32 || (four && K >= 64) ? 2 : 3; }
 
 // One grid's staged box as the encoder sees it.  With t the cell's float bits of
 // axis_cell (cell + kMagicBits) per axis, the byte address of the cell's first corner is

@@ -74,9 +74,10 @@ __device__ __forceinline__ float unord(uint32_t o) {
   return __uint_as_float(o ^ ((o & 0x80000000u) ? 0x80000000u : 0xffffffffu));
 }
 
-// VIEW: ray samples or voxels, else points in memory.  BOXES: with staged boxes.
-template <int K, int C, bool EVEN, bool F32, bool VIEW, bool BOXES>
-__global__ void __launch_bounds__(NT, fwd_ctas(K, F32, BOXES))
+// VIEW: ray samples or voxels, else points in memory.  BOXES: with staged boxes.  FAR: points far
+// apart.
+template <int K, int C, bool EVEN, bool F32, bool VIEW, bool BOXES, bool FAR>
+__global__ void __launch_bounds__(NT, fwd_ctas(K, F32, BOXES || FAR))
 k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> src, float* __restrict__ out,
       uint32_t pool_nodes) {
   using L = FwdLay<K, C, F32, BOXES>;
@@ -85,7 +86,7 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
   constexpr int CW = F32 && K == 16 ? 4 : 8;   // features per chunk
   constexpr int GPC = CW / C;                // grids per chunk
   constexpr int NCH = K / CW;                // chunks of a feature row
-  constexpr int PP = K < 64 || (!BOXES && (F32 || K < 128)) ? 1 : F32 || !BOXES ? 2 : 4;   // samples per thread
+  constexpr int PP = K < 64 || (!BOXES && (F32 || K < 128)) ? 1 : F32 || !(BOXES || FAR) ? 2 : 4;   // samples per thread
   constexpr int NQ = 8 / (T / (32 * PP));    // warps sharing the same samples, each its own chunks
   constexpr uint32_t kNB = 4 * C;            // bytes of a staged node
   extern __shared__ __align__(128) unsigned char sm[];
@@ -622,10 +623,10 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
   }
 }
 
-template <int K, int C, bool EVEN, bool F32, bool VIEW, bool BOXES>
+template <int K, int C, bool EVEN, bool F32, bool VIEW, bool BOXES, bool FAR = false>
 cudaError_t launch_k(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
   using Lay = FwdLay<K, C, F32, BOXES>;
-  auto kern = k_fwd<K, C, EVEN, F32, VIEW, BOXES>;
+  auto kern = k_fwd<K, C, EVEN, F32, VIEW, BOXES, FAR>;
   const int smem = BOXES ? fwd_smem(L.smem_sm, K, F32) : Lay::BOX;   // (what is left is L1)
   if (BOXES && smem < Lay::POOL + 64) return cudaErrorInvalidConfiguration;   // room for dropped reads (fwd_box)
   const int pool = BOXES ? (smem - Lay::POOL) / (4 * C) : 0;
@@ -640,7 +641,7 @@ cudaError_t launch_k(const Launch& L, const Model& md, const Bricks& br, const F
   }
   if (total == 0) return cudaSuccess;
   FwdSource s = src;
-  const int ctas = fwd_ctas(K, F32, BOXES) * L.num_sms;
+  const int ctas = fwd_ctas(K, F32, BOXES || FAR) * L.num_sms;
   s.run = std::max(1, std::min(4, total / (8 * ctas)));
   const int grid = std::min((total + s.run - 1) / s.run, ctas);
   kern<<<grid, NT, smem, L.stream>>>(md, br, s, out, (uint32_t)pool);
@@ -649,7 +650,11 @@ cudaError_t launch_k(const Launch& L, const Model& md, const Bricks& br, const F
 
 template <int K, int C, bool EVEN>
 cudaError_t launch_e(const Launch& L, const Model& md, const Bricks& br, const FwdSource& src, float* out) {
-  if (src.kind == kFwdPoints) return launch_k<K, C, EVEN, kF32, false, false>(L, md, br, src, out);
+  if (src.kind == kFwdPoints) {
+    if constexpr (K == 128 && !kF32)
+      if (src.far) return launch_k<K, C, EVEN, kF32, false, false, true>(L, md, br, src, out);
+    return launch_k<K, C, EVEN, kF32, false, false>(L, md, br, src, out);
+  }
   return src.boxes ? launch_k<K, C, EVEN, kF32, true, true>(L, md, br, src, out)
                    : launch_k<K, C, EVEN, kF32, true, false>(L, md, br, src, out);
 }
