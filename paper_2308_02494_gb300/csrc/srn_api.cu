@@ -351,7 +351,7 @@ cudaError_t forward_points(srn_handle* h, const srn::Launch& L, const srn::Model
   cudaError_t e = h->query_turn ? cudaStreamWaitEvent(L.stream, h->query_done, 0) : cudaSuccess;
   if (e != cudaSuccess) return e;
   src.sorted = h->query_scratch();
-  src.sorted.limit = (uint32_t)(n / 32);   // scan lines and other nearly sorted batches stay as they are
+  src.sorted.limit = (uint32_t)(n / 32);   // scan lines of 32 points and longer stay as they are
   if ((e = srn::launch_sort_query(L, br, xyz, src.sorted)) != cudaSuccess) return e;
   ++h->query_turn;
   h->query_stream = L.stream;
@@ -1080,8 +1080,9 @@ srn_status render_pixels(srn_handle* h, void* stream, const srn::RenderParams& r
   int32_t* next = reinterpret_cast<int32_t*>(h->ws + h->wl.r_next);
   // Ray groups, so that `full` samples (rg rays x full / rg samples), a query group with staged
   // boxes or a feature tile without, are about as deep as they are wide: rays `px` apart, in
-  // blocks of the raster order (at most 64) or in rows of the progressive order's last level (at
-  // most 16), samples `dt` apart along chords of about 2.
+  // blocks of the raster order (at most 64; sqrt(rg) px = full / rg dt) or in rows of the
+  // progressive order's last level (at most 16; rg px = full / rg dt), samples `dt` apart along
+  // chords of about 2.  rg is the power of two next to that, by ratio.
   srn::RenderParams rp = rpi;
   const srn::Model md = h->model();
   const bool f32 = h->cfg.precision != SRN_BF16;
@@ -1097,7 +1098,7 @@ srn_status render_pixels(srn_handle* h, void* stream, const srn::RenderParams& r
   rp.rg = rp.order ? 16 : 64;
   while (rp.rg > 1 && ((float)rp.rg > 1.42f * want || rp.rg > count || (int64_t)rp.rg * rp.samples > h->max_points))
     rp.rg /= 2;
-  const int per = full / rp.rg;
+  const int per = full / rp.rg;   // a ray's samples fill whole groups if that leaves an eighth empty at most
   const int64_t pad = ((int64_t)rp.samples + per - 1) / per * per;
   rp.spr = pad * 8 <= (int64_t)rp.samples * 9 && pad * rp.rg <= h->max_points ? (int)pad : rp.samples;
   // whole ray groups whose slots fit the workspace's max_points samples (and 31 bits)
