@@ -51,8 +51,8 @@ KERNELS_PER_STEP = {"bf16": 15, "fp32": 10}
 # DRAM bytes (read + write) per launch of each training-pass kernel, from an ncu capture
 # of the 8-brick step (profiles/).  They hold only for the kernel sources they were
 # taken on: any change to those files makes bench report traffic as null.
-NCU_TRAFFIC = {"sources_sha1": "73322001601b1f903f64ee9a83c237cd246f79fe",
-               "k_scat": 1082.62e6, "k_enc": 715.19e6, "k_mlp": 1336.33e6}
+NCU_TRAFFIC = {"sources_sha1": "0c601e6948b51ea88fa0e3eee9f84e2f8b11137a",
+               "k_scat": 1094.52e6, "k_enc": 715.78e6, "k_mlp": 1336.80e6}
 TRAFFIC_SOURCES = ("k_train_bf16.cu", "k_mlp_tc.cu", "common.cuh", "bf16_ops.cuh", "tc_ops.cuh", "enc_ops.cuh")
 
 

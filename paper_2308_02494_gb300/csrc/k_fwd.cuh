@@ -15,10 +15,10 @@
 // a warp.
 //
 // What bounds it: with boxes, instruction issue and the shared-memory pipe (55% and 65% busy
-// in a decode); without, the L1 pipe.  Reading the corners from global memory takes 116 warp
-// instructions per 32 (sample, grid) pairs (unpacking BF16 nodes, float-int conversions,
-// clamps); staged float32 nodes need no unpacking, one address for eight reads and packed
-// f32x2 blends: 88.  A sample outside a grid reads nothing, by predicated loads: reading, and
+// in a decode); without, the L1 pipe (82% in a query of 1.0 M sorted points, IPC 2.3).  Reading
+// the corners from global memory takes 103 warp instructions per 32 (sample, grid) pairs, of
+// which unpacking the BF16 nodes and eight addresses; staged float32 nodes need no unpacking
+// and one address for eight reads: 88.  A sample outside a grid reads nothing, by predicated loads: reading, and
 // dropping, some cell took 110.9 us where it takes 102.0 (200003 points in no order, K = 64).
 // Boxes of points in memory did not pay at any density: 1500000 points in order of the
 // paper-scale model took 568 us with them and 470 without, 60000 59 and 46.
