@@ -125,12 +125,13 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
 
   int cur = -1, hint = -1;
   // Runs of src.run consecutive groups (they share a brick and its weights): one for every CTA,
-  // and then in turn, or where the groups differ as CTAs are done (src.next; the next run is
+  // and then in turn, or, of rays in many rounds, as CTAs are done (src.next; the next run is
   // taken one ahead).  Dealt in turn, the rows of a view's groups could divide the CTAs evenly,
   // and some had the volume's middle in every round and others its empty sides (a progressive
   // pass with a third of its rays on the volume: 473 us, and 293 taken as they come).
   for (int r = blockIdx.x, k = 0; r * src.run < total; ++k) {
-  if (VIEW && src.next && tid == 0) s_run[k & 1] = (int)gridDim.x + atomicAdd(src.next, 1);
+  int after = 0;
+  if (VIEW && src.next && tid == 0) after = (int)gridDim.x + atomicAdd(src.next, 1);
   const int r0 = r * src.run, r1 = min(total, r0 + src.run);
   for (int grp = r0; grp < r1; ++grp) {
     // ---- the group's samples: coordinates and brick (-1: no sample)
@@ -193,7 +194,10 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
     unsigned long long mask = render || ns <= 0 ? 0ull : 1ull << (VIEW ? blk.brick : hint);
     // (a decode's block that is empty, at the end of a shorter brick, comes to no other barrier
     // before `blk` is written again)
-    if constexpr (VIEW) __syncthreads();
+    if constexpr (VIEW) {
+      if (tid == 0) s_run[k & 1] = after;   // (here, so that the samples hide the counter's latency)
+      __syncthreads();
+    }
     if (render) mask = (unsigned long long)s_mask[0] | ((unsigned long long)s_mask[1] << 32);
     const bool mixed = VIEW && (mask & (mask - 1)) != 0;
     if (mixed) {   // the bricks' samples one brick after the other, in order within each
@@ -618,7 +622,7 @@ k_fwd(Model md, Bricks brp, std::conditional_t<VIEW, FwdSource, FwdPointSource> 
       }
     }
   }
-  // (a group has a barrier at least, so s_run[k & 1] is not written again before it is read)
+  // (the next run's barriers come before s_run[k & 1] is written again)
   r = VIEW && src.next ? s_run[k & 1] : r + (int)gridDim.x;
   }
 }
@@ -643,6 +647,9 @@ cudaError_t launch_k(const Launch& L, const Model& md, const Bricks& br, const F
   FwdSource s = src;
   const int ctas = fwd_ctas(K, F32, BOXES || FAR) * L.num_sms;
   s.run = std::max(1, std::min(4, total / (8 * ctas)));
+  // (taken one ahead, the last runs of a few rounds go to whichever CTAs began first, three of an
+  // SM: batches of 512 groups 45 us each, dealt in turn 36)
+  if (total < 8 * ctas) s.next = nullptr;
   const int grid = std::min((total + s.run - 1) / s.run, ctas);
   kern<<<grid, NT, smem, L.stream>>>(md, br, s, out, (uint32_t)pool);
   return cudaGetLastError();

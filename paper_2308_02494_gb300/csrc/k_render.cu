@@ -107,10 +107,10 @@ __global__ void k_render_preview(RenderParams rp, int done, int level, const flo
 
 }  // namespace
 
-bool boxes_pay(const Model& md, int group, float x, float y, float z) {
+bool boxes_pay(const Model& md, int group, float each, float x, float y, float z) {
   const float cells = 0.5f * (float)(md.R - 1) * 1.15f, e = cbrtf((float)group);
   const float nodes = (e * x * cells + 2.f) * (e * y * cells + 2.f) * (e * z * cells + 2.f);
-  return nodes * (md.F16 ? 8.f : 16.f) <= (float)group;
+  return nodes * each <= (float)group;
 }
 
 cudaError_t launch_render_batch(const Launch& L, const RenderParams& rp, float* val, int32_t* next, int pix0, int npix,
@@ -125,7 +125,7 @@ cudaError_t launch_render_batch(const Launch& L, const RenderParams& rp, float* 
   const float edge = cbrtf(rp.cell);
   src.group = fwd_group(!md.F16, true);
   while (src.group > least && slots < (int64_t)src.group * 2 * L.num_sms) src.group /= 2;
-  src.boxes = boxes_pay(md, src.group, edge, edge, edge);
+  src.boxes = boxes_pay(md, src.group, ray_samples_per_node(!md.F16), edge, edge, edge);
   if (!src.boxes) src.group = std::min(src.group, fwd_group(!md.F16, false));
   src.groups = (int)((slots + src.group - 1) / src.group);
   src.next = next;
@@ -167,7 +167,12 @@ cudaError_t launch_decode(const Launch& L, const RenderParams& rp, const Model& 
   const int tile = md.F16 ? 128 : 64;   // (the kernel's)
   int cap = fwd_group(!md.F16, true);
   while (cap > tile && voxels / cap < 8 * (int64_t)L.num_sms) cap /= 2;
-  src.boxes = boxes_pay(md, cap, 2.f / (float)n[0], 2.f / (float)n[1], 2.f / (float)n[2]);
+  // A block of voxels is a cube along the bricks' axes, so full ones of BF16 pay sooner than rays
+  // (boxes and without, in us, at voxels per node: 64 grids, 3.0 1389 and 1362, 4.1 612 and 638, 4.5
+  // 2344 and 2600; 32 grids, 2.5 155 and 158, 4.4 337 and 387; 16 grids of 16^3, 3.9 101 and 109).
+  const float full = md.K == 128 ? 4.f : 2.5f;
+  const float each = md.F16 && cap == fwd_group(false, true) ? full : ray_samples_per_node(!md.F16);
+  src.boxes = boxes_pay(md, cap, each, 2.f / (float)n[0], 2.f / (float)n[1], 2.f / (float)n[2]);
   if (!src.boxes) cap = std::min(cap, fwd_group(!md.F16, false));
   double best = 0.0;
   for (int x = 1; x <= std::min(16, n[0]); ++x)

@@ -184,7 +184,7 @@ struct FwdPointSource {   // what a kernel over points in memory gets (the rest 
   int32_t kind;
   int32_t group, groups;   // (kFwdPoints counts its groups per brick itself)
   int32_t run;             // consecutive groups of a CTA (set by the launch)
-  int32_t* next;           // kFwdRender: zero; runs of groups taken beyond the CTAs' first
+  int32_t* next;           // kFwdRender: zero; runs of groups taken beyond the CTAs' first (NULL: in turn)
   int32_t boxes;           // 0 (always for points in memory): read every corner from global memory
   int32_t far;             // kFwdPoints: the points of a group are far apart
   const float* xyz;        // kFwdPoints, and their sorted copy, if one was made
@@ -251,13 +251,14 @@ inline cudaError_t launch_forward(const Launch& L, const Model& md, const Bricks
 // Whether staged boxes pay for groups of `group` of a brick's samples, x, y and z apart in its
 // coordinates: a cube's nodes in a grid are those of its extent in cells (the maps are on the
 // device: they are taken to zoom by 15%), a partial cell and a node at either end, and a node
-// should serve eight samples or more, sixteen in float32.  With boxes and without, in us, at
+// should serve `each` samples or more.  Rays: eight, sixteen in float32.  With boxes and without, in us, at
 // samples per node by this count: BF16, 64 grids, 11 (frame of 512^2 x 256 rays through 8 bricks)
 // 20300 and 23600, 6.6 (progressive pass of 9000 x 256) 967 and 925, 2.9 (the same, 4 bricks)
 // 1475 and 1059; 32 grids, 13 460 and 459; 16 grids, 14 (14400 x 256) 258 and 283.  Float32, 64
 // grids, 7 (frame of 160^2 x 320) 7036 and 7548, 2.6 (8 bricks) 10780 and 8910; 16 grids of 9^3,
 // 20 2805 and 2600.
-bool boxes_pay(const Model& md, int group, float x, float y, float z);
+bool boxes_pay(const Model& md, int group, float each, float x, float y, float z);
+inline float ray_samples_per_node(bool f32) { return f32 ? 16.f : 8.f; }
 // Rays pix0 .. pix0 + npix - 1 of rp's order; val: [max_points] scratch for their samples'
 // values, next: a counter that is zero, and again after a batch whose launches succeed.
 cudaError_t launch_render_batch(const Launch& L, const RenderParams& rp, float* val, int32_t* next, int pix0, int npix,

@@ -1093,7 +1093,7 @@ srn_status render_pixels(srn_handle* h, void* stream, const srn::RenderParams& r
   const float dt = 2.f / (float)rp.samples;
   rp.cell = px * px * dt * (float)(rp.grid[0] * rp.grid[1] * rp.grid[2]);
   const float edge = cbrtf(rp.cell);
-  const int full = srn::boxes_pay(md, srn::fwd_group(f32, true), edge, edge, edge) ? srn::fwd_group(f32, true) : f32 ? 64 : 128;
+  const int full = srn::boxes_pay(md, srn::fwd_group(f32, true), srn::ray_samples_per_node(f32), edge, edge, edge) ? srn::fwd_group(f32, true) : f32 ? 64 : 128;
   const float ratio = (float)full * dt / px, want = rp.order ? sqrtf(ratio) : powf(ratio, 2.f / 3.f);
   rp.rg = rp.order ? 16 : 64;
   while (rp.rg > 1 && ((float)rp.rg > 1.42f * want || rp.rg > count || (int64_t)rp.rg * rp.samples > h->max_points))
